@@ -1134,21 +1134,23 @@ int plan_lift(smf_ctx* ctx, const smf_basis* pb, const smf_bigmat* A, const smf_
     return SMF_OK;
 }
 
-// A^-1 mod p: workspace slots.  The blocked form (limb form, residues of at
-// most three digits, n above kInvBlockedMin) adds the panel scratch, the
-// panel's transform, the pivot rows, the product and its operand planes.
-constexpr int64_t kInvPanel = 128;
-constexpr int64_t kInvBlockedMin = 256;
-
+// A^-1 mod p: workspace slots.  The form by panels needs the panel's
+// transform, the pivot rows, the product and its operand planes when the
+// matrix takes more than one panel; the form by columns a second matrix.
 struct InverseLayout {
-    size_t res = 0, M = 0, col = 0, flag = 0, T = 0, S = 0, Mp = 0, C = 0, gemm = 0, gemm_bytes = 0, bytes = 0;
+    size_t res = 0, M = 0, col = 0, flag = 0, scratch = 0, S = 0, Mp = 0, C = 0, gemm = 0, gemm_bytes = 0, bytes = 0;
 };
 
-bool inverse_blocked(const smf_ctx* ctx, int64_t n, int digits) {
-    return ctx->form == SMF_FORM_INT8LIMB && n > kInvBlockedMin && digits <= 3;
+// By panels: any odd p when one panel holds the matrix; larger matrices need
+// the limb product of three-digit residues.
+bool inverse_panels(const smf_ctx* ctx, int64_t n, uint32_t p) {
+    if ((p & 1) == 0) return false;
+    return n <= kInvSingle || (ctx->form == SMF_FORM_INT8LIMB && digits_for(p / 2) <= 3);
 }
 
-InverseLayout inverse_layout(const smf_ctx* ctx, int64_t n, bool blocked) {
+// The workspace does not know p: it holds the larger of the two forms (their
+// parts overlap after res, col and flag).
+InverseLayout inverse_layout(const smf_ctx* ctx, int64_t n) {
     InverseLayout Lw;
     size_t off = 0;
     auto slot = [&](size_t bytes) {
@@ -1157,23 +1159,27 @@ InverseLayout inverse_layout(const smf_ctx* ctx, int64_t n, bool blocked) {
         return o;
     };
     Lw.res = slot((size_t)4 * n * n);
-    Lw.M = slot((size_t)8 * n * n);
-    Lw.col = slot((size_t)4 * n);
+    Lw.col = slot((size_t)8 * n);
     Lw.flag = slot(4);
-    if (blocked) {
-        Lw.T = slot((size_t)8 * n * kInvPanel);
-        Lw.S = slot((size_t)4 * n * kInvPanel);
-        Lw.Mp = slot((size_t)8 * n * kInvPanel);
-        Lw.C = slot((size_t)8 * n * n);
-        // the largest product plan over the panels (three-digit residues)
-        for (int64_t c0 = 0; c0 < n; c0 += kInvPanel) {
-            const int64_t b = std::min<int64_t>(kInvPanel, n - c0);
-            const GemmPlan g = plan_limb(1, n, 2 * n - c0 - b, b, false, 1u << 23, 1u << 23, ctx->num_sms);
+    Lw.scratch = slot(inv_scratch_bytes());
+    const size_t base = off;
+    Lw.M = slot((size_t)8 * n * n);
+    size_t end = off;
+    const int64_t w = inv_panel_width(n);
+    if (n > kInvSingle && ctx->form == SMF_FORM_INT8LIMB) {
+        off = base;
+        Lw.S = slot((size_t)4 * n * w);
+        Lw.Mp = slot((size_t)4 * n * w);
+        Lw.C = slot((size_t)4 * n * n);
+        // the largest product plan over the panels (three-digit residues): whole ones and the last
+        for (const int64_t b : {w, n % w ? n % w : w}) {
+            const GemmPlan g = plan_limb(1, n, n - b, b, false, 1u << 23, 1u << 23, ctx->num_sms);
             Lw.gemm_bytes = std::max(Lw.gemm_bytes, g.bytes);
         }
         Lw.gemm = slot(Lw.gemm_bytes);
+        end = std::max(end, off);
     }
-    Lw.bytes = off;
+    Lw.bytes = end;
     return Lw;
 }
 
@@ -1817,7 +1823,7 @@ int smf_padic_lift(smf_ctx* ctx, const smf_basis* p_basis, const smf_bigmat* A, 
 
 int smf_inverse_mod_p_workspace(smf_ctx* ctx, int64_t n, size_t* bytes) {
     if (!ctx || !bytes || n < 0) return SMF_E_INVALID;
-    *bytes = inverse_layout(ctx, n, inverse_blocked(ctx, n, 3)).bytes;
+    *bytes = inverse_layout(ctx, n).bytes;
     return SMF_OK;
 }
 
@@ -1834,8 +1840,7 @@ int smf_inverse_mod_p(smf_ctx* ctx, const smf_basis* p_basis, const smf_bigmat* 
     if (n == 0) return SMF_OK;
     if (!device_ptr(A_inv)) return fail(ctx, SMF_E_INVALID, "inverse_mod_p: A_inv must be device memory");
     const uint32_t p = p_basis->primes[0];
-    const bool blocked = inverse_blocked(ctx, n, digits_for(p / 2));
-    const InverseLayout Lw = inverse_layout(ctx, n, blocked);
+    const InverseLayout Lw = inverse_layout(ctx, n);
     cudaStream_t s = (cudaStream_t)stream;
     if (!workspace) {
         if (ctx->budget && Lw.bytes > ctx->budget) return fail(ctx, SMF_E_NOMEM, "inverse_mod_p: workspace over budget");
@@ -1860,32 +1865,32 @@ int smf_inverse_mod_p(smf_ctx* ctx, const smf_basis* p_basis, const smf_bigmat* 
     int* flag = (int*)(w + Lw.flag);
     const ReduceArgs ra{(const uint64_t*)A->data, n, n, A->ld, A->words, res, 0, 0, 0};
     SMF_CU(ctx, launch_reduce(p_basis->dev, ra, ReduceOut::kCanonical, ctx->d_status, s));
-    if (!blocked) {
+    if (!inverse_panels(ctx, n, p)) {
         SMF_CU(ctx, launch_inverse_mod_p(res, n, p, M, col, flag, A_inv, ctx->d_status, ctx->num_sms, s));
         return SMF_OK;
     }
-    // panels of kInvPanel columns; the rest of the elimination of each panel is
-    // one residue product with the panel's transform (inverse.cu)
-    uint32_t* T = (uint32_t*)(w + Lw.T);
-    int32_t* Sc = (int32_t*)(w + Lw.S);
+    // res is reduced in place by panels of w columns; the rest of each panel's
+    // elimination is one residue product with the panel's transform (inverse.cu)
+    uint32_t* Mn = (uint32_t*)res;
+    int* rowcol = (int*)col;
+    int* piv = rowcol + n;
+    int32_t* S = (int32_t*)(w + Lw.S);
     int32_t* Mp = (int32_t*)(w + Lw.Mp);
     int32_t* Cb = (int32_t*)(w + Lw.C);
-    const int64_t ld = 2 * n;
     const uint64_t h = p / 2;
     SMF_CU(ctx, cudaMemsetAsync(flag, 0, sizeof(int), s));
-    SMF_CU(ctx, launch_gj_init(res, n, M, s));
-    for (int64_t c0 = 0; c0 < n; c0 += kInvPanel) {
-        const int64_t b = std::min<int64_t>(kInvPanel, n - c0), c1 = c0 + b, R = ld - c1;
-        SMF_CU(ctx, cudaMemcpy2DAsync(T, 8 * b, M + c0, 4 * ld, 4 * b, n, cudaMemcpyDeviceToDevice, s));
-        SMF_CU(ctx, cudaMemset2DAsync(T + b, 8 * b, 0, 4 * b, n, s));
-        SMF_CU(ctx, launch_panel_factor(T, n, (int)b, c0, M, ld, c1, ld, p, col, flag, ctx->d_status, ctx->num_sms, s));
-        SMF_CU(ctx, cudaMemcpy2DAsync(Sc, 4 * b, T + b, 8 * b, 4 * b, n, cudaMemcpyDeviceToDevice, s));
-        SMF_CU(ctx, cudaMemcpy2DAsync(Mp, 4 * R, M + c0 * ld + c1, 4 * ld, 4 * R, b, cudaMemcpyDeviceToDevice, s));
-        if ((st = run_residue_gemm_i32(ctx, p_basis, Sc, n * b, Mp, Cb, n, R, b, h, h, w + Lw.gemm, Lw.gemm_bytes, s)))
+    SMF_CU(ctx, cudaMemsetAsync(rowcol, 0xFF, sizeof(int) * 2 * (size_t)n, s));
+    const int64_t pw = inv_panel_width(n);
+    for (int64_t c0 = 0; c0 < n; c0 += pw) {
+        const int64_t b = std::min<int64_t>(pw, n - c0), R = n - b;
+        SMF_CU(ctx, launch_inv_panel(Mn, n, c0, (int)b, p, rowcol, piv, R ? S : nullptr, w + Lw.scratch, flag, ctx->d_status, s));
+        if (R == 0) break;
+        SMF_CU(ctx, launch_inv_gather(Mn, n, c0, (int)b, piv, Mp, flag, s));
+        if ((st = run_residue_gemm_i32(ctx, p_basis, S, n * b, Mp, Cb, n, R, b, h, h, w + Lw.gemm, Lw.gemm_bytes, s)))
             return st;
-        SMF_CU(ctx, launch_panel_update(M, ld, n, c0, c1, R, Cb, p, s));
+        SMF_CU(ctx, launch_inv_update(Mn, n, c0, (int)b, rowcol, Cb, p, s));
     }
-    SMF_CU(ctx, cudaMemcpy2DAsync(A_inv, 4 * n, M + n, 4 * ld, 4 * n, n, cudaMemcpyDeviceToDevice, s));
+    SMF_CU(ctx, launch_inv_place(Mn, n, piv, rowcol, A_inv, flag, s));
     return SMF_OK;
 }
 

@@ -10,11 +10,13 @@
 //             f_k = 0);
 //   gj_elim:  every row i != k subtracts f_i times row k, over the columns
 //             j >= k (row k is zero left of column k).
-// Afterwards the right half is A^-1 mod p.  A column without a pivot means
-// p | det A: the pivot launch sets kStatusSingular and a device flag, and
+// Afterwards the right half is A^-1 mod p.  That is the general form; matrices
+// of up to kInvSingle columns (p odd), and larger ones in the limb form, go by
+// panels instead (below).  A column without a pivot means p | det A: the pivot launch sets kStatusSingular and a device flag, and
 // every later launch returns at once.
 #include <algorithm>
 
+#include "panel.h"
 #include "smf_internal.h"
 
 namespace smf {
@@ -131,141 +133,101 @@ __global__ void __launch_bounds__(kElimThreads) gj_elim_kernel(uint32_t* __restr
     }
 }
 
-// ---- blocked form: panels of bw columns
+// ---- by panels (panel.h)
 //
-// For panel columns [c0, c1) the scratch T = [P | S] (n x 2bw) holds a copy of
-// the panel P and a block S that starts at zero.  Column k of the panel is
-// reduced as above, restricted to T; the row swap is applied to M's columns
-// [c1, 2n) as well, and S's entry (k, k - c0) gains 1 right after the swap,
-// before the scaling.  By linearity S then ends as E S0, where E is the
-// panel's elimination with all swaps done first and S0 the unit rows at the
-// pivot positions c0 .. c1-1.  With Mp = M[c0:c1, c1:2n] after the swaps,
-// the whole elimination of the remaining columns is
-//   M[i, c1:] = (S Mp)_i                  for the pivot rows c0 <= i < c1,
-//   M[i, c1:] = M[i, c1:] + (S Mp)_i     for every other row,
-// one residue product with one prime (K = bw) and one elementwise pass.
+// M (n x n) is inverted in place: the panel's columns become its transform S,
+// the other columns M + S Mp (the panel's pivot rows S Mp), one residue product
+// with K = w and one pass.  When every column has had its pivot,
+// A^-1[k][c] = M[piv[k]][rowcol[c]].  Up to kInvSingle columns the matrix is one
+// panel, in the shared memory of one cluster (n = 512: 0.70 ms, n = 513 in five
+// panels 0.63 ms, n = 384 0.61 ms).
+//
+// GB300, 24-bit p: n = 1500 2.5 ms (15.3 ms with two launches per column of a
+// panel), n = 1024 1.3 ms, n = 128 0.12 ms.  Of a round of 16 columns at n = 1500
+// (31,000 cycles): the multiply-adds of the update 14,000 (28 of them a clock and
+// SM is what the integer pipe gives: 94 rows x 128 words x 16), the tile of the
+// pivots 10,000, the barriers and the way of Y through L2 7,000; the products
+// between panels add 60 us each.
 
-__global__ void __launch_bounds__(kPivotThreads)
-    panel_pivot_kernel(uint32_t* __restrict__ T, int64_t n, int bw, int64_t k, int j, uint32_t* __restrict__ M,
-                       int64_t ldM, int64_t lo, int64_t hi, uint32_t p, uint64_t mu, uint32_t* __restrict__ col,
-                       int* flag, int* status) {
-    __shared__ unsigned long long s_piv;
-    __shared__ uint32_t s_inv;
-    pdl_wait();
-    pdl_trigger();
-    if (*flag) return;
-    const int64_t ldT = 2 * (int64_t)bw;
-    if (threadIdx.x == 0) s_piv = (unsigned long long)n;
-    __syncthreads();
-    for (int64_t r = k + threadIdx.x; r < n; r += kPivotThreads) {
-        if (T[r * ldT + j] != 0) {
-            atomicMin(&s_piv, (unsigned long long)r);
-            break;
-        }
-    }
-    __syncthreads();
-    const int64_t r = (int64_t)s_piv;
-    if (r == n) {
-        if (threadIdx.x == 0) {
-            *flag = 1;
-            atomicOr(status, kStatusSingular);
-        }
-        return;
-    }
-    if (r != k) {
-        for (int64_t c = threadIdx.x; c < ldT; c += kPivotThreads) {
-            const uint32_t t = T[r * ldT + c];
-            T[r * ldT + c] = T[k * ldT + c];
-            T[k * ldT + c] = t;
-        }
-        for (int64_t c = lo + threadIdx.x; c < hi; c += kPivotThreads) {
-            const uint32_t t = M[r * ldM + c];
-            M[r * ldM + c] = M[k * ldM + c];
-            M[k * ldM + c] = t;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t* a = T + k * ldT + bw + j;  // S gains the unit of pivot row k
-        *a = *a + 1 == p ? 0u : *a + 1;
-        s_inv = powmod(T[k * ldT + j], p - 2, p, mu);
-    }
-    __syncthreads();
-    const uint32_t inv = s_inv;
-    for (int64_t c = j + threadIdx.x; c < ldT; c += kPivotThreads) T[k * ldT + c] = mulmod(T[k * ldT + c], inv, p, mu);
-    for (int64_t i = threadIdx.x; i < n; i += kPivotThreads) col[i] = i == k ? 0u : T[i * ldT + j];
+// The other columns of M: x < c0 stays, x >= c0 is column x + w.
+__global__ void __launch_bounds__(kElimThreads)
+    inv_gather_kernel(const uint32_t* __restrict__ M, int64_t ld, int64_t c0, int w, int64_t R,
+                      const int* __restrict__ piv, int32_t* __restrict__ Mp, const int* flag) {
+    const int64_t x = (int64_t)blockIdx.x * kElimThreads + threadIdx.x;
+    if (x >= R || *flag) return;  // (without a pivot there is no row to read)
+    const int t = blockIdx.y;
+    Mp[(int64_t)t * R + x] = (int32_t)M[(int64_t)piv[c0 + t] * ld + (x < c0 ? x : x + w)];
 }
 
+// M[i] = C[i] on the panel's pivot rows, M[i] + C[i] mod p on the others
 __global__ void __launch_bounds__(kElimThreads)
-    panel_elim_kernel(uint32_t* __restrict__ T, int64_t n, int bw, int64_t k, int j, uint32_t p, uint64_t mu,
-                      const uint32_t* __restrict__ col, const int* flag) {
-    pdl_wait();
-    pdl_trigger();
-    if (*flag) return;
-    const int64_t ldT = 2 * (int64_t)bw;
-    const int64_t c = j + (int64_t)blockIdx.x * kElimThreads + threadIdx.x;
-    if (c >= ldT) return;
-    const uint32_t rk = T[k * ldT + c];
-    if (rk == 0) return;
+    inv_update_kernel(uint32_t* __restrict__ M, int64_t ld, int64_t n, int64_t c0, int w, int64_t R,
+                      const int* __restrict__ rowcol, const int32_t* __restrict__ C, uint32_t p) {
+    const int64_t x = (int64_t)blockIdx.x * kElimThreads + threadIdx.x;
+    if (x >= R) return;
+    const int64_t c = x < c0 ? x : x + w;
     for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
-        const uint32_t f = col[i];
-        if (f == 0) continue;
-        const uint32_t t = mulmod(f, rk, p, mu);
-        uint32_t* e = T + i * ldT + c;
-        const uint32_t v = *e;
-        *e = v >= t ? v - t : v + p - t;
+        const int q = rowcol[i];
+        const uint32_t v = (uint32_t)C[i * R + x];
+        uint32_t* m = M + i * ld + c;
+        const uint32_t u = (q >= c0 && q < c0 + w) ? v : *m + v;  // both below p < 2^31
+        *m = u >= p ? u - p : u;
     }
 }
 
-// M[i, c1 + jj] = C[i][jj] on the pivot rows, M + C mod p on the others
+// A^-1[k][c] = M[piv[k]][rowcol[c]]
 __global__ void __launch_bounds__(kElimThreads)
-    panel_update_kernel(uint32_t* __restrict__ M, int64_t ldM, int64_t n, int64_t c0, int64_t c1, int64_t R,
-                        const int32_t* __restrict__ C, uint32_t p) {
-    const int64_t e = (int64_t)blockIdx.x * kElimThreads + threadIdx.x;
-    if (e >= n * R) return;
-    const int64_t i = e / R, jj = e - i * R;
-    const uint32_t v = (uint32_t)C[e];
-    uint32_t* m = M + i * ldM + c1 + jj;
-    if (i >= c0 && i < c1) {
-        *m = v;
-    } else {
-        const uint32_t w = *m + v;  // both below p < 2^31
-        *m = w >= p ? w - p : w;
-    }
+    inv_place_kernel(const uint32_t* __restrict__ M, int64_t n, const int* __restrict__ piv,
+                     const int* __restrict__ rowcol, int32_t* __restrict__ out, const int* flag) {
+    const int64_t c = (int64_t)blockIdx.x * kElimThreads + threadIdx.x;
+    if (c >= n || *flag) return;
+    const int64_t at = rowcol[c];
+    for (int64_t k = blockIdx.y; k < n; k += gridDim.y) out[k * n + c] = (int32_t)M[(int64_t)piv[k] * n + at];
 }
 
 }  // namespace
 
-cudaError_t launch_panel_factor(uint32_t* T, int64_t n, int bw, int64_t c0, uint32_t* M, int64_t ldM, int64_t lo,
-                                int64_t hi, uint32_t p, uint32_t* col, int* flag, int* status, int num_sms,
-                                cudaStream_t s) {
-    const uint64_t mu = UINT64_MAX / p;
-    const int64_t blocks = kElimBlocksPerSM * (num_sms > 0 ? num_sms : 148);
-    for (int j = 0; j < bw; j++) {
-        const int64_t k = c0 + j;
-        cudaError_t e = launch_pdl(panel_pivot_kernel, dim3(1), dim3(kPivotThreads), 0, s, T, n, bw, k, j, M, ldM, lo,
-                                   hi, p, mu, col, flag, status);
-        if (e != cudaSuccess) return e;
-        const int64_t gx = (2 * (int64_t)bw - j + kElimThreads - 1) / kElimThreads;
-        const int64_t gy = std::min<int64_t>(std::min<int64_t>(n, kMaxGridY), std::max<int64_t>(1, blocks / gx));
-        e = launch_pdl(panel_elim_kernel, dim3((unsigned)gx, (unsigned)gy), dim3(kElimThreads), 0, s, T, n, bw, k, j, p,
-                       mu, (const uint32_t*)col, (const int*)flag);
-        if (e != cudaSuccess) return e;
-    }
+int64_t inv_panel_width(int64_t n) { return n <= kInvSingle ? n : panel_width(n, 1, 128); }
+
+size_t inv_scratch_bytes() { return sizeof(uint32_t) * kSub * kInvSingle; }
+
+cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t p, int* rowcol, int* piv, int32_t* S,
+                             void* scratch, int* flag, int* status, cudaStream_t s) {
+    PanelArgs<1> a{};
+    a.M = M;
+    a.n = a.ld = n;
+    a.c0 = c0;
+    a.w = w;
+    panel_mod(a.md, 0, p, p);
+    a.ybuf = (uint32_t*)scratch;
+    a.piv = piv;
+    a.flag = flag;
+    a.rowcol = rowcol;
+    a.S = S;
+    a.status = status;
+    return launch_panel_red<1, PanelRed::kNarrow, PanelKind::kInverse>(a, n, s);  // (p odd, at most 26 bits)
+}
+
+cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t c0, int w, const int* piv, int32_t* Mp,
+                              const int* flag, cudaStream_t s) {
+    const int64_t R = n - w;
+    inv_gather_kernel<<<dim3((unsigned)((R + kElimThreads - 1) / kElimThreads), (unsigned)w), kElimThreads, 0, s>>>(
+        M, n, c0, w, R, piv, Mp, flag);
     return cudaGetLastError();
 }
 
-cudaError_t launch_panel_update(uint32_t* M, int64_t ldM, int64_t n, int64_t c0, int64_t c1, int64_t R,
-                                const int32_t* C, uint32_t p, cudaStream_t s) {
-    if (n * R == 0) return cudaSuccess;
-    panel_update_kernel<<<(unsigned)((n * R + kElimThreads - 1) / kElimThreads), kElimThreads, 0, s>>>(M, ldM, n, c0,
-                                                                                                        c1, R, C, p);
+cudaError_t launch_inv_update(uint32_t* M, int64_t n, int64_t c0, int w, const int* rowcol, const int32_t* C,
+                              uint32_t p, cudaStream_t s) {
+    const int64_t R = n - w;
+    inv_update_kernel<<<dim3((unsigned)((R + kElimThreads - 1) / kElimThreads), (unsigned)std::min<int64_t>(n, kMaxGridY)),
+                        kElimThreads, 0, s>>>(M, n, n, c0, w, R, rowcol, C, p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gj_init(const int32_t* res, int64_t n, uint32_t* M, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
-    gj_init_kernel<<<(unsigned)((2 * n * n + kElimThreads - 1) / kElimThreads), kElimThreads, 0, s>>>(res, n, M);
+cudaError_t launch_inv_place(const uint32_t* M, int64_t n, const int* piv, const int* rowcol, int32_t* out,
+                             const int* flag, cudaStream_t s) {
+    inv_place_kernel<<<dim3((unsigned)((n + kElimThreads - 1) / kElimThreads), (unsigned)std::min<int64_t>(n, kMaxGridY)),
+                       kElimThreads, 0, s>>>(M, n, piv, rowcol, out, flag);
     return cudaGetLastError();
 }
 

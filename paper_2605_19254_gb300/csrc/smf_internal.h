@@ -421,16 +421,24 @@ cudaError_t launch_widen(const int32_t* x, int64_t count, int64_t* out, cudaStre
 // scratch; C gets A^-1 mod p ([n][n]) unless kStatusSingular is raised.
 cudaError_t launch_inverse_mod_p(const int32_t* res, int64_t n, uint32_t p, uint32_t* M, uint32_t* col, int* flag,
                                  int32_t* C, int* status, int num_sms, cudaStream_t s);
-// The blocked form (inverse.cu): [res | I] into M (n x 2n); one panel of bw
-// columns from c0 reduced on the scratch T = [P | S] (n x 2bw, P filled from
-// M, S zero) with its row swaps applied to M's columns [lo, hi); and the
-// update of M's columns [c1, c1 + R) from C = S Mp (n x R, canonical).
-cudaError_t launch_gj_init(const int32_t* res, int64_t n, uint32_t* M, cudaStream_t s);
-cudaError_t launch_panel_factor(uint32_t* T, int64_t n, int bw, int64_t c0, uint32_t* M, int64_t ldM, int64_t lo,
-                                int64_t hi, uint32_t p, uint32_t* col, int* flag, int* status, int num_sms,
-                                cudaStream_t s);
-cudaError_t launch_panel_update(uint32_t* M, int64_t ldM, int64_t n, int64_t c0, int64_t c1, int64_t R,
-                                const int32_t* C, uint32_t p, cudaStream_t s);
+// The form by panels (inverse.cu), odd p < 2^31: M (n x n, canonical, the
+// matrix on entry) is reduced in place, panel by panel of w columns from c0:
+// the panel itself in one cluster (rowcol: -1 everywhere at the start; S gets
+// the panel's n x w transform), the pivot rows' other n - w columns gathered
+// into Mp (w x (n - w)), their product C = S Mp taken into M, and at the end
+// A^-1 placed from M by the pivots.  A panel as wide as the matrix (n <=
+// kInvSingle) needs no product: S may be null then.
+constexpr int64_t kInvSingle = 512;
+int64_t inv_panel_width(int64_t n);
+cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t p, int* rowcol, int* piv, int32_t* S,
+                             void* scratch, int* flag, int* status, cudaStream_t s);
+size_t inv_scratch_bytes();
+cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t c0, int w, const int* piv, int32_t* Mp,
+                              const int* flag, cudaStream_t s);
+cudaError_t launch_inv_update(uint32_t* M, int64_t n, int64_t c0, int w, const int* rowcol, const int32_t* C,
+                              uint32_t p, cudaStream_t s);
+cudaError_t launch_inv_place(const uint32_t* M, int64_t n, const int* piv, const int* rowcol, int32_t* out,
+                             const int* flag, cudaStream_t s);
 // Column sums of the p-adic digits weighted by W (invariant.cu):
 // out[s][j] = sum_i W[i][j] X[s][i][j] for X [steps][n][m], W [n][m].
 cudaError_t launch_lift_combine(const int32_t* X, int64_t steps, int64_t n, int64_t m, const uint32_t* W,
