@@ -442,8 +442,8 @@ int smf_smith_form(smf_ctx* ctx, const smf_bigmat* A, uint64_t seed, uint32_t* l
  * side): column k's pivot is the first unused row nonzero modulo every
  * prime, every other unused row subtracts its multiple; det = sign of the
  * pivot permutation times the pivots.  A column with no such row sends the
- * call back to one prime at a time.  Large matrices of 31-bit primes run by
- * panels of 16 columns (smf_set_elim_panels), with the same pivots.
+ * call back to one prime at a time.  Primes below 2^31 run by panels of up to
+ * 32 columns (smf_set_elim_panels), with pivots from any rows.
  * A: square, single-word entries, host or device.  det: host, count values
  * in [0, q_i).  Synchronous; allocates its
  * scratch (about n^2 (4 or 8) bytes per prime).  Errors: SMF_E_INVALID (a q_i
@@ -459,8 +459,8 @@ int smf_det_mod(smf_ctx* ctx, const smf_bigmat* A, const uint64_t* q, int32_t co
  * pivots that are units modulo every q_i, then per prime the block of unused
  * rows and deferred columns left: elimination over Z/(q^e) with unit pivots,
  * whose leftover block is divisible by q, is divided by q and is reduced
- * again over Z/(q^(e-1)).  Large matrices whose prime powers are below 2^31
- * run by panels of 16 columns (smf_set_elim_panels), with the same pivots.
+ * again over Z/(q^(e-1)).  Prime powers below 2^31 run by panels of up to 32
+ * columns (smf_set_elim_panels), with pivots from any rows.
  * A: square, single-word entries, host or device.
  * q_i^e_i < 2^62, count <= 16.  Synchronous.  Errors: SMF_E_INVALID,
  * SMF_E_NOMEM, SMF_E_CUDA. */
@@ -469,15 +469,14 @@ int smf_smith_local(smf_ctx* ctx, const smf_bigmat* A, const uint64_t* q, const 
 
 /* Section 2's eliminations over Z/(m) (smf_det_mod, smf_smith_local and the
  * Phases 2 and 3 of smf_smith_form) take matrices of at least min_n columns
- * by panels of 16 columns when their entries fit 32-bit words (primes and
- * prime powers below 2^31): per column of a panel a pivot search and the
- * update of the panel alone, then the panel's pivot rows and one pass over
- * the trailing columns, which are read and written once per panel instead of
- * once per column.  Smaller matrices take one launch per column.  The pivots,
- * and so every result, are the same either way.  min_n = 0 restores the
- * defaults, 2560 for determinants and 1536 for local Smith forms (below them
- * the column loop was measured faster); it applies to later calls on this
- * context.  Errors: SMF_E_INVALID (no context, min_n < 0). */
+ * by panels of up to 32 columns when their entries fit 32-bit words (primes
+ * and prime powers below 2^31): each panel is reduced in the shared memory of
+ * one thread-block cluster, then one pass takes it to the trailing columns,
+ * which are read and written once per panel instead of once per column.
+ * Smaller matrices, and wider moduli, take one launch per column.  Every result
+ * is the same either way (the pivot rows may differ).  min_n = 0 restores the
+ * default, every size by panels (measured faster from n = 16 on); it applies to
+ * later calls on this context.  Errors: SMF_E_INVALID (no context, min_n < 0). */
 int smf_set_elim_panels(smf_ctx* ctx, int64_t min_n);
 
 /* Rational reconstruction (host only, no device work): the fraction a / b in

@@ -645,6 +645,7 @@ int smf_create(smf_ctx** out, int device, smf_form form, size_t hbm_budget_bytes
               cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess;
     for (auto& e : c->pev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (hbm_budget_bytes && hbm_budget_bytes < kPoolKeep) c->pool_keep = hbm_budget_bytes;
     ok = ok && cudaEventCreateWithFlags(&c->gdesc_ev, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
         for (cudaStream_t st : {c->aux, c->h2d, c->d2h})
@@ -684,6 +685,7 @@ int smf_destroy(smf_ctx* c) {
     if (c->gdesc_host) cudaFreeHost(c->gdesc_host);
     for (void* ph : c->pinned)
         if (ph) cudaFreeHost(ph);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     delete c;
     return SMF_OK;
 }
@@ -1903,7 +1905,6 @@ int smf_set_fused_crt(smf_ctx* ctx, int enable) {
 int smf_set_elim_panels(smf_ctx* ctx, int64_t min_n) {
     if (!ctx || min_n < 0) return SMF_E_INVALID;
     ctx->elim_panel_min_n = min_n ? min_n : kElimPanelMinN;
-    ctx->elim_local_panel_min_n = min_n ? min_n : kElimLocalPanelMinN;
     return SMF_OK;
 }
 

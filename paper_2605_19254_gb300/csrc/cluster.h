@@ -25,10 +25,15 @@ __device__ __forceinline__ void cluster_store(uint32_t* p, int rank, uint32_t v)
 }
 #endif
 
-// One cluster of C blocks (up to 16), as a programmatic dependent of the kernel before it.
+// One cluster of C blocks (up to 16), as a programmatic dependent of the kernel
+// before it.  smem_limit: the most dynamic shared memory any launch of the kernel
+// takes (the attribute is the kernel's, not the launch's, and other threads may
+// launch it at the same time with other sizes).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster(void (*kernel)(KArgs...), int C, int threads, size_t smem, cudaStream_t s, Args&&... args) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t launch_cluster(void (*kernel)(KArgs...), int C, int threads, size_t smem, size_t smem_limit, cudaStream_t s,
+                           Args&&... args) {
+    if (smem > smem_limit) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit);
     if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};

@@ -21,9 +21,11 @@
 // f' = floor(f 2^w / m) makes f y mod m = f y - floor(y f' / 2^w) m, at most
 // one m too large (w = 32 for m < 2^31, 64 for m < 2^62).
 //
-// Determinants and lockstep local forms (two or more lanes) take one launch per
-// column: the launch for column k eliminates
-// it and, in the threads that update column k+1, copies that column's new values
+// Moduli below 2^31 go by panels of columns, each reduced by one thread-block
+// cluster (see "Elimination by panels" below).  Wider ones, and matrices below
+// the threshold of smf_set_elim_panels, go column by column: determinants and
+// lockstep local forms (two or more lanes) take one launch per
+// column: the launch for column k eliminates it and, in the threads that update column k+1, copies that column's new values
 // into a compact buffer and finds its first unused unit row (atomicMin).  The
 // last of those blocks to finish (a counter, no waiting) takes that row as
 // column k+1's pivot, marks it used and stores its inverse, so the next launch
@@ -38,6 +40,7 @@
 #include <vector>
 
 #include "modarith.h"
+#include "panel.h"
 #include "smf_internal.h"
 
 namespace smf {
@@ -144,9 +147,9 @@ __global__ void elim_init_kernel(const int64_t* __restrict__ A, int64_t lda, int
     const int64_t a = A[i * lda + j];
 #pragma unroll
     for (int l = 0; l < L; l++) {
-        if (l >= md.n) break;
-        const int64_t r = a % (int64_t)md.m[l];
-        M[e * L + l] = (T)(r < 0 ? r + (int64_t)md.m[l] : r);
+        const int64_t m = (int64_t)md.m[l < md.n ? l : 0];  // (lanes not in use repeat lane 0)
+        const int64_t r = a % m;
+        M[e * L + l] = (T)(r < 0 ? r + m : r);
     }
 }
 
@@ -448,15 +451,18 @@ struct ElimBufs {
     static size_t counters(int64_t n) {
         return 1 + (size_t)(((n + kStepRows - 1) / kStepRows + kCountGroup - 1) / kCountGroup);
     }
-    cudaError_t alloc(int64_t n, cudaStream_t s) {
+    cudaError_t alloc(smf_ctx* ctx, int64_t n, cudaStream_t s) { return M.alloc(ctx, sizeof(T) * L * (size_t)n * (size_t)n, s); }
+    // what the column loop needs beside the matrix
+    cudaError_t alloc_columns(smf_ctx* ctx, int64_t n, cudaStream_t s) {
         cudaError_t e;
+        if (used.p) return cudaSuccess;
         const size_t nl = sizeof(T) * L * (size_t)n;
-        if ((e = M.alloc(nl * (size_t)n, s)) || (e = used.alloc(sizeof(int) * (size_t)n, s)) ||
-            (e = pivrow.alloc(sizeof(int64_t) * (size_t)n, s)) || (e = pivval.alloc(nl, s)) ||
-            (e = pinv.alloc(nl, s)) || (e = pinvs.alloc(nl, s)) || (e = colbuf.alloc(2 * nl, s)) ||
-            (e = cand.alloc(sizeof(unsigned) * (size_t)(n + 1), s)) ||
-            (e = counter.alloc(sizeof(unsigned) * counters(n), s)) || (e = f.alloc(nl, s)) || (e = fs.alloc(nl, s)) ||
-            (e = dead.alloc(sizeof(int), s)))
+        if ((e = used.alloc(ctx, sizeof(int) * (size_t)n, s)) ||
+            (e = pivrow.alloc(ctx, sizeof(int64_t) * (size_t)n, s)) || (e = pivval.alloc(ctx, nl, s)) ||
+            (e = pinv.alloc(ctx, nl, s)) || (e = pinvs.alloc(ctx, nl, s)) || (e = colbuf.alloc(ctx, 2 * nl, s)) ||
+            (e = cand.alloc(ctx, sizeof(unsigned) * (size_t)(n + 1), s)) ||
+            (e = counter.alloc(ctx, sizeof(unsigned) * counters(n), s)) || (e = f.alloc(ctx, nl, s)) || (e = fs.alloc(ctx, nl, s)) ||
+            (e = dead.alloc(ctx, sizeof(int), s)))
             return e;
         return cudaSuccess;
     }
@@ -467,10 +473,10 @@ struct ElimBufs {
 // the columns after k are updated, a column without a pivot ends it); else the
 // local form (every column but k stays current: deferred columns are kept).
 template <typename T, int L>
-cudaError_t elim_columns(ElimBufs<T, L>& b, T* M, int64_t n, const Lanes<T, L>& md, bool field,
+cudaError_t elim_columns(smf_ctx* ctx, ElimBufs<T, L>& b, T* M, int64_t n, const Lanes<T, L>& md, bool field,
                          std::vector<int64_t>* pivrow, std::vector<T>* pivval, cudaStream_t s) {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(b.used.p, 0, sizeof(int) * (size_t)n, s)) ||
+    if ((e = b.alloc_columns(ctx, n, s)) || (e = cudaMemsetAsync(b.used.p, 0, sizeof(int) * (size_t)n, s)) ||
         (e = cudaMemsetAsync(b.dead.p, 0, sizeof(int), s)) ||
         (e = cudaMemsetAsync(b.counter.p, 0, sizeof(unsigned) * ElimBufs<T, L>::counters(n), s)) ||
         (e = cudaMemsetAsync(b.cand.p, 0xFF, sizeof(unsigned) * (size_t)(n + 1), s)) ||
@@ -506,340 +512,284 @@ cudaError_t elim_columns(ElimBufs<T, L>& b, T* M, int64_t n, const Lanes<T, L>& 
 }
 
 // ---------------------------------------------------------------------------
-// Blocked elimination (32-bit lanes).  The column loop above reads and writes
-// the whole trailing block once per column: about n^3/3 entry updates of
-// 2 x 16 bytes for four lanes, which bounds it by memory.  Here panels of
-// kPanel columns are eliminated first on the panel alone (per column: the
-// pivot search, then every unused row's multiplier and the update of the
-// panel's other live columns), the pivot rows' trailing parts are brought up
-// to date within the panel (U), and the trailing columns take the panel's
-// kPanel pivots in one pass: M[i][j] -= sum_t F[i][t] U[t][j].  The same
-// pivots, the same multipliers and the same values as one column at a time;
-// the trailing block is read and written once per panel.
+// Elimination by panels (32-bit lanes).  The column loop above reads and writes
+// the whole trailing block once per column, one launch each.  Here one cluster
+// reduces a panel of kPanel columns (panel.h) to its transform S, and one pass
+// applies it to the trailing columns, M[i][j] += sum_t S[i][t] M[p_t][j], for the
+// rows i without a pivot, whose list each panel hands to the next: the matrix is
+// read and written once per panel, and the pivot rows stay as they are.
 //
-// Two kinds (template flag LOC):
-//  - a determinant (LOC = false): a column without a pivot ends the call (the
-//    caller falls back to the column loop); the trailing columns are [c1, n);
-//  - a local Smith form (LOC = true): a column without a unit pivot is
-//    deferred and stays live, as in the column loop.  The deferred columns are
-//    listed in increasing order (dcols[0 .. *ndef)); *ndef0 is their count
-//    before the current panel.  The panel's own deferred columns are updated
-//    within the panel by its later pivots; the trailing columns of the panel
-//    are the earlier ones, dcols[0 .. *ndef0), followed by [c1, n).  A panel
-//    position without a pivot contributes U = 0.
-constexpr int kPanel = 16;
-// Matrices below the context's thresholds (elim_panel_min_n, 2560, for
-// determinants; elim_local_panel_min_n, 1536, for local forms; unless
-// smf_set_elim_panels changes them) keep the column loop: its one launch per
-// column against the panels' two per column plus two per panel (measured
-// four-lane determinants: n = 2003 0.045 s by columns, 0.053 s blocked;
-// n = 5003 0.416 against 0.205 s).
+//  - a determinant: a column without a unit ends the call (*fallback);
+//  - a local Smith form: such a column is deferred and stays live; the deferred
+//    columns are listed in increasing order (dcols[0 .. *ndef)), and the trailing
+//    columns are all of them, the panel's own too, followed by [c1, n).
+//
+// GB300, four 31-bit primes: n = 2003 8.1 ms (44 ms with a launch per column),
+// n = 5003 69 ms (210 ms by panels of 16 columns with two launches per column of
+// the panel).
+constexpr int kPanel = 32;
 
-// trailing column x of a panel: an earlier deferred column, then [c1, n)
-__device__ __forceinline__ int64_t trail_col(int64_t x, int64_t nd0, const int64_t* __restrict__ dcols, int64_t c1) {
-    return x < nd0 ? dcols[x] : c1 + (x - nd0);
+// trailing column x of a panel: a deferred column, then [c1, n)
+__device__ __forceinline__ int64_t trail_col(int64_t x, int64_t nd, const int* __restrict__ dcols, int64_t c1) {
+    return x < nd ? dcols[x] : c1 + (x - nd);
 }
 
-// The first unused row whose entry in column c is a unit in every lane
-// (atomicMin of each block's smallest candidate).  A local form's first column
-// of a panel also records the count of deferred columns before the panel.
-template <int L, bool LOC>
-__global__ void __launch_bounds__(256)
-bd_search_kernel(const uint32_t* __restrict__ M, int64_t n, int64_t c, int64_t c0, Lanes<uint32_t, L> md,
-                 const int* __restrict__ used, unsigned* __restrict__ cand, const int* __restrict__ dead,
-                 const int* __restrict__ ndef, int* __restrict__ ndef0) {
-    pdl_wait();
-    pdl_trigger();
-    if (*dead) return;
-    if (LOC && c == c0 && blockIdx.x == 0 && threadIdx.x == 0) *ndef0 = *ndef;
-    __shared__ unsigned wmin[8];
+__global__ void bd_init_kernel(int64_t n, int* __restrict__ live, int* __restrict__ count, int* __restrict__ flag,
+                               int* __restrict__ ndef, uint32_t* __restrict__ det, int dets) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned v = 0xFFFFFFFFu;
-    if (i < n && !used[i] && joint_unit<uint32_t, L>(M + (i * n + c) * L, md)) v = (unsigned)i;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) wmin[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned b = wmin[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); w++) b = min(b, wmin[w]);
-        if (b != 0xFFFFFFFFu) atomicMin(cand + c, b);
+    if (i < n) live[i] = (int)i;
+    if (i < dets) det[i] = 1;
+    if (i == 0) {
+        *count = (int)n;
+        *flag = 0;
+        *ndef = 0;
     }
 }
 
-// Column c (panel [c0, c1)): its pivot p = cand[c], the pivot's inverse in
-// every lane, each unused row's multiplier f = M[i][c] / M[p][c] with its
-// Shoup companion (kept in F and Fs at panel position c - c0), and
-// M[i][j] -= f M[p][j] for the panel's other live columns: j in (c, c1) and,
-// in a local form, the panel's deferred columns before c.  No pivot: a
-// determinant's call falls back to the column loop; a local form defers c.
-template <int L, bool LOC>
+// The pass over the trailing block: 64 live rows by 128 words per block.  A
+// thread keeps its word of the panel's KT pivot rows in registers and takes 32
+// rows, four at a time, whose multipliers it reads from shared memory.  Bound by
+// the integer pipe: KT 64-bit multiply-adds per word (28 a clock and SM), against
+// 8 bytes of memory traffic.
+constexpr int kTrailRows = 64, kTrailWords = 128;
+template <int L, PanelRed RED, int KT, bool LOC>
 __global__ void __launch_bounds__(256)
-bd_panel_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c, int64_t c0, int64_t c1, Lanes<uint32_t, L> md,
-                int* __restrict__ used, const unsigned* __restrict__ cand, int64_t* __restrict__ pivrow,
-                uint32_t* __restrict__ pivval, uint32_t* __restrict__ F, uint32_t* __restrict__ Fs,
-                int* __restrict__ dead, int64_t* __restrict__ dcols, int* __restrict__ ndef) {
+bd_trail_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c0, int w, int64_t c1,
+                const __grid_constant__ PanelMod<L> md, const int* __restrict__ live, const int* __restrict__ count,
+                const int* __restrict__ piv, const uint32_t* __restrict__ G, const int* __restrict__ flag,
+                const int* __restrict__ dcols, const int* __restrict__ ndef) {
+    constexpr int SW = KT + 4;  // padded row of multipliers of one lane
+    __shared__ __align__(16) uint32_t ss[kTrailRows * L * SW];
+    __shared__ int sid[kTrailRows], sp[KT];
     pdl_wait();
     pdl_trigger();
-    if (*dead) return;
-    const unsigned pu = cand[c];
-    if (pu >= (unsigned)n) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            if constexpr (LOC) {  // one writer: the list stays in column order
-                const int d = *ndef;
-                dcols[d] = c;
-                *ndef = d + 1;
-            } else {
-                *dead = 1;
-            }
-        }
-        return;
-    }
-    const int64_t p = pu;
-    const uint32_t* prow = M + (p * n) * L;
-    uint32_t inv[L];
-#pragma unroll
-    for (int l = 0; l < L; l++)
-        inv[l] = l < md.n ? inv_mod32(prow[c * L + l], md.m[l]) : 0u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {  // every other thread skips row p by its index
-        pivrow[c] = p;
-#pragma unroll
-        for (int l = 0; l < L; l++) pivval[c * L + l] = prow[c * L + l];
-        used[p] = 1;
-    }
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || i == p || used[i]) return;
-    uint32_t* row = M + (i * n) * L;
-    uint32_t f[L], fs[L];
-#pragma unroll
-    for (int l = 0; l < L; l++) {
-        f[l] = fs[l] = 0;
-        if (l < md.n) {
-            f[l] = mulmod32_rcp(row[c * L + l], inv[l], md.m[l], md.rcp[l]);
-            fs[l] = ModOps<uint32_t>::shoup_rcp(f[l], md.m[l], md.rcp[l]);
-        }
-        F[(i * kPanel + (c - c0)) * L + l] = f[l];
-        Fs[(i * kPanel + (c - c0)) * L + l] = fs[l];
-    }
-    // (columns before c in the panel: only a local form's deferred ones, whose
-    // pivrow was settled by an earlier launch, are still live)
-    for (int64_t j = LOC ? c0 : c + 1; j < c1; j++) {
-        if (LOC && j <= c && (j == c || pivrow[j] >= 0)) continue;
-#pragma unroll
-        for (int l = 0; l < L; l++) {
-            if (l >= md.n) break;
-            const uint32_t m = md.m[l];
-            const uint32_t t = ModOps<uint32_t>::mul(prow[j * L + l], f[l], fs[l], m);
-            const uint32_t a = row[j * L + l];
-            row[j * L + l] = a >= t ? a - t : a + m - t;
-        }
-    }
-}
-
-// The panel's pivot rows on the trailing columns (a determinant: [c1, n); a
-// local form: also the deferred columns before the panel): row p_t takes the
-// panel's earlier pivots' eliminations, U_t = M[p_t] - sum_(t' < t) F[p_t][t'] U_t'
-// (one thread per column, the panel's rows in registers), written back in
-// place.  Threads beyond the count of trailing columns return.
-template <int L, bool LOC>
-__global__ void __launch_bounds__(128)
-bd_urows_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c0, int w, int64_t c1, Lanes<uint32_t, L> md,
-                const int64_t* __restrict__ pivrow, const uint32_t* __restrict__ F, const uint32_t* __restrict__ Fs,
-                const int* __restrict__ dead, const int64_t* __restrict__ dcols, const int* __restrict__ ndef0) {
-    pdl_wait();
-    pdl_trigger();
-    if (*dead) return;
-    const int64_t nd0 = LOC ? (int64_t)*ndef0 : 0;
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= nd0 + (n - c1)) return;
-    const int64_t j = trail_col(x, nd0, dcols, c1);
-    uint32_t U[kPanel][L];
-#pragma unroll
-    for (int t = 0; t < kPanel; t++) {
-        if (t >= w) break;
-        const int64_t p = pivrow[c0 + t];
-#pragma unroll
-        for (int l = 0; l < L; l++) U[t][l] = 0;
-        if (LOC && p < 0) continue;  // a deferred panel column: no elimination
-        uint32_t* e = M + (p * n + j) * L;
-#pragma unroll
-        for (int l = 0; l < L; l++) {
-            if (l >= md.n) continue;
-            const uint32_t m = md.m[l];
-            uint32_t u = e[l];
-#pragma unroll
-            for (int t2 = 0; t2 < kPanel; t2++) {
-                if (t2 >= t) break;
-                const size_t fi = ((size_t)p * kPanel + t2) * L + l;
-                const uint32_t xx = ModOps<uint32_t>::mul(U[t2][l], F[fi], Fs[fi], m);
-                u = u >= xx ? u - xx : u + m - xx;
-            }
-            U[t][l] = u;
-            e[l] = u;
-        }
-    }
-}
-
-// The trailing block: every row still unused (after the panel) and every
-// trailing column takes M[i][j] -= sum_t F[i][t] U_t[j].  A block covers 32
-// rows by 64 trailing columns: the panel's U rows over its columns and its
-// rows' multipliers in shared memory, eight entries per thread.
-constexpr int kTrailRows = 32, kTrailCols = 64;
-template <int L, bool LOC>
-__global__ void __launch_bounds__(256)
-bd_trail_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c0, int w, int64_t c1, Lanes<uint32_t, L> md,
-                const int* __restrict__ used, const int64_t* __restrict__ pivrow, const uint32_t* __restrict__ F,
-                const uint32_t* __restrict__ Fs, const int* __restrict__ dead, const int64_t* __restrict__ dcols,
-                const int* __restrict__ ndef0) {
-    pdl_wait();
-    pdl_trigger();
-    if (*dead) return;
-    const int64_t nd0 = LOC ? (int64_t)*ndef0 : 0;
-    const int64_t ncols = nd0 + (n - c1);
-    const int64_t x0 = (int64_t)blockIdx.x * kTrailCols;
-    if (x0 >= ncols) return;  // (the grid bounds a local form's deferred count by c0)
-    __shared__ uint32_t Us[kPanel][kTrailCols][L];
-    __shared__ uint32_t Fsh[kTrailRows][kPanel][L], Fssh[kTrailRows][kPanel][L];
-    __shared__ int live[kTrailRows];
-    __shared__ int any;
-    const int64_t r0 = (int64_t)blockIdx.y * kTrailRows;
-    if (threadIdx.x == 0) any = 0;
-    __syncthreads();
-    if (threadIdx.x < kTrailRows) {
-        const int64_t i = r0 + threadIdx.x;
-        live[threadIdx.x] = i < n && !used[i];
-        if (live[threadIdx.x]) any = 1;
+    if (*flag) return;
+    const int64_t nd = LOC ? (int64_t)*ndef : 0;
+    const int64_t ncols = nd + (n - c1);
+    const int nl = *count;
+    const int64_t x0 = (int64_t)blockIdx.x * (kTrailWords / L);
+    const int r0 = (int)blockIdx.y * kTrailRows;
+    if (x0 >= ncols || r0 >= nl) return;  // (the grid bounds both)
+    const int nr = min(kTrailRows, nl - r0);
+    const int tid = threadIdx.x;
+    if (tid < nr) sid[tid] = live[r0 + tid];
+    if (tid < KT) sp[tid] = tid < w ? piv[c0 + tid] : -1;
+    for (int e = tid; e < nr * L * (KT / 4); e += 256) {
+        const uint4 v = *reinterpret_cast<const uint4*>(G + (size_t)r0 * L * KT + 4 * (size_t)e);
+        *reinterpret_cast<uint4*>(ss + e / (KT / 4) * SW + e % (KT / 4) * 4) = v;
     }
     __syncthreads();
-    if (!any) return;  // every row of the tile is a pivot row already
-    for (int x = threadIdx.x; x < kPanel * kTrailCols; x += blockDim.x) {
-        const int t = x / kTrailCols, jj = x % kTrailCols;
-        const int64_t xx = x0 + jj;
-        const int64_t p = t < w ? pivrow[c0 + t] : -1;
-        const bool ok = t < w && xx < ncols && p >= 0;
-        const int64_t j = ok ? trail_col(xx, nd0, dcols, c1) : 0;
-#pragma unroll
-        for (int l = 0; l < L; l++) Us[t][jj][l] = ok ? M[(p * n + j) * L + l] : 0u;
-    }
-    for (int x = threadIdx.x; x < kTrailRows * kPanel; x += blockDim.x) {
-        const int rr = x / kPanel, t = x % kPanel;
-        const int64_t i = r0 + rr;
-#pragma unroll
-        for (int l = 0; l < L; l++) {
-            const bool ok = t < w && live[rr];
-            Fsh[rr][t][l] = ok ? F[((size_t)i * kPanel + t) * L + l] : 0u;
-            Fssh[rr][t][l] = ok ? Fs[((size_t)i * kPanel + t) * L + l] : 0u;
-        }
-    }
-    __syncthreads();
-    const int jj = threadIdx.x % kTrailCols;
-    const int64_t xx = x0 + jj;
+    const int c = tid % kTrailWords, l = c % L;
+    const int64_t xx = x0 + c / L;
     if (xx >= ncols) return;
-    const int64_t j = trail_col(xx, nd0, dcols, c1);
-    for (int rr = threadIdx.x / kTrailCols; rr < kTrailRows; rr += blockDim.x / kTrailCols) {
-        if (!live[rr]) continue;
-        uint32_t* e = M + ((r0 + rr) * n + j) * L;
-        uint32_t v[L];
+    uint32_t* Mj = M + trail_col(xx, nd, dcols, c1) * L + l;
+    const size_t ld = (size_t)n * L;
+    uint32_t y[KT];
 #pragma unroll
-        for (int l = 0; l < L; l++) v[l] = e[l];
+    for (int t = 0; t < KT; t++) y[t] = sp[t] >= 0 ? Mj[sp[t] * ld] : 0u;
+    const uint32_t m = md.m[l], ninv = md.ninv[l];
+    for (int r = tid / kTrailWords; r < nr; r += 8) {
+        uint64_t acc[4];
+        const uint32_t* f[4];
 #pragma unroll
-        for (int t = 0; t < kPanel; t++) {
-            if (t >= w) break;
-#pragma unroll
-            for (int l = 0; l < L; l++) {
-                if (l >= md.n) break;
-                const uint32_t m = md.m[l];
-                const uint32_t y = ModOps<uint32_t>::mul(Us[t][jj][l], Fsh[rr][t][l], Fssh[rr][t][l], m);
-                v[l] = v[l] >= y ? v[l] - y : v[l] + m - y;
-            }
+        for (int i = 0; i < 4; i++) {
+            const int ri = r + 2 * i < nr ? r + 2 * i : r;
+            f[i] = ss + (ri * L + l) * SW;
+            acc[i] = mac_start<RED>(Mj[sid[ri] * ld], m);
         }
 #pragma unroll
-        for (int l = 0; l < L; l++) e[l] = v[l];
+        for (int t = 0; t < KT; t += 4)
+#pragma unroll
+            for (int i = 0; i < 4; i++) acc[i] = mac4<RED>(acc[i], *reinterpret_cast<const uint4*>(f[i] + t), y + t, m);
+#pragma unroll
+        for (int i = 0; i < 4; i++)
+            if (r + 2 * i < nr) Mj[sid[r + 2 * i] * ld] = mac_end<RED>(acc[i], m, ninv);
     }
 }
 
-// The blocked column loop on the n x n matrix in M (32-bit lanes): each
-// column's pivot row (-1 for a local form's deferred column) and its values,
-// as elim_columns gives them.  A determinant's *fallback: a column without a
-// pivot that is a unit in every lane (the caller then takes the column loop
-// above); a local form never falls back.
+template <int L, PanelRed RED, bool LOC>
+cudaError_t launch_trail(int gw, uint32_t* M, int64_t n, int64_t c0, int w, int64_t c1, int64_t cols, int64_t rows,
+                         const PanelMod<L>& md, const int* live, const int* count, const int* piv, const uint32_t* G,
+                         const int* flag, const int* dcols, const int* ndef, cudaStream_t s) {
+    const dim3 grid((unsigned)((cols + kTrailWords / L - 1) / (kTrailWords / L)),
+                    (unsigned)((rows + kTrailRows - 1) / kTrailRows));
+    return gw > 16 ? launch_pdl(bd_trail_kernel<L, RED, 32, LOC>, grid, dim3(256), 0, s, M, n, c0, w, c1, md, live, count,
+                                piv, G, flag, dcols, ndef)
+                   : launch_pdl(bd_trail_kernel<L, RED, 16, LOC>, grid, dim3(256), 0, s, M, n, c0, w, c1, md, live, count,
+                                piv, G, flag, dcols, ndef);
+}
+
+// An elimination by panels on the stream: what it leaves on the device.
+struct Blocked {
+    StreamBuf buf;
+    int* piv;       // [n] each column's pivot row (-1 for a local form's deferred column)
+    int* flag;      // a determinant: a column without a pivot that is a unit in every lane
+    uint32_t* det;  // [2 L] its pivots' product in every lane, numerators and denominators
+    int* live;      // the rows without a pivot, and their count
+    int* count;
+    int* dcols;     // the deferred columns
+};
+
+// The n x n matrix in M (32-bit lanes) by panels.  Only enqueues.
 template <int L, bool LOC>
-cudaError_t elim_blocked(ElimBufs<uint32_t, L>& b, uint32_t* M, int64_t n, const Lanes<uint32_t, L>& md,
-                         std::vector<int64_t>* pivrow, std::vector<uint32_t>* pivval, bool* fallback, cudaStream_t s) {
+cudaError_t elim_blocked(smf_ctx* ctx, uint32_t* M, int64_t n, const Lanes<uint32_t, L>& md, Blocked* out,
+                         cudaStream_t s) {
     cudaError_t e;
-    StreamBuf F, Fs, dl, nd;
-    const size_t fb = sizeof(uint32_t) * (size_t)n * kPanel * L;
-    if ((e = F.alloc(fb, s)) || (e = Fs.alloc(fb, s))) return e;
-    if (LOC) {
-        // a deferred panel position leaves F stale; zeros keep every read defined
-        if ((e = dl.alloc(sizeof(int64_t) * (size_t)n, s)) || (e = nd.alloc(2 * sizeof(int), s)) ||
-            (e = cudaMemsetAsync(nd.p, 0, 2 * sizeof(int), s)) || (e = cudaMemsetAsync(F.p, 0, fb, s)) ||
-            (e = cudaMemsetAsync(Fs.p, 0, fb, s)))
-            return e;
+    PanelArgs<L> a{};
+    for (int l = 0; l < L; l++) panel_mod(a.md, l, md.m[l < md.n ? l : 0], md.q[l < md.n ? l : 0]);
+    const PanelRed red = panel_red(a.md);
+    const int pw = panel_width(n, L, kPanel), gw = pw > 16 ? 32 : 16;
+    // scratch: G, ybuf, then [piv n | flag | det 2L] read back in one copy, live lists, counts, deferred columns
+    const size_t words = (size_t)n * L * gw + panel_scratch(pw * L) + (size_t)n + 1 + 2 * L + 2 * (size_t)n + 2 + (size_t)n + 1;
+    if ((e = out->buf.alloc(ctx, sizeof(uint32_t) * words, s))) return e;
+    uint32_t* G = (uint32_t*)out->buf.p;
+    uint32_t* ybuf = G + (size_t)n * L * gw;
+    int* piv = (int*)(ybuf + panel_scratch(pw * L));
+    int* flag = piv + n;
+    uint32_t* det = (uint32_t*)flag + 1;
+    int* live[2] = {(int*)det + 2 * L, (int*)det + 2 * L + n};
+    int* count = live[1] + n;
+    int* ndef = count + 2;
+    int* dcols = ndef + 1;
+    bd_init_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, live[0], count, flag, ndef, det, 2 * L);
+    if ((e = cudaGetLastError())) return e;
+    a.M = M;
+    a.n = a.ld = n;
+    a.ybuf = ybuf;
+    a.piv = piv;
+    a.flag = flag;
+    a.G = G;
+    a.gw = gw;
+    a.det = det;
+    a.dcols = dcols;
+    a.ndef = ndef;
+    int k = 0;
+    for (int64_t c0 = 0; c0 < n; c0 += pw, k ^= 1) {
+        const int64_t c1 = std::min<int64_t>(n, c0 + pw);
+        a.c0 = c0;
+        a.w = (int)(c1 - c0);
+        a.live = live[k];
+        a.count = count + k;
+        a.live_out = live[k ^ 1];
+        a.count_out = count + (k ^ 1);
+        if ((e = launch_panel<L, LOC ? PanelKind::kLocal : PanelKind::kDet>(a, n, s))) return e;
+        if (!LOC && c1 >= n) continue;
+        // a determinant leaves n - c1 rows; a local form's rows and deferred columns are known on the device
+        const int64_t cols = LOC ? n : n - c1, rows = LOC ? n : n - c1;
+        e = red == PanelRed::kNarrow
+                ? launch_trail<L, PanelRed::kNarrow, LOC>(gw, M, n, c0, a.w, c1, cols, rows, a.md, a.live_out, a.count_out,
+                                                          piv, G, flag, dcols, ndef, s)
+                : launch_trail<L, PanelRed::kWide, LOC>(gw, M, n, c0, a.w, c1, cols, rows, a.md, a.live_out, a.count_out,
+                                                        piv, G, flag, dcols, ndef, s);
+        if (e) return e;
     }
-    if ((e = cudaMemsetAsync(b.used.p, 0, sizeof(int) * (size_t)n, s)) ||
-        (e = cudaMemsetAsync(b.dead.p, 0, sizeof(int), s)) ||
-        (e = cudaMemsetAsync(b.cand.p, 0xFF, sizeof(unsigned) * (size_t)(n + 1), s)) ||
-        (e = cudaMemsetAsync(b.pivrow.p, 0xFF, sizeof(int64_t) * (size_t)n, s)))
-        return e;
-    int* used = (int*)b.used.p;
-    int* dead = (int*)b.dead.p;
-    unsigned* cand = (unsigned*)b.cand.p;
-    int64_t* pr = (int64_t*)b.pivrow.p;
-    uint32_t* pv = (uint32_t*)b.pivval.p;
-    int64_t* dcols = LOC ? (int64_t*)dl.p : nullptr;
-    int* ndef = LOC ? (int*)nd.p : nullptr;  // [0]: deferred so far, [1]: before the current panel
-    int* ndef0 = LOC ? (int*)nd.p + 1 : nullptr;
-    const unsigned rblocks = (unsigned)((n + 255) / 256);
-    for (int64_t c0 = 0; c0 < n; c0 += kPanel) {
-        const int64_t c1 = std::min<int64_t>(n, c0 + kPanel);
-        const int w = (int)(c1 - c0);
-        for (int64_t c = c0; c < c1; c++) {
-            if ((e = launch_pdl(bd_search_kernel<L, LOC>, dim3(rblocks), dim3(256), 0, s, (const uint32_t*)M, n, c, c0,
-                                md, (const int*)used, cand, (const int*)dead, (const int*)ndef, ndef0)) ||
-                (e = launch_pdl(bd_panel_kernel<L, LOC>, dim3(rblocks), dim3(256), 0, s, M, n, c, c0, c1, md, used,
-                                (const unsigned*)cand, pr, pv, (uint32_t*)F.p, (uint32_t*)Fs.p, dead, dcols, ndef)))
-                return e;
-        }
-        if (!LOC && c1 >= n) break;
-        // trailing columns: at most c0 deferred ones (a local form) and [c1, n)
-        const int64_t rest = (LOC ? c0 : 0) + (n - c1);
-        if (rest == 0) continue;
-        if ((e = launch_pdl(bd_urows_kernel<L, LOC>, dim3((unsigned)((rest + 127) / 128)), dim3(128), 0, s, M, n, c0,
-                            w, c1, md, (const int64_t*)pr, (const uint32_t*)F.p, (const uint32_t*)Fs.p,
-                            (const int*)dead, (const int64_t*)dcols, (const int*)ndef0)))
-            return e;
-        const dim3 grid((unsigned)((rest + kTrailCols - 1) / kTrailCols), (unsigned)((n + kTrailRows - 1) / kTrailRows));
-        if ((e = launch_pdl(bd_trail_kernel<L, LOC>, grid, dim3(256), 0, s, M, n, c0, w, c1, md, (const int*)used,
-                            (const int64_t*)pr, (const uint32_t*)F.p, (const uint32_t*)Fs.p, (const int*)dead,
-                            (const int64_t*)dcols, (const int*)ndef0)))
-            return e;
-    }
-    int dead_h = 0;
-    pivrow->resize(n);
-    pivval->resize((size_t)n * L);
-    if ((e = cudaMemcpyAsync(&dead_h, dead, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
-        (e = cudaMemcpyAsync(pivrow->data(), pr, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, s)) ||
-        (e = cudaMemcpyAsync(pivval->data(), pv, sizeof(uint32_t) * L * n, cudaMemcpyDeviceToHost, s)) ||
+    out->piv = piv;
+    out->flag = flag;
+    out->det = det;
+    out->live = live[k];
+    out->count = count + k;
+    out->dcols = dcols;
+    return cudaSuccess;
+}
+
+// Waits for it: the pivot rows, and for a determinant (dets not null) the
+// fractions dets[l] / dets[L + l] and whether a column had no pivot.
+template <int L>
+cudaError_t read_blocked(const Blocked& b, int64_t n, std::vector<int64_t>* pivrow, uint32_t* dets, bool* no_pivot,
+                         cudaStream_t s) {
+    cudaError_t e;
+    std::vector<int> h((size_t)n + 1 + 2 * L);
+    if ((e = cudaMemcpyAsync(h.data(), b.piv, sizeof(int) * h.size(), cudaMemcpyDeviceToHost, s)) ||
         (e = cudaStreamSynchronize(s)))
         return e;
-    *fallback = dead_h != 0;
+    pivrow->assign(h.begin(), h.begin() + n);
+    if (!dets) return cudaSuccess;
+    *no_pivot = h[n] != 0;
+    for (int l = 0; l < 2 * L; l++) dets[l] = (uint32_t)h[n + 1 + l];
     return cudaSuccess;
+}
+
+// The levels of a small block that a joint elimination leaves (rows live[],
+// columns dcols[], nb of each): block l of the grid takes modulus l = q^e.
+// While an entry is a unit it is a pivot and its row and column go; then every
+// entry left is divided by q, and the rest goes on over Z/(q^(e-1)).
+// out[l][t]: the size left after level t, the number of invariant factors
+// divisible by q^(t+1); out[L][0] = nb, and nothing else when nb > kSmallBlock.
+// One launch and one read, where each level took an elimination, a read and a
+// gather (about 0.3 ms a level).
+constexpr int kSmallBlock = 192, kSmallThreads = 256, kSmallLevels = 32;
+struct SmallLevels {
+    uint32_t m[4], q[4];
+    int e[4];
+};
+template <int L>
+__global__ void __launch_bounds__(kSmallThreads)
+local_small_kernel(const uint32_t* __restrict__ M, int64_t n, const int* __restrict__ live,
+                   const int* __restrict__ count, const int* __restrict__ dcols, SmallLevels lv, int* __restrict__ out) {
+    extern __shared__ uint32_t B[];  // [nb][nb]
+    __shared__ int ri[kSmallBlock], ci[kSmallBlock];
+    __shared__ unsigned s_at;
+    __shared__ uint32_t s_inv;
+    const int nb = *count, l = blockIdx.x, tid = threadIdx.x;
+    if (l == 0 && tid == 0) out[L * kSmallLevels] = nb;
+    if (nb > kSmallBlock) return;
+    const uint32_t q = lv.q[l];
+    uint32_t m = lv.m[l];
+    for (int x = tid; x < nb * nb; x += kSmallThreads) {
+        const int a = x / nb, b = x % nb;
+        B[x] = M[((size_t)live[a] * n + dcols[b]) * L + l];
+    }
+    for (int x = tid; x < nb; x += kSmallThreads) ri[x] = ci[x] = x;  // the rows and columns left: [0, k)
+    int k = nb;
+    for (int t = 0; t < lv.e[l] && k > 0; t++, m /= q) {
+        const uint64_t rcp = UINT64_MAX / m;
+        for (;;) {
+            __syncthreads();
+            if (tid == 0) s_at = 0xFFFFFFFFu;
+            __syncthreads();
+            for (int x = tid; x < k * k; x += kSmallThreads)
+                if (B[ri[x / k] * nb + ci[x % k]] % q != 0) {
+                    atomicMin(&s_at, (unsigned)x);
+                    break;
+                }
+            __syncthreads();
+            const unsigned at = s_at;
+            if (at == 0xFFFFFFFFu) break;
+            const int pr = ri[at / k], pc = ci[at % k], lr = ri[k - 1], lc = ci[k - 1];
+            if (tid == 0) s_inv = inv_mod32(B[pr * nb + pc], m);
+            __syncthreads();
+            if (tid == 0) {  // the last row and column take the places of the pivot's
+                ri[at / k] = lr;
+                ci[at % k] = lc;
+            }
+            k--;
+            __syncthreads();
+            for (int x = tid; x < k * k; x += kSmallThreads) {
+                const int r = ri[x / k], c = ci[x % k];
+                const uint32_t f = mulmod32_rcp(B[r * nb + pc], s_inv, m, rcp);
+                const uint32_t y = mulmod32_rcp(f, B[pr * nb + c], m, rcp), v = B[r * nb + c];
+                B[r * nb + c] = v >= y ? v - y : v + m - y;
+            }
+        }
+        if (tid == 0) out[l * kSmallLevels + t] = k;
+        for (int x = tid; x < k * k; x += kSmallThreads) B[ri[x / k] * nb + ci[x % k]] /= q;
+    }
 }
 
 // The column loop of a local form (every column but k stays current), by
 // panels when the entries are 32-bit and the matrix has at least
-// ctx->elim_local_panel_min_n columns.
+// ctx->elim_panel_min_n columns.
 template <typename T, int L>
 cudaError_t elim_local(smf_ctx* ctx, ElimBufs<T, L>& b, T* M, int64_t n, const Lanes<T, L>& md,
                        std::vector<int64_t>* pivrow, std::vector<T>* pivval, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
-        if (n >= ctx->elim_local_panel_min_n) {
-            bool fallback = false;
-            return elim_blocked<L, true>(b, M, n, md, pivrow, pivval, &fallback, s);
+        if (n >= ctx->elim_panel_min_n) {
+            Blocked r;
+            const cudaError_t e = elim_blocked<L, true>(ctx, M, n, md, &r, s);
+            return e ? e : read_blocked<L>(r, n, pivrow, nullptr, nullptr, s);
         }
     }
-    return elim_columns<T, L>(b, M, n, md, false, pivrow, pivval, s);
+    return elim_columns<T, L>(ctx, b, M, n, md, false, pivrow, pivval, s);
 }
 
 uint64_t mulmod_host(uint64_t a, uint64_t b, uint64_t m) { return (uint64_t)((unsigned __int128)a * b % m); }
@@ -867,7 +817,7 @@ int det_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const uint
         md.rcp[l] = UINT64_MAX / (uint64_t)q[l];
     }
     ElimBufs<T, L> b;
-    cudaError_t e = b.alloc(n, s);
+    cudaError_t e = b.alloc(ctx, n, s);
     if (e) return elim_fail(ctx, "det_mod: device allocation", e);
     T* M = (T*)b.M.p;
     elim_init_kernel<T, L><<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(A, lda, n, M, md);
@@ -876,26 +826,28 @@ int det_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const uint
     if ((e = cudaGetLastError())) return elim_fail(ctx, "det_mod", e);
     bool blocked = false;
     if constexpr (sizeof(T) == 4) {
-        // 31-bit primes and a matrix of several panels: blocked elimination;
-        // a column without a joint unit pivot goes back to the column loop
+        // 31-bit primes: by panels.  A column without a joint unit pivot sends
+        // several primes back to one at a time (below); with one prime det = 0
         if (n >= ctx->elim_panel_min_n) {
-            bool fallback = false;
-            if ((e = elim_blocked<L, false>(b, M, n, md, &pr, &pv, &fallback, s))) return elim_fail(ctx, "det_mod", e);
-            blocked = !fallback;
-            if (fallback) {  // the matrix again, for the column loop
-                elim_init_kernel<T, L><<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(A, lda, n, M, md);
-                if ((e = cudaGetLastError())) return elim_fail(ctx, "det_mod", e);
-            }
+            bool no_pivot = false;
+            uint32_t dets[2 * L];
+            Blocked r;
+            if ((e = elim_blocked<L, false>(ctx, M, n, md, &r, s)) ||
+                (e = read_blocked<L>(r, n, &pr, dets, &no_pivot, s)))
+                return elim_fail(ctx, "det_mod", e);
+            blocked = true;
+            if (no_pivot) pr.assign(n, -1);
+            else pv.assign(dets, dets + 2 * L);
         }
     }
-    if (!blocked && (e = elim_columns<T, L>(b, M, n, md, true, &pr, &pv, s))) return elim_fail(ctx, "det_mod", e);
+    if (!blocked && (e = elim_columns<T, L>(ctx, b, M, n, md, true, &pr, &pv, s))) return elim_fail(ctx, "det_mod", e);
     if (std::any_of(pr.begin(), pr.end(), [](int64_t r) { return r < 0; })) {
         if (nq == 1) {
             det[0] = 0;
             return SMF_OK;
         }
         for (int l = 0; l < nq; l++) {
-            const int st = det_lanes<T, L>(ctx, A, lda, n, q + l, 1, det + l, s);
+            const int st = det_lanes<T, 1>(ctx, A, lda, n, q + l, 1, det + l, s);
             if (st) return st;
         }
         return SMF_OK;
@@ -910,7 +862,9 @@ int det_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const uint
     }
     for (int l = 0; l < nq; l++) {
         uint64_t d = 1 % q[l];
-        for (int64_t k = 0; k < n; k++) d = mulmod_host(d, (uint64_t)pv[k * L + l], q[l]);
+        if (blocked) d = mulmod_host(pv[l], inv_mod32((uint32_t)pv[L + l], (uint32_t)q[l]), q[l]);
+        else
+            for (int64_t k = 0; k < n; k++) d = mulmod_host(d, (uint64_t)pv[k * L + l], q[l]);
         if (((n - cycles) & 1) && d) d = q[l] - d;
         det[l] = d;
     }
@@ -928,7 +882,7 @@ int local_levels(smf_ctx* ctx, ElimBufs<T, 1>& b, StreamBuf& M2, int64_t nb, uin
     T* M = (T*)b.M.p;
     T* Mn = (T*)M2.p;
     StreamBuf idx;
-    cudaError_t ce = idx.alloc(sizeof(int64_t) * 2 * (size_t)std::max<int64_t>(nb, 1), s);
+    cudaError_t ce = idx.alloc(ctx, sizeof(int64_t) * 2 * (size_t)std::max<int64_t>(nb, 1), s);
     if (ce) return elim_fail(ctx, "smith_local: device allocation", ce);
     int64_t size = nb;
     std::vector<int64_t> pr;
@@ -996,14 +950,45 @@ int local_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const ui
     StreamBuf joint, idx;
     {
         ElimBufs<T, L> b;
-        cudaError_t ce = b.alloc(n, s);
+        cudaError_t ce = b.alloc(ctx, n, s);
         if (ce) return elim_fail(ctx, "smith_local: device allocation", ce);
         T* M = (T*)b.M.p;
         elim_init_kernel<T, L><<<(unsigned)((n * n + 255) / 256), 256, 0, s>>>(A, lda, n, M, md);
         std::vector<int64_t> pr;
         std::vector<T> pv;
-        if ((ce = cudaGetLastError()) || (ce = elim_local<T, L>(ctx, b, M, n, md, &pr, &pv, s)))
-            return elim_fail(ctx, "smith_local", ce);
+        if ((ce = cudaGetLastError())) return elim_fail(ctx, "smith_local", ce);
+        bool done = false;
+        if constexpr (sizeof(T) == 4) {
+            if (n >= ctx->elim_panel_min_n) {  // by panels, and the block left at once when it is small
+                Blocked r;
+                StreamBuf ob;
+                constexpr int words = L * kSmallLevels + 1;
+                int h[words];
+                const size_t sm = sizeof(uint32_t) * kSmallBlock * kSmallBlock;
+                SmallLevels lv{};
+                for (int l = 0; l < nq; l++) {
+                    lv.m[l] = md.m[l];
+                    lv.q[l] = md.q[l];
+                    lv.e[l] = e[l];
+                }
+                if ((ce = elim_blocked<L, true>(ctx, M, n, md, &r, s)) || (ce = ob.alloc(ctx, sizeof(h), s)) ||
+                    (ce = cudaMemsetAsync(ob.p, 0, sizeof(h), s)) ||
+                    (ce = cudaFuncSetAttribute(local_small_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)))
+                    return elim_fail(ctx, "smith_local", ce);
+                local_small_kernel<L><<<(unsigned)nq, kSmallThreads, sm, s>>>(M, n, r.live, r.count, r.dcols, lv, (int*)ob.p);
+                if ((ce = cudaGetLastError()) || (ce = cudaMemcpyAsync(h, ob.p, sizeof(h), cudaMemcpyDeviceToHost, s)) ||
+                    (ce = cudaStreamSynchronize(s)))
+                    return elim_fail(ctx, "smith_local", ce);
+                if (h[words - 1] <= kSmallBlock) {
+                    for (int l = 0; l < nq; l++)
+                        for (int t = 0; t < e[l]; t++) (*counts)[l][t + 1] += h[l * kSmallLevels + t];
+                    return SMF_OK;
+                }
+                if ((ce = read_blocked<L>(r, n, &pr, nullptr, nullptr, s))) return elim_fail(ctx, "smith_local", ce);
+                done = true;
+            }
+        }
+        if (!done && (ce = elim_local<T, L>(ctx, b, M, n, md, &pr, &pv, s))) return elim_fail(ctx, "smith_local", ce);
         std::vector<char> row_used(n, 0);
         for (int64_t k = 0; k < n; k++)
             if (pr[k] >= 0) row_used[pr[k]] = 1;
@@ -1020,15 +1005,15 @@ int local_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const ui
         // keep the joint matrix, free the rest of the scratch
         std::swap(joint.p, b.M.p);
         joint.s = s;
-        if ((ce = idx.alloc(sizeof(int64_t) * 2 * nb, s)) ||
+        if ((ce = idx.alloc(ctx, sizeof(int64_t) * 2 * nb, s)) ||
             (ce = cudaMemcpyAsync(idx.p, id.data(), sizeof(int64_t) * 2 * nb, cudaMemcpyHostToDevice, s)))
             return elim_fail(ctx, "smith_local", ce);
     }
     // each prime on the block that is left (the joint pivots are units for all of them)
     ElimBufs<T, 1> b1;
     StreamBuf M2;
-    cudaError_t ce = b1.alloc(nb, s);
-    if (!ce) ce = M2.alloc(sizeof(T) * (size_t)nb * nb, s);
+    cudaError_t ce = b1.alloc(ctx, nb, s);
+    if (!ce) ce = M2.alloc(ctx, sizeof(T) * (size_t)nb * nb, s);
     if (ce) return elim_fail(ctx, "smith_local: device allocation", ce);
     for (int l = 0; l < nq; l++) {
         elim_gather_kernel<T, L><<<(unsigned)((nb * nb + 255) / 256), 256, 0, s>>>(

@@ -193,7 +193,7 @@ int smf::lif_run(smf_ctx* ctx, const smf_bigmat* A, const LifOptions& o, LifResu
     const int64_t nb = (int64_t)std::ceil(hn) + clog2(n) + kWeightBits + 1;
     // scratch in stream order on s (no device-wide synchronisation when freed)
     StreamBuf Ad, Cd, inv_ws, Rd, Wd, Xd, cd, lift_ws, Qd, pd;
-    if (Ad.alloc(8 * (size_t)n * n, s) != cudaSuccess || Cd.alloc(4 * (size_t)n * n, s) != cudaSuccess) {
+    if (Ad.alloc(ctx, 8 * (size_t)n * n, s) != cudaSuccess || Cd.alloc(ctx, 4 * (size_t)n * n, s) != cudaSuccess) {
         cudaGetLastError();
         return fail_with(ctx, SMF_E_NOMEM, "largest_invariant_factor: device allocation failed");
     }
@@ -202,7 +202,7 @@ int smf::lif_run(smf_ctx* ctx, const smf_bigmat* A, const LifOptions& o, LifResu
     smf_bigmat Am{n, n, n, 1, abits, Ad.p, 1, 0};
     size_t inv_bytes = 0;
     smf_inverse_mod_p_workspace(ctx, n, &inv_bytes);
-    if (inv_ws.alloc(inv_bytes, s) != cudaSuccess) {
+    if (inv_ws.alloc(ctx, inv_bytes, s) != cudaSuccess) {
         cudaGetLastError();
         return fail_with(ctx, SMF_E_NOMEM, "largest_invariant_factor: device allocation failed");
     }
@@ -247,10 +247,10 @@ int smf::lif_run(smf_ctx* ctx, const smf_bigmat* A, const LifOptions& o, LifResu
     std::vector<uint32_t> Qh((size_t)n * cp);  // [i][a]: the functionals of the pairing
     for (auto& w : Qh) w = 1 + (uint32_t)rng.below((1u << kWeightBits) - 1);
     const int64_t chunk = std::min<int64_t>(kChunk, k);
-    if (Rd.alloc(8 * (size_t)n * m, s) != cudaSuccess || Wd.alloc(4 * (size_t)n * m, s) != cudaSuccess ||
-        Xd.alloc(4 * (size_t)chunk * n * m, s) != cudaSuccess || cd.alloc(8 * (size_t)chunk * m, s) != cudaSuccess ||
-        (cp && (Qd.alloc(4 * (size_t)n * cp, s) != cudaSuccess ||
-                pd.alloc(8 * (size_t)chunk * cp * cq, s) != cudaSuccess))) {
+    if (Rd.alloc(ctx, 8 * (size_t)n * m, s) != cudaSuccess || Wd.alloc(ctx, 4 * (size_t)n * m, s) != cudaSuccess ||
+        Xd.alloc(ctx, 4 * (size_t)chunk * n * m, s) != cudaSuccess || cd.alloc(ctx, 8 * (size_t)chunk * m, s) != cudaSuccess ||
+        (cp && (Qd.alloc(ctx, 4 * (size_t)n * cp, s) != cudaSuccess ||
+                pd.alloc(ctx, 8 * (size_t)chunk * cp * cq, s) != cudaSuccess))) {
         cudaGetLastError();
         return fail_with(ctx, SMF_E_NOMEM, "largest_invariant_factor: device allocation failed");
     }
@@ -264,7 +264,7 @@ int smf::lif_run(smf_ctx* ctx, const smf_bigmat* A, const LifOptions& o, LifResu
     smf_bigmat Rm{n, m, m, 1, rbits, Rd.p, 1, 0};
     size_t lift_bytes = 0;
     if ((st = smf_padic_lift_workspace(ctx, pb, &Am, &Rm, &lift_bytes))) return st;
-    if (lift_bytes && lift_ws.alloc(lift_bytes, s) != cudaSuccess) {
+    if (lift_bytes && lift_ws.alloc(ctx, lift_bytes, s) != cudaSuccess) {
         cudaGetLastError();
         return fail_with(ctx, SMF_E_NOMEM, "largest_invariant_factor: device allocation failed");
     }

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kElimThreads)
 
 int64_t inv_panel_width(int64_t n) { return n <= kInvSingle ? n : panel_width(n, 1, 128); }
 
-size_t inv_scratch_bytes() { return sizeof(uint32_t) * kSub * kInvSingle; }
+size_t inv_scratch_bytes() { return sizeof(uint32_t) * panel_scratch(kInvSingle); }
 
 cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t p, int* rowcol, int* piv, int32_t* S,
                              void* scratch, int* flag, int* status, cudaStream_t s) {
@@ -205,7 +205,7 @@ cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t
     a.rowcol = rowcol;
     a.S = S;
     a.status = status;
-    return launch_panel_red<1, PanelRed::kNarrow, PanelKind::kInverse>(a, n, s);  // (p odd, at most 26 bits)
+    return launch_panel_red<1, PanelRed::kOddNarrow, PanelKind::kInverse>(a, n, s);  // (p odd, at most 26 bits)
 }
 
 cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t c0, int w, const int* piv, int32_t* Mp,

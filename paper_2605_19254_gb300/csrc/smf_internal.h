@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
@@ -74,9 +75,15 @@ struct smf_prof_rec {
     cudaEvent_t start, stop;
 };
 
-// default thresholds of the eliminations by panels (smf_set_elim_panels)
-constexpr int64_t kElimPanelMinN = 2560;       // determinants
-constexpr int64_t kElimLocalPanelMinN = 1536;  // local Smith forms
+// default threshold of the eliminations by panels (smf_set_elim_panels): every
+// size.  Four 31-bit determinants, by panels / one launch per column: n = 16
+// 0.10 / 0.30 ms, 128 0.32 / 1.7, 1009 2.7 / 14.4, 2003 8.1 / 44; three local
+// forms of a planted matrix: n = 32 0.13 / 1.2 ms, 1009 2.5 / 12.9.
+constexpr int64_t kElimPanelMinN = 1;
+
+// unused bytes a context's memory pool may keep: the eliminations' scratch up to
+// n = 4000 with four moduli
+constexpr uint64_t kPoolKeep = 256ull << 20;
 
 struct smf_ctx {
     int device;
@@ -107,15 +114,19 @@ struct smf_ctx {
     // epilogue run as one fused kernel (smf_set_fused_crt)
     int fused_crt = 0;
     // eliminations over Z/(m) of matrices with at least this many columns run
-    // by panels of 16 columns (smf_set_elim_panels): determinants, and local
-    // Smith forms, whose column loop keeps every column live and so gains from
-    // panels at smaller sizes (measured: n = 1009 9 % slower by panels, n = 2003
-    // 9 % faster)
+    // by panels when the moduli fit 31 bits (smf_set_elim_panels)
     int64_t elim_panel_min_n = kElimPanelMinN;
-    int64_t elim_local_panel_min_n = kElimLocalPanelMinN;
     // grouped-product plans: the autotuner's measured choice per product class
     // (key: basis size, A's digit count and the log2 sizes; value: 1 = three digits)
     std::vector<std::pair<uint64_t, int>> tune_cache;
+    // stream-ordered scratch of the Smith-form driver and the eliminations.  The
+    // pool keeps up to kPoolKeep bytes that are not in use (the device's default
+    // pool gives everything back at each synchronisation, and the next call maps
+    // it again: 0.2 ms of a 16 x 16 determinant's 0.28 ms); they go back when the
+    // context is destroyed
+    cudaMemPool_t pool = nullptr;  // made on first use
+    std::once_flag pool_once;
+    uint64_t pool_keep = kPoolKeep;
     // pinned host staging of the Smith-form driver's digit sums, kept across calls
     // (allocating and freeing pinned memory per call would synchronise the device)
     void* pinned[2] = {nullptr, nullptr};
@@ -183,19 +194,33 @@ struct ProfScope {
     }
 };
 
-// Stream-ordered device scratch (cudaMallocAsync / cudaFreeAsync on the stream
-// the work runs on): no device-wide synchronisation when it is freed, so calls
-// on different streams keep overlapping.
+// Stream-ordered device scratch from the context's own memory pool (freed on the
+// stream the work runs on): no device-wide synchronisation when it is freed, so
+// calls on different streams keep overlapping.
 struct StreamBuf {
     void* p = nullptr;
     cudaStream_t s = nullptr;
     StreamBuf() = default;
     StreamBuf(const StreamBuf&) = delete;
     StreamBuf& operator=(const StreamBuf&) = delete;
-    cudaError_t alloc(size_t bytes, cudaStream_t st) {
+    cudaError_t alloc(smf_ctx* ctx, size_t bytes, cudaStream_t st) {
         release();
         s = st;
-        return cudaMallocAsync(&p, bytes ? bytes : 1, st);
+        std::call_once(ctx->pool_once, [ctx] {
+            cudaMemPoolProps pp{};
+            pp.allocType = cudaMemAllocationTypePinned;
+            pp.location.type = cudaMemLocationTypeDevice;
+            pp.location.id = ctx->device;
+            if (cudaMemPoolCreate(&ctx->pool, &pp) != cudaSuccess) {
+                cudaGetLastError();
+                ctx->pool = nullptr;
+            } else {
+                uint64_t keep = ctx->pool_keep;
+                cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            }
+        });
+        if (!ctx->pool) return cudaErrorMemoryAllocation;
+        return cudaMallocFromPoolAsync(&p, bytes ? bytes : 1, ctx->pool, st);
     }
     void release() {
         if (p) cudaFreeAsync(p, s);

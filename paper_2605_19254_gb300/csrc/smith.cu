@@ -155,14 +155,14 @@ struct DeviceA {
     StreamBuf copy;
     const int64_t* p = nullptr;
     int64_t ld = 0;
-    bool load(const smf_bigmat* A, cudaStream_t s) {
+    bool load(smf_ctx* ctx, const smf_bigmat* A, cudaStream_t s) {
         const int64_t n = A->rows;
         if (A->on_device || n == 0) {
             p = (const int64_t*)A->data;
             ld = A->ld;
             return true;
         }
-        if (copy.alloc(8 * (size_t)n * n, s) != cudaSuccess ||
+        if (copy.alloc(ctx, 8 * (size_t)n * n, s) != cudaSuccess ||
             cudaMemcpy2DAsync(copy.p, 8 * n, A->data, 8 * A->ld, 8 * n, n, cudaMemcpyHostToDevice, s) != cudaSuccess) {
             cudaGetLastError();
             return false;
@@ -190,7 +190,7 @@ extern "C" int smf_det_mod(smf_ctx* ctx, const smf_bigmat* A, const uint64_t* q,
     cudaGetDevice(&dev0);
     cudaSetDevice(ctx->device);
     DeviceA Ad;
-    int st = Ad.load(A, (cudaStream_t)stream) ? det_mod_device(ctx, Ad.p, Ad.ld, A->rows, q, count, det, (cudaStream_t)stream)
+    int st = Ad.load(ctx, A, (cudaStream_t)stream) ? det_mod_device(ctx, Ad.p, Ad.ld, A->rows, q, count, det, (cudaStream_t)stream)
                         : fail_smith(ctx, SMF_E_NOMEM, "det_mod: copy of A failed");
     cudaSetDevice(dev0);
     return st;
@@ -212,7 +212,7 @@ extern "C" int smf_smith_local(smf_ctx* ctx, const smf_bigmat* A, const uint64_t
     DeviceA Ad;
     std::vector<std::vector<int64_t>> cnt;
     std::vector<int> ev(e, e + count);
-    int st = Ad.load(A, (cudaStream_t)stream) ? local_smith_device(ctx, Ad.p, Ad.ld, A->rows, q, ev.data(), count, &cnt, (cudaStream_t)stream)
+    int st = Ad.load(ctx, A, (cudaStream_t)stream) ? local_smith_device(ctx, Ad.p, Ad.ld, A->rows, q, ev.data(), count, &cnt, (cudaStream_t)stream)
                         : fail_smith(ctx, SMF_E_NOMEM, "smith_local: copy of A failed");
     cudaSetDevice(dev0);
     if (st == SMF_OK) {
@@ -242,7 +242,7 @@ extern "C" int smf_smith_form(smf_ctx* ctx, const smf_bigmat* A, uint64_t seed, 
     const int64_t n = A->rows;
     // A contiguous on the device (the eliminations), in stream order on s
     StreamBuf Ad;
-    if (Ad.alloc(8 * (size_t)n * n, s) != cudaSuccess) {
+    if (Ad.alloc(ctx, 8 * (size_t)n * n, s) != cudaSuccess) {
         cudaGetLastError();
         return fail_smith(ctx, SMF_E_NOMEM, "smith_form: device allocation failed");
     }

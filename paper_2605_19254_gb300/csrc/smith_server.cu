@@ -150,6 +150,7 @@ int smf_smith_server_create(int device, smf_form form, size_t budget_bytes, int 
     for (int w = 0; w < workers; w++) {
         smf_ctx* c = nullptr;
         int rc = smf_create(&c, device, form, 0);
+        if (rc == SMF_OK && budget_bytes) c->pool_keep = 64ull << 20;  // no more than the constant part of a footprint
         cudaStream_t st = nullptr;
         if (rc == SMF_OK && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
             cudaGetLastError();

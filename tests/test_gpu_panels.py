@@ -43,3 +43,38 @@ def test_inverse_by_panels(ctx, n, p_max):
         prod = ((f @ hi.astype(np.float64)).astype(np.int64) % p * 4096 + (f @ lo.astype(np.float64)).astype(np.int64)) % p
         assert np.array_equal(prod, np.eye(n, dtype=np.int64))
     pb.destroy()
+
+
+# determinants and local forms by panels of 32 columns at every size: one to
+# four lanes, all moduli odd and small, odd up to 31 bits, and with a power of two
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 64, 65, 130, 513])
+@pytest.mark.parametrize("q", [(2,), (101, 2), (65537, 3, 268435399), (2147483647, 2, 2147483629, 5)])
+def test_det_by_panels(ctx, orc, n, q):
+    A = inputs.uniform_int(n, "A", (n, n), -(1 << 20), 1 << 20)
+    ctx.set_elim_panels(1)
+    try:
+        got = ctx.det_mod(torch.from_numpy(A[..., None].copy()).cuda(), list(q), a_bits=20)
+    finally:
+        ctx.set_elim_panels(0)
+    assert got == [orc.det_mod(A, v) for v in q]
+
+
+@pytest.mark.parametrize("n", [12, 31, 33, 64, 65, 200, 520])
+@pytest.mark.parametrize("qe", [((2, 9), (3, 6), (5, 4)), ((2, 30),), ((3, 19), (46337, 2)), ((3, 3), (5, 2)),
+                                ((7, 2), (2, 1), (3, 2), (11, 1), (13, 3))])
+def test_local_by_panels(ctx, n, qe):
+    # s: a chain of products of the primes, below 2^34 so that the entries fit 64 bits
+    primes = [q for q, _ in qe]
+    s, cur = [], 1
+    for k in range(min(n, 9)):
+        q = primes[k % len(primes)]
+        cur *= q if cur * q < 1 << 34 else 1
+        s.append(cur)
+    s = [1] * (n - len(s)) + s
+    A = inputs.smith_known_matrix_np(n, s, n)
+    ctx.set_elim_panels(1)
+    try:
+        got = ctx.smith_local(torch.from_numpy(A[..., None].copy()).cuda(), primes, [e for _, e in qe], a_bits=62)
+    finally:
+        ctx.set_elim_panels(0)
+    assert got == [[sum(v % q ** t == 0 for v in s) for t in range(e + 1)] for q, e in qe]
