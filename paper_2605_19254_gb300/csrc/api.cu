@@ -215,38 +215,7 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
         ginv[i] = inv_mod(w, p[i]);
         ginvs[i] = shoup(ginv[i], p[i]);
     }
-    // device blob
     const int ml = (int)M.size();
-    size_t off = 0;
-    auto slot = [&](size_t bytes) {
-        size_t o = off;
-        off = align256(off + bytes);
-        return o;
-    };
-    const size_t o_p = slot(4 * L), o_mu = slot(8 * L), o_pow = slot(4 * L), o_inv = slot(8 * L);
-    const size_t o_gw = slot(4 * (size_t)L * L), o_gws = slot(4 * (size_t)L * L), o_ginv = slot(4 * L),
-                 o_ginvs = slot(4 * L), o_m = slot(4 * ml);
-    std::vector<uint8_t> host(off, 0);
-    memcpy(&host[o_p], p.data(), 4 * L);
-    memcpy(&host[o_mu], mu.data(), 8 * L);
-    memcpy(&host[o_pow], pow32.data(), 4 * L);
-    memcpy(&host[o_inv], inv_p.data(), 8 * L);
-    memcpy(&host[o_gw], gw.data(), 4 * (size_t)L * L);
-    memcpy(&host[o_gws], gws.data(), 4 * (size_t)L * L);
-    memcpy(&host[o_ginv], ginv.data(), 4 * L);
-    memcpy(&host[o_ginvs], ginvs.data(), 4 * L);
-    memcpy(&host[o_m], M.data(), 4 * ml);
-    DeviceGuard g(ctx->device);
-    cudaError_t e = cudaMalloc(&b->dev_blob, off);
-    // A copy from pageable memory may return before its DMA lands, and kernels on
-    // non-blocking streams are not ordered after the legacy stream: wait for it.
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->dev_blob, host.data(), off, cudaMemcpyHostToDevice, cudaStreamLegacy);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
-    if (e != cudaSuccess) {
-        if (b->dev_blob) cudaFree(b->dev_blob);
-        delete b;
-        return fail(ctx, SMF_E_CUDA, std::string("basis tables: ") + cudaGetErrorString(e));
-    }
     b->gw = gw;
     b->gws = gws;
     b->ginv = ginv;
@@ -288,12 +257,58 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
     b->crt.ginv = b->ginv.data();
     b->crt.ginvs = b->ginvs.data();
     b->crt.m = b->m_limbs.data();
+    // device blob
+    size_t off = 0;
+    auto slot = [&](size_t bytes) {
+        size_t o = off;
+        off = align256(off + bytes);
+        return o;
+    };
+    const size_t o_p = slot(4 * L), o_mu = slot(8 * L), o_pow = slot(4 * L), o_inv = slot(8 * L);
+    const size_t o_gw = slot(4 * (size_t)L * L), o_gws = slot(4 * (size_t)L * L), o_ginv = slot(4 * L),
+                 o_ginvs = slot(4 * L), o_m = slot(4 * ml), o_mi = slot(4 * (size_t)L * ml);
+    size_t pc = 0;
+    const size_t image = crt_image_bytes(b->crt, &pc), o_image = slot(image);
+    size_t o_red[4];
+    for (int k = 0; k < 4; k++) o_red[k] = slot(reduce_image_bytes(L, p[0], 1 << k));
+    std::vector<uint8_t> host(off, 0);
+    memcpy(&host[o_p], p.data(), 4 * L);
+    memcpy(&host[o_mu], mu.data(), 8 * L);
+    memcpy(&host[o_pow], pow32.data(), 4 * L);
+    memcpy(&host[o_inv], inv_p.data(), 8 * L);
+    memcpy(&host[o_gw], gw.data(), 4 * (size_t)L * L);
+    memcpy(&host[o_gws], gws.data(), 4 * (size_t)L * L);
+    memcpy(&host[o_ginv], ginv.data(), 4 * L);
+    memcpy(&host[o_ginvs], ginvs.data(), 4 * L);
+    memcpy(&host[o_m], M.data(), 4 * ml);
+    memcpy(&host[o_mi], b->mi.data(), 4 * (size_t)L * ml);
+    if (image) crt_image_make(b->crt, &host[o_image]);
+    for (int k = 0; k < 4; k++)
+        if (reduce_image_bytes(L, p[0], 1 << k)) reduce_image_make(p.data(), L, 1 << k, &host[o_red[k]]);
+    DeviceGuard g(ctx->device);
+    cudaError_t e = cudaMalloc(&b->dev_blob, off);
+    // A copy from pageable memory may return before its DMA lands, and kernels on
+    // non-blocking streams are not ordered after the legacy stream: wait for it.
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->dev_blob, host.data(), off, cudaMemcpyHostToDevice, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) {
+        if (b->dev_blob) cudaFree(b->dev_blob);
+        delete b;
+        return fail(ctx, SMF_E_CUDA, std::string("basis tables: ") + cudaGetErrorString(e));
+    }
     uint8_t* d = (uint8_t*)b->dev_blob;
     b->dev.L = L;
     b->dev.m_limbs = ml;
     b->dev.p = (const uint32_t*)(d + o_p);
     b->dev.mu = (const uint64_t*)(d + o_mu);
     b->dev.pow32 = (const uint32_t*)(d + o_pow);
+    for (int k = 0; k < 4; k++) b->dev.red[k] = d + o_red[k];
+    b->dev.p_top = p[0];
+    b->crt.d_mi = (const uint32_t*)(d + o_mi);
+    b->crt.d_m = (const uint32_t*)(d + o_m);
+    b->crt.d_image = d + o_image;
+    b->crt.d_pc = d + o_image + pc;
+    b->dev.sms = ctx->num_sms;
     b->dev.inv_p = (const double*)(d + o_inv);
     b->dev.gw = (const uint32_t*)(d + o_gw);
     b->dev.gws = (const uint32_t*)(d + o_gws);
@@ -581,7 +596,7 @@ int run_pipelined(smf_ctx* ctx, const MatmulPlan& P, smf_basis* basis, const smf
         }
         {
             ProfScope ps(ctx, 3, s);
-            SMF_CU(ctx, launch_crt(basis->crt, R, mc, N, X, ldX, C->words, s));
+            SMF_CU(ctx, launch_crt(basis->crt, R, mc, N, X, ldX, C->words, ctx->num_sms, s));
         }
         if (!C->on_device) {
             SMF_CU(ctx, cudaEventRecord(ev[kEvCReady + slot], s));
@@ -763,7 +778,7 @@ int smf_crt_reconstruct(smf_ctx* ctx, const smf_basis* b, const int32_t* residue
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     ProfScope ps(ctx, 3, s);
-    SMF_CU(ctx, launch_crt(b->crt, residues, X->rows, X->cols, (uint64_t*)X->data, X->ld, X->words, s));
+    SMF_CU(ctx, launch_crt(b->crt, residues, X->rows, X->cols, (uint64_t*)X->data, X->ld, X->words, ctx->num_sms, s));
     return SMF_OK;
 }
 
@@ -897,7 +912,7 @@ int smf_rns_matmul(smf_ctx* ctx, const smf_bigmat* A, const smf_bigmat* B, smf_b
     }
     if (!fused) {
         ProfScope ps(ctx, 3, s);
-        SMF_CU(ctx, launch_crt(basis->crt, R, M, N, dC, ldC, C->words, s));
+        SMF_CU(ctx, launch_crt(basis->crt, R, M, N, dC, ldC, C->words, ctx->num_sms, s));
     }
     if (!C->on_device) {
         ProfScope ps(ctx, 4, s);
@@ -1247,7 +1262,7 @@ int build_grouped(smf_ctx* ctx, const GroupPlan& G, int count, const smf_bigmat*
                             (int)entry_bits(&B[i])};
         if (it.a_shared) {
             ReduceItem& si = split[b.nsplit++];
-            si = ReduceItem{ra.X, ra.rows, ra.cols, ra.ld, adig, ra.ld_out, ra.W, ra.t, ra.bits, 0, b.usplit, 0u, 0};
+            si = ReduceItem{ra.X, ra.rows, ra.cols, ra.ld, adig, ra.ld_out, ra.W, ra.t, ra.bits, b.usplit, 0u, 0};
             b.usplit += split_units(it.M, it.K, &si.div_m, &si.div_s);
         } else {
             b.one_by_one.emplace_back(ra, ReduceOut::kDigits);
@@ -1255,7 +1270,7 @@ int build_grouped(smf_ctx* ctx, const GroupPlan& G, int count, const smf_bigmat*
         if (reduce_t_groupable(basis->dev, rb)) {
             const int cls = rb.W == 1 ? 0 : rb.W == 2 ? 1 : rb.W == 4 ? 2 : 3;
             bt_w[cls].push_back(
-                ReduceItem{rb.X, rb.rows, rb.cols, rb.ld, bdig, rb.ld_out, rb.W, rb.t, rb.bits, 0, 0, 0u, 0});
+                ReduceItem{rb.X, rb.rows, rb.cols, rb.ld, bdig, rb.ld_out, rb.W, rb.t, rb.bits, 0, 0u, 0});
         } else {
             b.one_by_one.emplace_back(rb, ReduceOut::kDigitsT);
         }
@@ -1272,7 +1287,7 @@ int build_grouped(smf_ctx* ctx, const GroupPlan& G, int count, const smf_bigmat*
         GroupBuild::BtClass k{1 << c, nbt, 0, 0};
         for (ReduceItem r : bt_w[c]) {
             r.base = k.units;
-            k.units += reduce_t_units(r.rows, r.cols, &r.rb);
+            k.units += reduce_t_units(r.rows, r.cols);
             bt[nbt++] = r;
             k.n++;
         }

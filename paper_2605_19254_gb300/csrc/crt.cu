@@ -3,7 +3,9 @@
 // thread, result in (-M/2, M/2] written as W two's complement words; and the
 // conversion between RNS bases.  The per-entry reconstruction (Lagrange form
 // with an fp32 quotient, exact mixed-radix fallback) is in crt_dev.h.
-#include "crt_dev.h"
+#include <vector>
+
+#include "rns_mma.h"
 
 namespace smf {
 namespace {
@@ -171,6 +173,403 @@ convert_kernel(const __grid_constant__ ConvConst<LMAX> v, const int32_t* __restr
 }
 
 
+// ---------------------------------------------------------------------------
+// CRT of bases of at most 48 primes below 2^24, on the tensor cores (rns_mma.h).
+// x = sum_i xi_i M_i - alpha M - H modulo 2^(8 N), where N bytes hold the signed
+// result; the columns of the product are the balanced base-256 digits of the
+// 2^(8u) M_i, lane 4g + t owns 2 NT consecutive ones (NT / 2 limbs), and the carry
+// into the next lane's limbs is passed by a shuffle.  The limbs go through shared
+// memory, so that the words are stored in order.
+// What bounds it is instruction issue; one limb-sum thread per entry took 1815
+// instructions with 23 primes.  The product of 1009 x 1009 by 1009 x 100 with 34
+// primes (reduction and CRT both so) went from 303 to 218 us, a batch of 512 products
+// from 8.02 to 7.15 ms, one of 64 x 64 by 64 x 16 from 39 to 26 us.
+template <int LMAX>
+struct CrtMma {
+    static constexpr int NT = (3 * LMAX / 4 + 3) / 4 * 2;  // n8 tiles
+    static constexpr int LPT = NT / 2, NL = 4 * LPT;       // limbs per lane, limbs
+    static constexpr int SE = NL + 1;                      // staged entry (odd: no bank conflicts)
+    static constexpr int KS = XiShape<LMAX>::KS;
+    // the tables, made with the basis and copied to shared memory by each block:
+    // fragments, pc, cn (per limb {128 (1 + 2^8 + 2^16) sum_i M_i - H, -M}: the digits
+    // of xi are less 128), 1 / p_i
+    static constexpr size_t kPc = sizeof(uint2) * NT * KS * 32, kCn = kPc + sizeof(uint4) * LMAX,
+                            kIp = kCn + sizeof(uint2) * NL, kImage = kIp + sizeof(float) * LMAX;
+    static constexpr size_t kSmem = kImage + sizeof(uint32_t) * (kMmaThreads * SE);
+    static_assert(kCn % 16 == 0 && kIp % 16 == 0 && kImage % 16 == 0, "copied 16 bytes at a time");
+};
+
+template <int LMAX>
+struct CrtSmem {
+    const uint2* wf;
+    const uint2* cn;
+    const uint4* pc;
+    const float* ip;
+    uint32_t* st;
+    __device__ CrtSmem(uint8_t* p, const uint8_t* image) {
+        using Q = CrtMma<LMAX>;
+        stage(p, image, Q::kImage);
+        wf = (const uint2*)p;
+        pc = (const uint4*)(p + Q::kPc);
+        cn = (const uint2*)(p + Q::kCn);
+        ip = (const float*)(p + Q::kIp);
+        st = (uint32_t*)(p + Q::kImage) + (threadIdx.x >> 5) * 32 * Q::SE;
+        __syncthreads();
+    }
+};
+
+// Entries e0 .. e0 + 31 (those below count) of one output, by one warp.
+template <int LMAX>
+__device__ __forceinline__ void crt_chunk(const XiExact& q, const CrtSmem<LMAX>& sm,
+                                          const int32_t* __restrict__ R, int64_t count, int64_t cols, int64_t e0,
+                                          uint64_t* __restrict__ X, int64_t ld, int W) {
+    using Q = CrtMma<LMAX>;
+    const int lane = threadIdx.x & 31, t = lane & 3;
+    const bool vec = (count & 3) == 0 && ((uintptr_t)R & 15) == 0;
+    uint32_t a[2][Q::KS][4], alpha[4];
+    xi_frags<LMAX>(q, sm.pc, sm.ip, R, count, e0, vec, a, alpha);
+    uint32_t x[Q::LPT][4];
+    int32_t carry[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int l = 0; l < Q::LPT; l++) {
+        float acc[2][2][4] = {};
+#pragma unroll
+        for (int ks = 0; ks < Q::KS; ks++) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const uint2 b = sm.wf[((2 * l + h) * Q::KS + ks) * 32 + lane];
+                mma_f16(acc[0][h], a[0][ks], b);
+                mma_f16(acc[1][h], a[1][ks], b);
+            }
+        }
+        const uint2 k = sm.cn[t * Q::LPT + l];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            uint32_t s[4];  // the four column sums, each 0x4B400000 too large
+#pragma unroll
+            for (int b = 0; b < 4; b++) s[b] = __float_as_uint(acc[e >> 1][b >> 1][2 * (e & 1) + (b & 1)] + kMagic);
+            const int32_t lo = (int32_t)(s[0] + (s[1] << 8) - kMagicBits * 257u);  // below 2^30 in absolute value
+            const int32_t hi = (int32_t)(s[2] + (s[3] << 8) - kMagicBits * 257u);
+            const int64_t v = (int64_t)((uint64_t)alpha[e] * k.y + k.x) + (int64_t)hi * 65536 + ((int64_t)lo + carry[e]);
+            x[l][e] = (uint32_t)v;
+            carry[e] = (int32_t)(v >> 32);
+        }
+    }
+    // the carries into the next lane's limbs; rarely more than one round (a carry
+    // that passes all of a lane's limbs)
+    for (;;) {
+        bool more = false;
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            int32_t c = __shfl_up_sync(0xffffffffu, carry[e], 1);
+            if (t == 0) c = 0;
+#pragma unroll
+            for (int l = 0; l < Q::LPT; l++) {
+                const int64_t v = (int64_t)x[l][e] + c;
+                x[l][e] = (uint32_t)v;
+                c = (int32_t)(v >> 32);
+            }
+            carry[e] = t == 3 ? 0 : c;
+            more |= carry[e] != 0;
+        }
+        if (!__any_sync(0xffffffffu, more)) break;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+#pragma unroll
+        for (int l = 0; l < Q::LPT; l++) sm.st[((lane >> 2) * 4 + e) * Q::SE + t * Q::LPT + l] = x[l][e];
+    __syncwarp();
+    const int left = (int)min((int64_t)32, count - e0);
+    const int de = 32 / W, dw = 32 % W;
+    int e = lane / W, w = lane % W;
+    while (e < left) {
+        const uint32_t* s = sm.st + e * Q::SE;
+        const uint32_t ext = (uint32_t)((int32_t)s[Q::NL - 1] >> 31);
+        const uint32_t lo = 2 * w < Q::NL ? s[2 * w] : ext, hi = 2 * w + 1 < Q::NL ? s[2 * w + 1] : ext;
+        int64_t at = e0 + e;
+        if (ld != cols) at = at / cols * ld + at % cols;
+        X[at * W + w] = (uint64_t)hi << 32 | lo;
+        e += de;
+        w += dw;
+        if (w >= W) {
+            w -= W;
+            e++;
+        }
+    }
+    __syncwarp();
+}
+
+template <int LMAX>
+__global__ void __launch_bounds__(kMmaThreads, LMAX <= 24 ? 4 : 1)
+crt_mma_kernel(const uint8_t* __restrict__ image, XiExact q, const int32_t* __restrict__ R, int64_t rows,
+               int64_t cols, uint64_t* __restrict__ X, int64_t ld, int W) {
+    extern __shared__ __align__(16) uint8_t dyn[];
+    const CrtSmem<LMAX> sm(dyn, image);
+    const int64_t count = rows * cols;
+    for (int64_t e0 = (int64_t)blockIdx.x * kMmaThreads + (threadIdx.x & ~31); e0 < count;
+         e0 += (int64_t)gridDim.x * kMmaThreads)
+        crt_chunk<LMAX>(q, sm, R, count, cols, e0, X, ld, W);
+}
+
+// Several outputs of one basis in one launch: unit u is the 128 consecutive
+// entries u - base_i of item i (found by bisection).
+template <int LMAX>
+__global__ void __launch_bounds__(kMmaThreads, LMAX <= 24 ? 4 : 1)
+crt_mma_grouped_kernel(const uint8_t* __restrict__ image, XiExact q, const CrtItem* __restrict__ items, int n,
+                       int64_t units) {
+    extern __shared__ __align__(16) uint8_t dyn[];
+    const CrtSmem<LMAX> sm(dyn, image);
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const CrtItem* it = find_item(items, n, u);
+        const int64_t count = it->rows * it->cols, e0 = (u - it->base) * kMmaThreads + (threadIdx.x & ~31);
+        if (e0 < count) crt_chunk<LMAX>(q, sm, it->R, count, it->cols, e0, it->X, it->ld, it->W);
+    }
+}
+
+// The image of the tables for a basis.  Lane 4n + t of tile nt owns result bytes
+// (n / 2) 2 NT + 2 nt and + 1, whose digit of 2^(8u) M_i is digit (byte - u) of M_i.
+template <int LMAX>
+void crt_image(const CrtHost& h, uint8_t* image) {
+    using Q = CrtMma<LMAX>;
+    constexpr int NL = Q::NL;
+    std::vector<uint32_t> bal((size_t)h.L * NL);  // M_i + 0x80..80: its bytes less 128 are the balanced digits of M_i
+    uint64_t sum[NL] = {};
+    for (int i = 0; i < h.L; i++) {
+        uint64_t c = 0;
+        for (int k = 0; k < NL; k++) {
+            const uint32_t mi = k < h.m_limbs ? h.mi[(size_t)i * h.m_limbs + k] : 0u;
+            sum[k] += mi;
+            c += (uint64_t)mi + 0x80808080u;
+            bal[(size_t)i * NL + k] = (uint32_t)c;
+            c >>= 32;
+        }
+    }
+    uint16_t* wf = (uint16_t*)image;
+    for (int nt = 0; nt < Q::NT; nt++)
+        for (int ks = 0; ks < Q::KS; ks++)
+            for (int lane = 0; lane < 32; lane++)
+                for (int kap = 0; kap < 4; kap++) {
+                    const int n = lane >> 2, byte = (n >> 1) * 2 * Q::NT + 2 * nt + (n & 1);
+                    int i, u, d = 0;
+                    if (xi_slot<LMAX>(ks, kap, lane & 3, &i, &u) && i < h.L && byte >= u)
+                        d = (int)(bal[(size_t)i * NL + ((byte - u) >> 2)] >> (8 * ((byte - u) & 3)) & 255u) - 128;
+                    *wf++ = half_bits(d);
+                }
+    uint4* pc = (uint4*)(image + Q::kPc);
+    float* ip = (float*)(image + Q::kIp);
+    for (int i = 0; i < LMAX; i++) {  // beyond L: xi = 0
+        pc[i] = i < h.L ? make_uint4(h.p[i], h.hmod[i], h.c[i], h.cs[i]) : make_uint4(1, 0, 0, 0);
+        ip[i] = i < h.L ? 1.0f / (float)h.p[i] : 0.f;
+    }
+    uint2* cn = (uint2*)(image + Q::kCn);
+    uint64_t c = 0, b = 0, g = 0;
+    for (int k = 0; k < NL; k++) {
+        c += sum[k] * (128u * 65793u);
+        b = (uint64_t)(uint32_t)c - (k < h.m_limbs ? h.h[k] : 0u) - b;
+        g = 0ull - (k < h.m_limbs ? h.m[k] : 0u) - g;
+        cn[k] = make_uint2((uint32_t)b, (uint32_t)g);
+        b >>= 63;
+        g >>= 63;
+        c >>= 32;
+    }
+}
+
+XiExact xi_exact(const CrtHost& h) { return {h.d_mi, h.d_m, h.L, h.m_limbs}; }
+
+// As many blocks as are resident at once (each makes the tables once).
+template <auto kernel>
+cudaError_t mma_grid(size_t smem, int num_sms, int64_t units, unsigned* grid) {
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e) return e;
+    }
+    // a property of the kernel's code, asked once (1 us a call)
+    static const int per = [smem] {
+        int n = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kMmaThreads, smem);
+        return n > 0 ? n : 1;
+    }();
+    const int64_t most = (int64_t)num_sms * per;
+    *grid = (unsigned)(units < most ? units : most);
+    return cudaSuccess;
+}
+
+template <int LMAX>
+cudaError_t launch_crt_mma(const CrtHost& h, const int32_t* R, int64_t rows, int64_t cols, uint64_t* X, int64_t ld,
+                           int W, int num_sms, cudaStream_t s) {
+    using Q = CrtMma<LMAX>;
+    unsigned grid;
+    const cudaError_t e = mma_grid<crt_mma_kernel<LMAX>>(Q::kSmem, num_sms, (rows * cols + kMmaThreads - 1) / kMmaThreads, &grid);
+    if (e) return e;
+    crt_mma_kernel<LMAX><<<grid, kMmaThreads, Q::kSmem, s>>>(h.d_image, xi_exact(h), R, rows, cols, X, ld, W);
+    return cudaGetLastError();
+}
+
+template <int LMAX>
+cudaError_t launch_crt_mma_grouped(const CrtHost& h, const CrtItem* items, int n, int64_t units, int num_sms,
+                                   cudaStream_t s) {
+    using Q = CrtMma<LMAX>;
+    unsigned grid;
+    const cudaError_t e = mma_grid<crt_mma_grouped_kernel<LMAX>>(Q::kSmem, num_sms, units, &grid);
+    if (e) return e;
+    crt_mma_grouped_kernel<LMAX><<<grid, kMmaThreads, Q::kSmem, s>>>(h.d_image, xi_exact(h), items, n, units);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Conversion to primes below 2^24, on the tensor cores (rns_mma.h): the columns of
+// the product are the balanced digits of w_ij 2^(8u) mod q_j, w_ij = M_i mod q_j.
+// Lane 4g + t owns target primes j = 4b + t, three columns each; three n8 tiles
+// hold two targets of a lane.  A residue is then
+//   v = S_0 + 2^8 S_1 + 2^16 S_2 + C_j - alpha (M mod q_j)  mod q_j:
+// the quotient in fp32 (|v / q_j| < 2^14, its error below 2^-7, so a floor taken
+// 2^-6 low leaves [0, 1.04 q_j)), the remainder in wrapping 32 bits.
+// 23 -> 23 primes, 1M entries: 159 -> 79 us (28 us of HBM traffic); bound by issue.
+template <int LMAX>
+struct ConvMma {
+    const uint4* pc;          // the source's constants (device)
+    XiExact xi;
+    uint32_t w[LMAX * LMAX];  // w_ij at j LMAX + i
+    uint4 ti[LMAX];           // q_j, M mod q_j, C_j with the biases of the sums and the quotient taken out
+    float4 tf[LMAX];          // 1 / q_j, (M mod q_j) / q_j, C_j / q_j - 1/2 - 2^-6
+    int LQ;
+};
+static_assert(sizeof(ConvMma<48>) <= 32000, "kernel parameter space");
+
+template <int LMAX>
+__global__ void __launch_bounds__(kMmaThreads)
+convert_mma_kernel(const __grid_constant__ ConvMma<LMAX> v, const int32_t* __restrict__ R, int32_t* __restrict__ out,
+                   int64_t count) {
+    constexpr int KS = XiShape<LMAX>::KS, NB = LMAX / 8;  // groups of eight targets
+    __shared__ uint2 wf[NB * 3 * KS * 32];
+    __shared__ uint4 pc[LMAX], ti[LMAX];
+    __shared__ float4 tf[LMAX];
+    __shared__ float ip[LMAX];
+    const int LQ = v.LQ, L = v.xi.L, lane = threadIdx.x & 31, t = lane & 3;
+    for (int i = threadIdx.x; i < LMAX; i += kMmaThreads) {
+        const uint4 c = i < L ? __ldg(v.pc + i) : make_uint4(1, 0, 0, 0);
+        pc[i] = c;
+        ip[i] = i < L ? 1.0f / (float)c.x : 0.f;
+    }
+    for (int j = threadIdx.x; j < LQ; j += kMmaThreads) {
+        ti[j] = v.ti[j];
+        tf[j] = v.tf[j];
+    }
+    for (int x = threadIdx.x; x < (LQ + 7) / 8 * 3 * KS * 32; x += kMmaThreads) wf[x] = make_uint2(0, 0);
+    __syncthreads();
+    // the three digits of w_ij 2^(8u) mod q_j to where the fragments have them (xi_slot)
+    for (int x = threadIdx.x; x < LQ * LMAX * 3; x += kMmaThreads) {
+        const int i = x % LMAX, u = x / LMAX % 3, j = x / (3 * LMAX);
+        if (i >= L) continue;
+        const int a = i >> 2, pr = u < 2 ? a : LMAX / 4 + a / 2, kap = 2 * (pr & 1) + (u < 2 ? u : a & 1);
+        // to within half of q_j and a little (the quotient is below 2^16)
+        const uint32_t w = v.w[j * LMAX + i], q = ti[j].x;
+        const int quo = __float2int_rn((float)w * ((float)(1 << 8 * u) * tf[j].x));
+        int32_t r = (int32_t)((w << 8 * u) - (uint32_t)quo * q);
+#pragma unroll
+        for (int dig = 0; dig < 3; dig++) {
+            const int c6 = (j >> 2 & 1) * 3 + dig, nt = (j >> 3) * 3 + c6 / 2, ln = (2 * (j & 3) + (c6 & 1)) * 4 + (i & 3);
+            ((__half*)wf)[((nt * KS + pr / 2) * 32 + ln) * 4 + kap] = __int2half_rn(dig < 2 ? ((r + 128) & 255) - 128 : r);
+            r = (r + 128) >> 8;
+        }
+    }
+    __syncthreads();
+    const bool vec = (count & 3) == 0 && ((uintptr_t)R & 15) == 0, vout = (count & 3) == 0 && ((uintptr_t)out & 15) == 0;
+    for (int64_t e0 = (int64_t)blockIdx.x * kMmaThreads + (threadIdx.x & ~31); e0 < count;
+         e0 += (int64_t)gridDim.x * kMmaThreads) {
+        uint32_t a[2][KS][4], alpha[4];
+        float al[4];
+        xi_frags<LMAX>(v.xi, pc, ip, R, count, e0, vec, a, alpha);
+#pragma unroll
+        for (int x = 0; x < 4; x++) al[x] = (float)alpha[x];
+        const int64_t e = e0 + (lane >> 2) * 4;
+#pragma unroll 1
+        for (int nb = 0; 8 * nb < LQ; nb++) {
+            float acc[2][3][4] = {};
+#pragma unroll
+            for (int ks = 0; ks < KS; ks++) {
+#pragma unroll
+                for (int h = 0; h < 3; h++) {
+                    const uint2 b = wf[((3 * nb + h) * KS + ks) * 32 + lane];
+                    mma_f16(acc[0][h], a[0][ks], b);
+                    mma_f16(acc[1][h], a[1][ks], b);
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < 2; b++) {
+                const int j = 8 * nb + 4 * b + t;
+                if (j >= LQ) continue;
+                const uint4 ci = ti[j];
+                const float4 cf = tf[j];
+                uint32_t r[4];
+#pragma unroll
+                for (int x = 0; x < 4; x++) {
+                    float s[3];
+#pragma unroll
+                    for (int k = 0; k < 3; k++) s[k] = acc[x >> 1][(3 * b + k) >> 1][2 * (x & 1) + ((3 * b + k) & 1)];
+                    float f = fmaf(fmaf(s[2], 65536.f, fmaf(s[1], 256.f, s[0])), cf.x, cf.z);
+                    f = fmaf(-al[x], cf.y, f);
+                    const uint32_t quo = __float_as_uint(f + kMagic);
+                    uint32_t y = __float_as_uint(s[0] + kMagic) + (__float_as_uint(s[1] + kMagic) << 8) +
+                                 (__float_as_uint(s[2] + kMagic) << 16) + ci.z;
+                    y -= alpha[x] * ci.y;
+                    y -= quo * ci.x;
+                    r[x] = min(y, y - ci.x);
+                }
+                int32_t* o = out + (size_t)j * count + e;
+                if (vout) {
+                    if (e < count) *(int4*)o = make_int4((int)r[0], (int)r[1], (int)r[2], (int)r[3]);
+                } else {
+#pragma unroll
+                    for (int x = 0; x < 4; x++)
+                        if (e + x < count) o[x] = (int32_t)r[x];
+                }
+            }
+        }
+    }
+}
+
+// a mod q of the integer with 32-bit limbs x[0 .. n) (q < 2^32)
+uint32_t limbs_mod(const uint32_t* x, int n, uint32_t q) {
+    uint64_t r = 0;
+    for (int k = n - 1; k >= 0; k--) r = ((r << 32) | x[k]) % q;
+    return (uint32_t)r;
+}
+
+template <int LMAX>
+cudaError_t launch_convert_mma(const CrtHost& h, const uint32_t* q, int LQ, const int32_t* R, int32_t* out,
+                               int64_t count, int num_sms, cudaStream_t s) {
+    ConvMma<LMAX> v{};
+    v.pc = (const uint4*)h.d_pc;
+    v.xi = xi_exact(h);
+    const int L = h.L;
+    for (int j = 0; j < LQ; j++) {
+        const uint32_t qj = q[j];
+        // M_i mod q_j by products of the primes before and after p_i
+        uint32_t* w = v.w + j * LMAX;
+        uint64_t before = 1 % qj, after = 1 % qj, sum = 0;
+        for (int i = 0; i < L; i++) {
+            w[i] = (uint32_t)before;
+            before = before * h.p[i] % qj;
+        }
+        for (int i = L - 1; i >= 0; i--) {
+            w[i] = (uint32_t)(w[i] * after % qj);
+            after = after * h.p[i] % qj;
+            sum += w[i];
+        }
+        const uint32_t m = (uint32_t)before, hm = limbs_mod(h.h, h.m_limbs, qj);
+        const uint32_t c = (uint32_t)((sum * (128u * 65793u) + qj - hm) % qj);  // (every digit of xi is less 128)
+        v.ti[j] = make_uint4(qj, m, c - kMagicBits * 65793u + qj * kMagicBits, 0);
+        v.tf[j] = make_float4(1.0f / (float)qj, (float)m / (float)qj, (float)c / (float)qj - 0.5f - 0x1p-6f, 0.f);
+    }
+    v.LQ = LQ;
+    unsigned grid;
+    const cudaError_t e = mma_grid<convert_mma_kernel<LMAX>>(0, num_sms, (count + kMmaThreads - 1) / kMmaThreads, &grid);
+    if (e) return e;
+    convert_mma_kernel<LMAX><<<grid, kMmaThreads, 0, s>>>(v, R, out, count);
+    return cudaGetLastError();
+}
+
 template <int LMAX, bool FAST, int PB>
 cudaError_t launch_crt_t(const CrtHost& h, const int32_t* R, int64_t rows, int64_t cols, uint64_t* X, int64_t ld,
                          int W, cudaStream_t s) {
@@ -189,13 +588,6 @@ cudaError_t launch_crt_grouped_t(const CrtHost& h, const CrtItem* items, int n, 
     crt_const(h, q);
     crt_grouped_kernel<LMAX, FAST, PB><<<(unsigned)units, 128, 0, s>>>(q, items, n);
     return cudaGetLastError();
-}
-
-// a mod q of the integer with 32-bit limbs x[0 .. n) (q < 2^32)
-uint32_t limbs_mod(const uint32_t* x, int n, uint32_t q) {
-    uint64_t r = 0;
-    for (int k = n - 1; k >= 0; k--) r = ((r << 32) | x[k]) % q;
-    return (uint32_t)r;
 }
 
 template <int LMAX>
@@ -238,16 +630,41 @@ cudaError_t launch_convert_t(const CrtHost& h, const uint32_t* q, int LQ, const 
     return cudaGetLastError();
 }
 
+// The tensor-core kernels take primes below 2^24 (the limb form's bases), whose
+// three digits keep the fp32 sums exact; wider primes keep the multiply-adds.
+bool narrow_basis(const CrtHost& h) { return h.L > 0 && h.L <= 48 && h.p[0] < (1u << 24); }
+
 }  // namespace
 
+size_t crt_image_bytes(const CrtHost& h, size_t* pc) {
+    if (!narrow_basis(h)) return 0;
+#define SMF_IMAGE(N) (*pc = CrtMma<N>::kPc, CrtMma<N>::kImage)
+    return h.L <= 8 ? SMF_IMAGE(8) : h.L <= 16 ? SMF_IMAGE(16) : h.L <= 24 ? SMF_IMAGE(24) : h.L <= 32 ? SMF_IMAGE(32) : SMF_IMAGE(48);
+#undef SMF_IMAGE
+}
+
+void crt_image_make(const CrtHost& h, uint8_t* image) {
+    if (h.L <= 8) crt_image<8>(h, image);
+    else if (h.L <= 16) crt_image<16>(h, image);
+    else if (h.L <= 24) crt_image<24>(h, image);
+    else if (h.L <= 32) crt_image<32>(h, image);
+    else crt_image<48>(h, image);
+}
+
 cudaError_t launch_crt(const CrtHost& h, const int32_t* R, int64_t rows, int64_t cols, uint64_t* X, int64_t ld,
-                       int W, cudaStream_t s) {
+                       int W, int num_sms, cudaStream_t s) {
     if (rows == 0 || cols == 0) return cudaSuccess;
-    const bool narrow = h.L > 0 && h.p[0] < (1u << 24);  // primes of at most 24 bits: fewer limbs of M
-    if (h.L <= 8) return narrow ? launch_crt_t<8, true, 24>(h, R, rows, cols, X, ld, W, s) : launch_crt_t<8, true, 26>(h, R, rows, cols, X, ld, W, s);
-    if (h.L <= 16) return narrow ? launch_crt_t<16, true, 24>(h, R, rows, cols, X, ld, W, s) : launch_crt_t<16, true, 26>(h, R, rows, cols, X, ld, W, s);
-    if (h.L <= 24) return narrow ? launch_crt_t<24, true, 24>(h, R, rows, cols, X, ld, W, s) : launch_crt_t<24, true, 26>(h, R, rows, cols, X, ld, W, s);
-    if (h.L <= 32) return narrow ? launch_crt_t<32, true, 24>(h, R, rows, cols, X, ld, W, s) : launch_crt_t<32, true, 26>(h, R, rows, cols, X, ld, W, s);
+    if (narrow_basis(h)) {
+        if (h.L <= 8) return launch_crt_mma<8>(h, R, rows, cols, X, ld, W, num_sms, s);
+        if (h.L <= 16) return launch_crt_mma<16>(h, R, rows, cols, X, ld, W, num_sms, s);
+        if (h.L <= 24) return launch_crt_mma<24>(h, R, rows, cols, X, ld, W, num_sms, s);
+        if (h.L <= 32) return launch_crt_mma<32>(h, R, rows, cols, X, ld, W, num_sms, s);
+        return launch_crt_mma<48>(h, R, rows, cols, X, ld, W, num_sms, s);
+    }
+    if (h.L <= 8) return launch_crt_t<8, true, 26>(h, R, rows, cols, X, ld, W, s);
+    if (h.L <= 16) return launch_crt_t<16, true, 26>(h, R, rows, cols, X, ld, W, s);
+    if (h.L <= 24) return launch_crt_t<24, true, 26>(h, R, rows, cols, X, ld, W, s);
+    if (h.L <= 32) return launch_crt_t<32, true, 26>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 48) return launch_crt_t<48, true, 26>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 64) return launch_crt_t<64, false, 26>(h, R, rows, cols, X, ld, W, s);
     return cudaErrorNotSupported;
@@ -255,15 +672,21 @@ cudaError_t launch_crt(const CrtHost& h, const int32_t* R, int64_t rows, int64_t
 
 int64_t crt_units(int64_t rows, int64_t cols) { return (rows * cols + 127) / 128; }
 
-cudaError_t launch_crt_grouped(const CrtHost& h, const CrtItem* items, int n, int64_t units, int /*num_sms*/,
+cudaError_t launch_crt_grouped(const CrtHost& h, const CrtItem* items, int n, int64_t units, int num_sms,
                                cudaStream_t s) {
     if (n == 0 || units == 0) return cudaSuccess;
     if (units > 0x7FFFFFFF) return cudaErrorInvalidValue;
-    const bool narrow = h.L > 0 && h.p[0] < (1u << 24);
-    if (h.L <= 8) return narrow ? launch_crt_grouped_t<8, true, 24>(h, items, n, units, s) : launch_crt_grouped_t<8, true, 26>(h, items, n, units, s);
-    if (h.L <= 16) return narrow ? launch_crt_grouped_t<16, true, 24>(h, items, n, units, s) : launch_crt_grouped_t<16, true, 26>(h, items, n, units, s);
-    if (h.L <= 24) return narrow ? launch_crt_grouped_t<24, true, 24>(h, items, n, units, s) : launch_crt_grouped_t<24, true, 26>(h, items, n, units, s);
-    if (h.L <= 32) return narrow ? launch_crt_grouped_t<32, true, 24>(h, items, n, units, s) : launch_crt_grouped_t<32, true, 26>(h, items, n, units, s);
+    if (narrow_basis(h)) {
+        if (h.L <= 8) return launch_crt_mma_grouped<8>(h, items, n, units, num_sms, s);
+        if (h.L <= 16) return launch_crt_mma_grouped<16>(h, items, n, units, num_sms, s);
+        if (h.L <= 24) return launch_crt_mma_grouped<24>(h, items, n, units, num_sms, s);
+        if (h.L <= 32) return launch_crt_mma_grouped<32>(h, items, n, units, num_sms, s);
+        return launch_crt_mma_grouped<48>(h, items, n, units, num_sms, s);
+    }
+    if (h.L <= 8) return launch_crt_grouped_t<8, true, 26>(h, items, n, units, s);
+    if (h.L <= 16) return launch_crt_grouped_t<16, true, 26>(h, items, n, units, s);
+    if (h.L <= 24) return launch_crt_grouped_t<24, true, 26>(h, items, n, units, s);
+    if (h.L <= 32) return launch_crt_grouped_t<32, true, 26>(h, items, n, units, s);
     if (h.L <= 48) return launch_crt_grouped_t<48, true, 26>(h, items, n, units, s);
     if (h.L <= 64) return launch_crt_grouped_t<64, false, 26>(h, items, n, units, s);
     return cudaErrorNotSupported;
@@ -273,6 +696,16 @@ cudaError_t launch_convert(const CrtHost& from, const uint32_t* q, int LQ, const
                            int64_t count, int num_sms, cudaStream_t s) {
     if (count == 0 || LQ == 0) return cudaSuccess;
     const int n = from.L > LQ ? from.L : LQ;
+    bool narrow = narrow_basis(from);
+    for (int j = 0; j < LQ; j++) narrow &= q[j] < (1u << 24);
+    if (narrow) {
+        if (n <= 8) return launch_convert_mma<8>(from, q, LQ, R, out, count, num_sms, s);
+        if (n <= 16) return launch_convert_mma<16>(from, q, LQ, R, out, count, num_sms, s);
+        if (n <= 24) return launch_convert_mma<24>(from, q, LQ, R, out, count, num_sms, s);
+        if (n <= 32) return launch_convert_mma<32>(from, q, LQ, R, out, count, num_sms, s);
+        if (n <= 48) return launch_convert_mma<48>(from, q, LQ, R, out, count, num_sms, s);
+        return cudaErrorNotSupported;
+    }
     if (n <= 8) return launch_convert_t<8>(from, q, LQ, R, out, count, num_sms, s);
     if (n <= 16) return launch_convert_t<16>(from, q, LQ, R, out, count, num_sms, s);
     if (n <= 24) return launch_convert_t<24>(from, q, LQ, R, out, count, num_sms, s);

@@ -11,7 +11,9 @@
 // launch's group are built once per block in shared memory.
 #include <cuda_bf16.h>
 
-#include "smf_internal.h"
+#include <vector>
+
+#include "rns_mma.h"
 
 namespace smf {
 namespace {
@@ -226,153 +228,290 @@ reduce_kernel(BasisDev b, ReduceArgs a, int group) {
     }
 }
 
-// rns_reduce of B straight into transposed, digit-major bf16 planes
-// [t][L][cols][ld_out] (digit u of prime i at plane u * L + i).  A block takes
-// 256 consecutive rows by NC columns; each thread reduces its row's NC
-// entries (W words each, held in registers) modulo the block's group of
-// primes, so the per-block table of 2^(32 j) mod p is amortised over NC
-// entries.  With 2W <= 16 the limb products of one prime sum below 2^62 and a
-// single Barrett reduction finishes each residue.
-//
-// Per prime: {p, 2^32 mod p, its Shoup companion, floor(2^32 / p)}, then
-// c_j = 2^(32 j) mod p for j <= 2W, padded to 16-byte rows.
-template <int W>
-struct RtTable {
-    static constexpr int NW = 4 + ((2 * W + 1 + 3) & ~3);
+// ---------------------------------------------------------------------------
+// The reductions modulo at most 64 primes below 2^24 of entries of 1, 2, 4 or 8
+// words, on the tensor cores (rns_mma.h has the layout).  x mod p_i is a product
+// of the entry's 8 W bytes with the constants 2^(8b) mod p_i: bytes less 128 (the
+// top one signed as it is) and balanced digits of the constants, fp32 sums below
+// 2^20, exact.  Lane 4g + t takes a quarter of the bytes of entries 4g .. 4g+3,
+// which follow one another along the output's contiguous dimension, so that its
+// results are stored 8 or 16 bytes at a time: the limb sums stored two bytes at a
+// time, 69 stores an entry with 23 primes.  The bound is instruction issue: about
+// 650 thread instructions per entry with 23 primes (2670 as limb sums).
+struct RmArgs {
+    const uint64_t* X;
+    int64_t minor_n, major_n;  // entries along the output's contiguous dimension, and across it
+    int64_t smin, smaj;        // their strides in X, in entries
+    void* out;                 // element (i, u, major, minor) at i si + u su + major ldo + minor
+    int64_t ldo, si, su;
+    int t;                     // digits per residue
+    int bits;
+    int* status;
 };
 
 template <int W>
-__device__ __forceinline__ void reduce_t_table(const BasisDev& b, uint32_t* ctab, int i0, int G) {
-    constexpr int NW = RtTable<W>::NW;
-    for (int e = threadIdx.x; e < G; e += blockDim.x) {
-        const uint32_t p = b.p[i0 + e];
-        const uint64_t mu = b.mu[i0 + e];
-        const uint32_t r32 = b.pow32[i0 + e];
-        uint32_t* row = ctab + e * NW;
-        row[0] = p;
-        row[1] = r32;
-        row[2] = (uint32_t)(((uint64_t)r32 << 32) / p);
-        row[3] = (uint32_t)((1ull << 32) / p);
-        uint32_t c = 1 % p;
-        for (int j = 0; j < NW - 4; j++) {
-            row[4 + j] = j <= 2 * W ? c : 0u;
-            c = barrett64((uint64_t)c * r32, p, mu);
-        }
-    }
-}
+struct RmShape {
+    static constexpr int KS = W == 1 ? 1 : W / 2;  // K steps of 16 bytes: a limb per lane and step
+};
 
-// One thread of the transposed reduce: row r, columns [cb, cb + NC), primes
-// i0 .. i0 + G - 1 (their table in ctab).
-template <int W, int NC>
-__device__ __forceinline__ void reduce_t_thread(const BasisDev& b, const uint32_t* ctab, int i0, int G,
-                                                const uint64_t* __restrict__ X, int64_t rows, int64_t cols,
-                                                int64_t ld, uint16_t* __restrict__ out, int64_t ld_out, int t,
-                                                int64_t r, int64_t cb, int bits, int* status) {
-    constexpr int NW = RtTable<W>::NW;
-    if (r >= rows) return;
-    const int64_t plane = cols * ld_out;
-    const int64_t dstride = plane * b.L;  // between digit planes of one prime
-    for (int cc = 0; cc < NC; cc++) {
-        const int64_t c = cb + cc;
-        if (c >= cols) break;
-        const uint64_t* x = X + (size_t)(r * ld + c) * W;
-        uint32_t v[2 * W];
-#pragma unroll
-        for (int j = 0; j < W; j += 2) {
-            if (j + 1 < W) {
-                const ulonglong2 q = __ldg((const ulonglong2*)(x + j));
-                v[2 * j] = (uint32_t)q.x;
-                v[2 * j + 1] = (uint32_t)(q.x >> 32);
-                v[2 * j + 2] = (uint32_t)q.y;
-                v[2 * j + 3] = (uint32_t)(q.y >> 32);
-            } else {
-                const uint64_t q = __ldg(x + j);
-                v[2 * j] = (uint32_t)q;
-                v[2 * j + 1] = (uint32_t)(q >> 32);
-            }
-        }
-        const bool neg = (v[2 * W - 1] >> 31) != 0;
-        if (status && i0 == 0 && over_bits<W>(v, W, bits)) flag_bound(status);
-        uint16_t* o = out + (size_t)i0 * plane + c * ld_out + r;
-        for (int e = 0; e < G; e++, o += plane) {
-            const uint32_t* ct = ctab + e * NW;
-            const uint4 hd = *(const uint4*)ct;
-            const uint32_t p = hd.x;
-            // sum_j v_j c_j < 16 * 2^56 < 2^62 (2W <= 16), as hi 2^32 + lo
-            uint32_t lo = 0, hi = 0;
-#pragma unroll
-            for (int j4 = 0; j4 < 2 * W; j4 += 4) {
-                const uint4 c4 = *(const uint4*)(ct + 4 + j4);
-                const uint32_t cj[4] = {c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-                for (int q = 0; q < 4; q++)
-                    if (j4 + q < 2 * W) mac64(lo, hi, v[j4 + q], cj[q]);
-            }
-            // hi (2^32 mod p) by Shoup, lo by its reciprocal quotient
-            const uint32_t t1 = hi * hd.y - __umulhi(hi, hd.z) * p;  // [0, 2p)
-            const uint32_t t2 = lo - __umulhi(lo, hd.w) * p;         // [0, 2p)
-            uint32_t rr = t1 + t2;                                   // [0, 4p)
-            if (rr >= 2 * p) rr -= 2 * p;
-            if (rr >= p) rr -= p;
-            if (neg) {  // subtract 2^(64W) mod p
-                const uint32_t cw = ct[4 + 2 * W];
-                rr = rr >= cw ? rr - cw : rr + p - cw;
-            }
-            int32_t val = rr > (p >> 1) ? (int32_t)rr - (int32_t)p : (int32_t)rr;
-            if (t == 3) {  // balanced digits in closed form: a = v + 128, b = (a >> 8) + 128
-                const int32_t a = val + 128;
-                const int32_t b = (a >> 8) + 128;
-                o[0] = bf16_bits_small((a & 255) - 128);
-                o[dstride] = bf16_bits_small((b & 255) - 128);
-                o[2 * dstride] = bf16_bits_small(b >> 8);
-            } else {
-                uint16_t* od = o;
-                for (int u = 0; u < t - 1; u++, od += dstride) {
-                    const int32_t d = ((val + 128) & 255) - 128;
-                    *od = bf16_bits_small(d);
-                    val = (val - d) >> 8;
+__host__ __device__ constexpr size_t rm_frag(int L, int KS) { return sizeof(uint2) * ((L + 7) / 8 * 3) * KS * 32; }
+
+// The tables of a basis, made with it and copied to shared memory by each block:
+// the constants' fragments (three n8 tiles for the eight primes 8B .. 8B + 7, as in
+// the conversion), and per prime {p, constant, 1 / p, constant / p - 1/2 - 2^-6},
+// for centred and then for canonical results: the constant is what the bytes' 128s
+// take off, (p - 1) / 2 for centred results, and the biases of the sums and the quotient.
+template <int W>
+void reduce_image(const uint32_t* p, int L, uint8_t* image) {
+    constexpr int KS = RmShape<W>::KS;
+    std::vector<uint64_t> c((size_t)L * 2 * W);  // 2^(32 j) mod p_i
+    for (int i = 0; i < L; i++)
+        for (int j = 0; j < 2 * W; j++) c[i * 2 * W + j] = j ? (c[i * 2 * W + j - 1] << 32) % p[i] : 1 % p[i];
+    uint16_t* wf = (uint16_t*)image;
+    for (int nt = 0; nt < (L + 7) / 8 * 3; nt++)
+        for (int ks = 0; ks < KS; ks++)
+            for (int ln = 0; ln < 32; ln++) {
+                const int n = ln >> 2, t = ln & 3, col = nt % 3 * 2 + (n & 1);
+                const int i = 4 * (nt / 3 * 2 + col / 3) + (n >> 1), dig = col % 3, limb = t * KS + ks;
+                const uint64_t w = i < L && limb < 2 * W ? c[i * 2 * W + limb] : 0;
+                for (int k = 0; k < 4; k++) {
+                    int32_t r = 0;
+                    if (i < L && limb < 2 * W) {
+                        r = (int32_t)((w << 8 * k) % p[i]);
+                        if (r > (int32_t)(p[i] >> 1)) r -= (int32_t)p[i];
+                        for (int z = 0; z < dig; z++) r = (r + 128) >> 8;
+                        if (dig < 2) r = ((r + 128) & 255) - 128;
+                    }
+                    *wf++ = half_bits(r);
                 }
-                *od = bf16_bits_small(val);
+            }
+    uint4* ti = (uint4*)(image + rm_frag(L, KS));
+    for (int ints = 0; ints < 2; ints++)
+        for (int i = 0; i < L; i++) {
+            uint64_t w = 1, sum = 0;  // 128 sum of 2^(8b) over the bytes below the top one
+            for (int b = 0; b < 8 * W - 1; b++) {
+                sum += 128 * w;
+                w = w * 256 % p[i];
+            }
+            const uint32_t c = (uint32_t)((sum + (ints ? 0u : p[i] >> 1)) % p[i]);
+            const float ip = 1.0f / (float)p[i], fc = (float)c * ip - 0.5f - 0x1p-6f;
+            uint32_t bits[2];
+            memcpy(&bits[0], &ip, 4);
+            memcpy(&bits[1], &fc, 4);
+            *ti++ = make_uint4(p[i], c - kMagicBits * 65793u + p[i] * kMagicBits, bits[0], bits[1]);
+        }
+}
+
+template <int W, bool INT>
+__device__ __forceinline__ void rm_tables(const uint8_t* __restrict__ image, int L, uint8_t* to) {
+    const size_t nf = rm_frag(L, RmShape<W>::KS);
+    stage(to, image, nf);
+    stage(to + nf, image + nf + (INT ? sizeof(uint4) * L : 0), sizeof(uint4) * L);
+    __syncthreads();
+}
+
+constexpr int word_class(int W) { return W == 1 ? 0 : W == 2 ? 1 : W == 4 ? 2 : 3; }
+
+// Does an entry, its limbs spread over the quad's lanes, lie outside [-2^bits, 2^bits] (as over_bits)?
+template <int W>
+__device__ __forceinline__ bool rm_over(const uint32_t (&v)[RmShape<W>::KS], int bits) {
+    constexpr int KS = RmShape<W>::KS;
+    const int lane = threadIdx.x & 31, t = lane & 3, Lb = bits >> 5, sh = bits & 31;
+    const bool neg = __shfl_sync(0xffffffffu, v[KS - 1], (lane & ~3) | (W == 1 ? 1 : 3)) >> 31;
+    bool over = false, one = false, nz = false;
+#pragma unroll
+    for (int k = 0; k < KS; k++) {
+        const int j = t * KS + k;
+        if (j >= 2 * W) continue;
+        if (j < Lb) {
+            nz |= v[k] != 0;
+        } else if (j == Lb) {
+            const uint32_t hi = v[k] >> sh;
+            if (neg) {
+                over |= hi != (0xFFFFFFFFu >> sh);
+            } else {
+                over |= hi > 1;
+                one |= hi == 1;
+                nz |= sh && (v[k] << (32 - sh)) != 0;
+            }
+        } else {
+            over |= v[k] != (neg ? 0xFFFFFFFFu : 0u);
+        }
+    }
+    const unsigned quad = 0xFu << (lane & ~3);
+    const unsigned bo = __ballot_sync(0xffffffffu, over), b1 = __ballot_sync(0xffffffffu, one),
+                   bn = __ballot_sync(0xffffffffu, nz);
+    return (bo & quad) || ((b1 & quad) && (bn & quad));
+}
+
+// 32 entries from minor m0 of one major, by one warp.
+template <int W, bool INT>
+__device__ __forceinline__ void rm_chunk(const RmArgs& a, int L, const uint2* wf, const uint4* ti, int64_t m0,
+                                         int64_t major) {
+    constexpr int KS = RmShape<W>::KS;
+    const int lane = threadIdx.x & 31, t = lane & 3;
+    const int64_t m = m0 + (lane >> 2) * 4;
+    uint32_t v[4][KS];
+#pragma unroll
+    for (int x = 0; x < 4; x++) {
+#pragma unroll
+        for (int k = 0; k < KS; k++) v[x][k] = 0;
+        if (m + x < a.minor_n && (W > 1 || t < 2)) {
+            const uint32_t* src = (const uint32_t*)(a.X + (size_t)((m + x) * a.smin + major * a.smaj) * W) + t * KS;
+            if constexpr (KS == 4) {
+                const uint4 q = __ldg((const uint4*)src);
+                v[x][0] = q.x;
+                v[x][1] = q.y;
+                v[x][2] = q.z;
+                v[x][3] = q.w;
+            } else if constexpr (KS == 2) {
+                const uint2 q = __ldg((const uint2*)src);
+                v[x][0] = q.x;
+                v[x][1] = q.y;
+            } else {
+                v[x][0] = __ldg(src);
+            }
+        }
+    }
+    if (a.status && a.bits < 64 * W - 1) {
+#pragma unroll
+        for (int x = 0; x < 4; x++)
+            if (rm_over<W>(v[x], a.bits)) flag_bound(a.status);
+    }
+    uint32_t f[2][KS][4];
+    const uint32_t top = t == (W == 1 ? 1 : 3) ? 0x80000000u : 0u;  // the sign: the top byte as it is
+#pragma unroll
+    for (int x = 0; x < 4; x++) {
+#pragma unroll
+        for (int k = 0; k < KS; k++) {
+            const uint32_t z = k == KS - 1 ? v[x][k] ^ top : v[x][k];
+            f[x >> 1][k][x & 1] = centre2(__byte_perm(z, 0x64u, 0x4140));
+            f[x >> 1][k][(x & 1) + 2] = centre2(__byte_perm(z, 0x64u, 0x4342));
+        }
+    }
+    const int64_t at0 = major * a.ldo + m;
+    const bool full = m + 3 < a.minor_n &&
+                      (((uint64_t)a.si | (uint64_t)a.su | (uint64_t)a.ldo) & 3) == 0 && ((uintptr_t)a.out & (INT ? 15 : 7)) == 0;
+    // a centred residue plus this has its balanced digits plus 128 as bytes
+    const uint32_t bias = a.t == 3 ? 0x808080u : a.t == 2 ? 0x8080u : 0x80u;
+#pragma unroll 1
+    for (int nb = 0; 8 * nb < L; nb++) {
+        float acc[2][3][4] = {};
+#pragma unroll
+        for (int k = 0; k < KS; k++) {
+#pragma unroll
+            for (int h = 0; h < 3; h++) {
+                const uint2 b = wf[((3 * nb + h) * KS + k) * 32 + lane];
+                mma_f16(acc[0][h], f[0][k], b);
+                mma_f16(acc[1][h], f[1][k], b);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const int i = 8 * nb + 4 * q + t;
+            if (i >= L || m >= a.minor_n) continue;
+            const uint4 c = ti[i];
+            uint32_t r[4];
+#pragma unroll
+            for (int x = 0; x < 4; x++) {
+                float s[3];
+#pragma unroll
+                for (int k = 0; k < 3; k++) s[k] = acc[x >> 1][(3 * q + k) >> 1][2 * (x & 1) + ((3 * q + k) & 1)];
+                const float g = fmaf(fmaf(s[2], 65536.f, fmaf(s[1], 256.f, s[0])), __uint_as_float(c.z), __uint_as_float(c.w));
+                uint32_t y = __float_as_uint(s[0] + kMagic) + (__float_as_uint(s[1] + kMagic) << 8) +
+                             (__float_as_uint(s[2] + kMagic) << 16) + c.y;
+                y -= __float_as_uint(g + kMagic) * c.x;
+                r[x] = min(y, y - c.x);  // [0, p)
+            }
+            const int64_t at = at0 + i * a.si;
+            if constexpr (INT) {
+                int32_t* o = (int32_t*)a.out + at;
+                if (full) {
+                    *(int4*)o = make_int4((int)r[0], (int)r[1], (int)r[2], (int)r[3]);
+                } else {
+#pragma unroll
+                    for (int x = 0; x < 4; x++)
+                        if (m + x < a.minor_n) o[x] = (int32_t)r[x];
+                }
+            } else {
+                const uint32_t off = bias - (c.x >> 1);
+                uint16_t* o = (uint16_t*)a.out + at;
+#pragma unroll
+                for (int u = 0; u < 3; u++) {
+                    if (u >= a.t) break;
+                    uint32_t d[4];
+#pragma unroll
+                    for (int x = 0; x < 4; x++) {
+                        const uint32_t z = r[x] + off;
+                        // byte u, or all that is left (up to 256) at the top, in the low bits of 0x4B400000
+                        const uint32_t e = u == 2              ? __byte_perm(z, kMagicBits, 0x7632)
+                                           : u == a.t - 1      ? (z >> 8 * u) + kMagicBits
+                                                               : __byte_perm(z, kMagicBits, 0x7640 + u);
+                        d[x] = __float_as_uint(__uint_as_float(e) - (kMagic + 128.f));
+                    }
+                    const uint32_t lo = __byte_perm(d[0], d[1], 0x7632), hi = __byte_perm(d[2], d[3], 0x7632);
+                    if (full) {
+                        *(uint2*)o = make_uint2(lo, hi);
+                    } else {
+                        if (m + 0 < a.minor_n) o[0] = (uint16_t)lo;
+                        if (m + 1 < a.minor_n) o[1] = (uint16_t)(lo >> 16);
+                        if (m + 2 < a.minor_n) o[2] = (uint16_t)hi;
+                        if (m + 3 < a.minor_n) o[3] = (uint16_t)(hi >> 16);
+                    }
+                    o += a.su;
+                }
             }
         }
     }
 }
 
-template <int W, int NC>
-__global__ void __launch_bounds__(kThreads)
-reduce_digits_t_kernel(BasisDev b, const uint64_t* __restrict__ X, int64_t rows, int64_t cols, int64_t ld,
-                       uint16_t* __restrict__ out, int64_t ld_out, int t, int group, int bits, int* status) {
-    extern __shared__ uint32_t ctab[];  // [G][NW]
-    const int i0 = blockIdx.z * group;
-    const int G = min(group, b.L - i0);
-    reduce_t_table<W>(b, ctab, i0, G);
-    __syncthreads();
-    reduce_t_thread<W, NC>(b, ctab, i0, G, X, rows, cols, ld, out, ld_out, t,
-                           (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)blockIdx.y * NC, bits, status);
+// Unit: 32 entries along the minor dimension by kMmaThreads / 32 majors, one per warp.
+template <int W, bool INT>
+__global__ void __launch_bounds__(kMmaThreads)
+reduce_mma_kernel(BasisDev b, const __grid_constant__ RmArgs a) {
+    extern __shared__ __align__(16) uint8_t dyn[];
+    uint2* wf = (uint2*)dyn;
+    uint4* ti = (uint4*)(dyn + rm_frag(b.L, RmShape<W>::KS));
+    rm_tables<W, INT>(b.red[word_class(W)], b.L, dyn);
+    const int64_t nm = (a.minor_n + 31) / 32, units = nm * ((a.major_n + 3) / 4);
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const int64_t major = u / nm * 4 + (threadIdx.x >> 5);
+        if (major < a.major_n) rm_chunk<W, INT>(a, b.L, wf, ti, u % nm * 32, major);
+    }
 }
 
-// The transposed reduce of several B operands (all of W words) in one
-// persistent launch: the table of every prime is built once per block, then
-// the block walks the items' units.  A unit is rb rows (rb = 32 .. 256, fitted
-// to the item's row count so that short operands keep the threads busy) by
-// (256 / rb) * NC columns; consecutive threads take consecutive rows.
-template <int W, int NC>
-__global__ void __launch_bounds__(kThreads, 4)  // 64 registers: four blocks per SM (measured 2 % faster than 74)
-reduce_digits_t_grouped_kernel(BasisDev b, const ReduceItem* __restrict__ items, int n, int64_t units,
-                               int* status) {
-    extern __shared__ uint32_t ctab[];  // [L][NW]
-    reduce_t_table<W>(b, ctab, 0, b.L);
-    __syncthreads();
+// The transposed reduce of several B operands (all of W words) in one persistent
+// launch.  Unit: 32 rows by kRmCols columns of one item, adjacent columns in
+// adjacent warps (an item's rows are contiguous in memory).
+constexpr int kRmCols = 16;
+template <int W>
+__global__ void __launch_bounds__(kMmaThreads)
+reduce_mma_grouped_kernel(BasisDev b, const ReduceItem* __restrict__ items, int n, int64_t units, int* status) {
+    extern __shared__ __align__(16) uint8_t dyn[];
+    uint2* wf = (uint2*)dyn;
+    uint4* ti = (uint4*)(dyn + rm_frag(b.L, RmShape<W>::KS));
+    rm_tables<W, false>(b.red[word_class(W)], b.L, dyn);
     for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
         const ReduceItem* it = find_item(items, n, u);
-        const int rb = it->rb;
-        const int64_t gx = (it->rows + rb - 1) / rb;
-        const int64_t lu = u - it->base;
-        const int64_t r = (lu % gx) * rb + threadIdx.x % rb;
-        const int64_t cb = ((lu / gx) * (kThreads / rb) + threadIdx.x / rb) * NC;
-        reduce_t_thread<W, NC>(b, ctab, 0, b.L, it->X, it->rows, it->cols, it->ld, (uint16_t*)it->out, it->ld_out,
-                               it->t, r, cb, it->bits, status);
+        const int64_t plane = it->cols * it->ld_out;
+        const RmArgs a{it->X, it->rows, it->cols, it->ld, 1, it->out, it->ld_out, plane, plane * b.L, it->t, it->bits, status};
+        const int64_t nm = (it->rows + 31) / 32, lu = u - it->base;
+        for (int k = threadIdx.x >> 5; k < kRmCols; k += kMmaThreads / 32) {
+            const int64_t c = lu / nm * kRmCols + k;
+            if (c < it->cols) rm_chunk<W, false>(a, b.L, wf, ti, lu % nm * 32, c);
+        }
     }
+}
+
+// Blocks of `kernel` resident at once with the tables of 24 primes (asked once: a property of its code).
+template <auto kernel, int W>
+int64_t rm_resident() {
+    static const int per = [] {
+        int nb = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kMmaThreads, rm_frag(24, RmShape<W>::KS) + 24 * sizeof(uint4));
+        return nb > 0 ? nb : 1;
+    }();
+    return per;
 }
 
 // Digit split of a matrix whose int64 entries (low word of W) are their own
@@ -538,6 +677,51 @@ cudaError_t launch_reduce_kind(const BasisDev& b, const ReduceArgs& a, dim3 grid
     return cudaGetLastError();
 }
 
+// The tensor-core reduction takes whole limbs per lane and three digits; other
+// word counts, wider primes and larger bases keep reduce_kernel.
+static bool mma_reducible(const BasisDev& b, const ReduceArgs& a) {
+    return !a.identity && b.L <= 64 && b.p_top < (1u << 24) && (a.W == 1 || a.W == 2 || a.W == 4 || a.W == 8) &&
+           ((uintptr_t)a.X & (a.W == 8 ? 15 : 7)) == 0;
+}
+
+template <int W>
+static cudaError_t launch_reduce_mma(const BasisDev& b, const ReduceArgs& a, ReduceOut kind, cudaStream_t s) {
+    const bool trans = kind == ReduceOut::kDigitsT, ints = kind == ReduceOut::kCanonical;
+    RmArgs r{a.X, trans ? a.rows : a.cols, trans ? a.cols : a.rows, trans ? a.ld : 1, trans ? 1 : a.ld,
+             a.out, ints ? a.cols : a.ld_out, 0, 0, a.t, a.bits, a.status};
+    if (ints) {  // [L][rows][cols]
+        r.si = r.su = a.rows * a.cols;
+    } else if (trans) {  // [t][L][cols][ld_out]
+        r.si = a.cols * a.ld_out;
+        r.su = r.si * b.L;
+    } else {  // [L][t][rows][ld_out]
+        r.su = a.rows * a.ld_out;
+        r.si = r.su * a.t;
+    }
+    const size_t sm = rm_frag(b.L, RmShape<W>::KS) + (size_t)b.L * sizeof(uint4);
+    const int64_t units = ((r.minor_n + 31) / 32) * ((r.major_n + 3) / 4);
+    if (ints) {
+        const int64_t most = b.sms * rm_resident<reduce_mma_kernel<W, true>, W>();
+        reduce_mma_kernel<W, true><<<(unsigned)(units < most ? units : most), kMmaThreads, sm, s>>>(b, r);
+    } else {
+        const int64_t most = b.sms * rm_resident<reduce_mma_kernel<W, false>, W>();
+        reduce_mma_kernel<W, false><<<(unsigned)(units < most ? units : most), kMmaThreads, sm, s>>>(b, r);
+    }
+    return cudaGetLastError();
+}
+
+size_t reduce_image_bytes(int L, uint32_t p_top, int W) {
+    if (L > 64 || p_top >= (1u << 24)) return 0;
+    return rm_frag(L, W == 1 ? 1 : W / 2) + 2 * (size_t)L * sizeof(uint4);
+}
+
+void reduce_image_make(const uint32_t* p, int L, int W, uint8_t* image) {
+    if (W == 1) reduce_image<1>(p, L, image);
+    else if (W == 2) reduce_image<2>(p, L, image);
+    else if (W == 4) reduce_image<4>(p, L, image);
+    else reduce_image<8>(p, L, image);
+}
+
 cudaError_t launch_reduce(const BasisDev& b, const ReduceArgs& a_in, ReduceOut kind, int* d_status,
                           cudaStream_t s) {
     if (a_in.rows == 0 || a_in.cols == 0) return cudaSuccess;
@@ -555,23 +739,11 @@ cudaError_t launch_reduce(const BasisDev& b, const ReduceArgs& a_in, ReduceOut k
     }
     const int nw = (2 * a.W + 1 + 3) & ~3;
     int group = a.identity ? 1 : max(1, min(b.L, kTableWords / (nw + 4)));
-    if (kind == ReduceOut::kDigitsT && !a.identity && (((uintptr_t)a.X & 15) == 0) &&
-        (a.W == 1 || a.W == 2 || a.W == 4 || a.W == 8) && (a.W == 1 || a.ld % 2 == 0)) {
-        constexpr int NC = 4;
-        dim3 grid((unsigned)((a.rows + kThreads - 1) / kThreads), (unsigned)((a.cols + NC - 1) / NC),
-                  (unsigned)((b.L + group - 1) / group));
-        if (grid.y > 65535) goto generic;
-        const size_t sm = sizeof(uint32_t) * (size_t)group * (nw + 4);
-        uint16_t* o = (uint16_t*)a.out;
-        switch (a.W) {
-            case 1: reduce_digits_t_kernel<1, NC><<<grid, kThreads, sm, s>>>(b, a.X, a.rows, a.cols, a.ld, o, a.ld_out, a.t, group, a.bits, a.status); break;
-            case 2: reduce_digits_t_kernel<2, NC><<<grid, kThreads, sm, s>>>(b, a.X, a.rows, a.cols, a.ld, o, a.ld_out, a.t, group, a.bits, a.status); break;
-            case 4: reduce_digits_t_kernel<4, NC><<<grid, kThreads, sm, s>>>(b, a.X, a.rows, a.cols, a.ld, o, a.ld_out, a.t, group, a.bits, a.status); break;
-            default: reduce_digits_t_kernel<8, NC><<<grid, kThreads, sm, s>>>(b, a.X, a.rows, a.cols, a.ld, o, a.ld_out, a.t, group, a.bits, a.status); break;
-        }
-        return cudaGetLastError();
-    }
-generic:
+    if (mma_reducible(b, a) && (kind == ReduceOut::kCanonical || (kind != ReduceOut::kCentered && a.t <= 3)))
+        return a.W == 1   ? launch_reduce_mma<1>(b, a, kind, s)
+               : a.W == 2 ? launch_reduce_mma<2>(b, a, kind, s)
+               : a.W == 4 ? launch_reduce_mma<4>(b, a, kind, s)
+                          : launch_reduce_mma<8>(b, a, kind, s);
     const int groups = a.identity ? 1 : (b.L + group - 1) / group;
     const bool trans = kind == ReduceOut::kDigitsT;
     const int64_t minor_n = trans ? a.rows : a.cols;
@@ -606,8 +778,6 @@ cudaError_t launch_residue_digits(const BasisDev& b, const int32_t* R, int64_t p
 }
 
 namespace {
-constexpr int kNC = 4;  // columns per block of the transposed reduce
-
 // blocks of `kernel` resident per SM (at least one), computed once per kernel
 template <class Kern>
 int resident(Kern kernel, int threads, size_t smem) {
@@ -627,28 +797,16 @@ int64_t persistent_grid(int64_t units, int num_sms, int per_sm) {
 template <int W>
 cudaError_t launch_rt_grouped_w(const BasisDev& b, const ReduceItem* items, int n, int64_t units, int num_sms,
                                 int* status, cudaStream_t s) {
-    const size_t sm = sizeof(uint32_t) * (size_t)b.L * RtTable<W>::NW;
-    static int per_sm = 0;
-    if (!per_sm) per_sm = resident(reduce_digits_t_grouped_kernel<W, kNC>, kThreads, sizeof(uint32_t) * 64 * RtTable<W>::NW);
-    const int64_t grid = persistent_grid(units, num_sms, per_sm);
-    reduce_digits_t_grouped_kernel<W, kNC><<<(unsigned)grid, kThreads, sm, s>>>(b, items, n, units, status);
+    const size_t sm = rm_frag(b.L, RmShape<W>::KS) + (size_t)b.L * sizeof(uint4);
+    const int64_t grid = persistent_grid(units, num_sms, (int)rm_resident<reduce_mma_grouped_kernel<W>, W>());
+    reduce_mma_grouped_kernel<W><<<(unsigned)grid, kMmaThreads, sm, s>>>(b, items, n, units, status);
     return cudaGetLastError();
 }
 }  // namespace
 
-int64_t reduce_t_units(int64_t rows, int64_t cols, int* rb) {
-    int h = 32;
-    while (h < kThreads && h < rows) h *= 2;
-    *rb = h;
-    const int64_t cpu = (int64_t)(kThreads / h) * kNC;  // columns per unit
-    return ((rows + h - 1) / h) * ((cols + cpu - 1) / cpu);
-}
+int64_t reduce_t_units(int64_t rows, int64_t cols) { return ((rows + 31) / 32) * ((cols + kRmCols - 1) / kRmCols); }
 
-bool reduce_t_groupable(const BasisDev& b, const ReduceArgs& a) {
-    const int nw = (2 * a.W + 1 + 3) & ~3;
-    return !a.identity && ((uintptr_t)a.X & 15) == 0 && (a.W == 1 || a.W == 2 || a.W == 4 || a.W == 8) &&
-           (a.W == 1 || a.ld % 2 == 0) && b.L <= 64 && b.L <= kTableWords / (nw + 4);
-}
+bool reduce_t_groupable(const BasisDev& b, const ReduceArgs& a) { return mma_reducible(b, a) && a.t <= 3; }
 
 int64_t split_units(int64_t rows, int64_t cols, uint32_t* div_m, int* div_s) {
     // m = ceil(2^(32+s) / d) with 2^s >= d lies in (2^32, 2^33]; its low 32 bits

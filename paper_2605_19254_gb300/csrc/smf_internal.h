@@ -28,6 +28,9 @@ struct BasisDev {
     const uint32_t* p;        // [L] primes, descending
     const uint64_t* mu;       // [L] floor((2^64 - 1) / p_i), Barrett reduction
     const uint32_t* pow32;    // [L] 2^32 mod p_i
+    const uint8_t* red[4];    // tables of the tensor-core reductions of entries of 1, 2, 4, 8 words (reduce_image)
+    uint32_t p_top;           // the largest prime
+    int sms;                  // SMs of the device the tables are on
     const double* inv_p;      // [L] 1/p_i rounded to fp64 (Section 3.1 fast reduction)
     // Garner: for j < i, w[i*L + j] = p_j mod p_i with its Shoup companion
     // floor(w * 2^32 / p_i); inv[i] = (p_0 ... p_{i-1})^-1 mod p_i likewise.
@@ -53,6 +56,12 @@ struct CrtHost {
     const uint32_t* cs = nullptr;     // [L] Shoup companions of c
     const uint32_t* mi = nullptr;     // [L][m_limbs] limbs of M_i
     const uint32_t* h = nullptr;      // [m_limbs] limbs of H
+    // on the device: limbs of M_i and M; for primes below 2^24 the tensor-core
+    // kernels' tables (crt_image_make), and in them {p_i, H mod p_i, c_i, companion}
+    const uint32_t* d_mi = nullptr;
+    const uint32_t* d_m = nullptr;
+    const uint8_t* d_image = nullptr;
+    const uint8_t* d_pc = nullptr;
 };
 
 }  // namespace smf
@@ -290,7 +299,6 @@ struct ReduceItem {       // one operand of a grouped digit split or transposed 
     int64_t ld_out;
     int W, t;
     int bits;             // declared bound of the entries (checked; >= 64 W - 1: not checked)
-    int rb;               // transposed reduce: rows per unit (set by reduce_t_units)
     int64_t base;
     // digit split: floor(e / cols) = (umulhi(e, div_m) + e) >> div_s for e < 2^32
     // (division by an invariant integer, Granlund and Montgomery; set by split_units)
@@ -323,11 +331,10 @@ __device__ __forceinline__ const Item* find_item(const Item* items, int n, int64
     return items + lo;
 }
 #endif
-// Work units of one item: transposed reduce of B (rb rows by 1024 / rb
-// columns, rb fitted to the row count and returned), digit split of a
-// shared-digit A (2048 entries), CRT (128 entries).
-int64_t reduce_t_units(int64_t rows, int64_t cols, int* rb);
-bool reduce_t_groupable(const BasisDev& b, const ReduceArgs& a);  // W in {1, 2, 4, 8}, aligned, one prime group
+// Work units of one item: transposed reduce of B (32 rows by 16 columns),
+// digit split of a shared-digit A (2048 entries), CRT (128 entries).
+int64_t reduce_t_units(int64_t rows, int64_t cols);
+bool reduce_t_groupable(const BasisDev& b, const ReduceArgs& a);  // W in {1, 2, 4, 8}, at most 64 primes below 2^24
 int64_t split_units(int64_t rows, int64_t cols, uint32_t* div_m, int* div_s);
 int64_t crt_units(int64_t rows, int64_t cols);
 // One persistent launch each (grid: the SMs times the blocks resident per SM).
@@ -426,9 +433,16 @@ int64_t limb_crt_units(int64_t M, int64_t N);
 cudaError_t launch_gemm_limb_crt(smf_ctx* ctx, const BasisDev& b, const CrtHost& h, const LimbGemmArgs& a,
                                  int* count, uint64_t* X, int64_t ld, int W, cudaStream_t s);
 
+// The CRT's tables for the tensor cores (0 bytes: the basis is not for them), and
+// where the per-prime constants lie in them; the reductions' tables for W words.
+size_t crt_image_bytes(const CrtHost& h, size_t* pc);
+void crt_image_make(const CrtHost& h, uint8_t* image);
+size_t reduce_image_bytes(int L, uint32_t p_top, int W);
+void reduce_image_make(const uint32_t* p, int L, int W, uint8_t* image);
+
 // CRT reconstruction: Lagrange form with an fp32 correction, exact mixed-radix (Garner) fallback.
 cudaError_t launch_crt(const CrtHost& h, const int32_t* R, int64_t rows, int64_t cols,
-                       uint64_t* X, int64_t ld, int W, cudaStream_t s);
+                       uint64_t* X, int64_t ld, int W, int num_sms, cudaStream_t s);
 
 cudaError_t launch_crt_grouped(const CrtHost& h, const CrtItem* items, int n, int64_t units, int num_sms,
                                cudaStream_t s);
