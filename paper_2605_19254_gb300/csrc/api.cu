@@ -1069,11 +1069,7 @@ int plan_lift_limb(smf_ctx* ctx, const smf_bigmat* A, int pbits, LiftPlan* P) {
     const int LQ = (int)Q->primes.size();
     if (LQ > kLiftMaxPrimes) return fail(ctx, SMF_E_UNSUPPORTED, "padic_lift: product basis over four primes");
     P->Q = Q;
-    P->lq.L = LQ;
-    for (int j = 0; j < LQ; j++) {
-        P->lq.q[j] = Q->primes[j];
-        P->lq.inv[j] = Q->ginv[j];
-    }
+    lift_basis(*Q, P->p, &P->lq);
     const uint64_t h = P->p / 2, hL = Q->primes.back() / 2, h0 = Q->primes[0] / 2;
     P->a_shared = ab < 62 && (1ull << ab) <= hL && ab <= 30;
     P->amax2 = P->a_shared ? (1ull << ab) : h0;
@@ -1813,12 +1809,12 @@ int smf_padic_lift(smf_ctx* ctx, const smf_basis* p_basis, const smf_bigmat* A, 
             l1.bn = P.g1.bn;
             ctx->inject = 0;
             SMF_CU(ctx, launch_gemm_limb(ctx, p_basis->dev, l1, s));
-            SMF_CU(ctx, launch_lift_x(c1, P.g1.split, n, m, P.p, Xi, P.lq, xdig, P.g2.ldb, P.g2.TB, s));
+            SMF_CU(ctx, launch_lift_x(c1, P.g1.split, n, m, Xi, P.lq, xdig, P.g2.ldb, P.g2.TB, s));
             LimbGemmArgs l2{adig, P.g2.lda, P.a_shared ? 1 : 0, xdig, P.g2.ldb, c2, n, m, n, P.g2.TA,
                             P.g2.TB, ctx->d_status, 0, P.amax2, P.bmax2, c2, P.g2.split, P.g2.kchunk, 1, 1};
             l2.bn = P.g2.bn;
             SMF_CU(ctx, launch_gemm_limb(ctx, P.Q->dev, l2, s));
-            SMF_CU(ctx, launch_lift_step(c2, P.g2.split, n, m, P.lq, (int64_t*)R->data, R->ld, P.p,
+            SMF_CU(ctx, launch_lift_step(c2, P.g2.split, n, m, P.lq, (int64_t*)R->data, R->ld,
                                          i + 1 < steps ? rdig : nullptr, P.g1.ldb, P.g1.TB, ctx->d_status, s));
         }
         return SMF_OK;

@@ -612,8 +612,6 @@ __device__ __forceinline__ void wide_body(const CUtensorMap* tmA, const CUtensor
                                           const FusedCrt* fz) {
     using namespace wide;
     constexpr bool GROUPED = MODE == 1;
-    pdl_wait();  // a no-op unless launched as a programmatic dependent
-    pdl_trigger();
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE_BYTES);
@@ -662,6 +660,10 @@ __device__ __forceinline__ void wide_body(const CUtensorMap* tmA, const CUtensor
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // As a programmatic dependent the set-up above overlaps the kernel before;
+    // operands are read and results written only after it.
+    pdl_wait();
+    pdl_trigger();
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer: a continuous stream of K steps over this CTA's tiles

@@ -487,18 +487,25 @@ cudaError_t launch_lift_combine(const int32_t* X, int64_t steps, int64_t n, int6
 constexpr int kLiftMaxPrimes = 4;
 struct LiftBasis {
     int L;
-    uint32_t q[kLiftMaxPrimes];
-    uint32_t inv[kLiftMaxPrimes];
+    uint32_t q[kLiftMaxPrimes], rcp[kLiftMaxPrimes];      // and floor(2^32 / q_j)
+    uint32_t inv[kLiftMaxPrimes], invs[kLiftMaxPrimes];   // (q_0 ... q_(j-1))^-1 mod q_j, Shoup companion
+    uint32_t w[kLiftMaxPrimes][kLiftMaxPrimes];           // q_0 ... q_(i-1) mod q_j, i < j
+    uint32_t ws[kLiftMaxPrimes][kLiftMaxPrimes];
+    uint64_t W[kLiftMaxPrimes], Q;                        // q_0 ... q_(j-1) and their product, mod 2^64
+    uint32_t p, prcp, p32, p32s;                          // floor(2^32 / p); 2^32 mod p, Shoup companion
+    uint64_t pinv;                                        // p^-1 mod 2^64
+    int64_t qmax;                                         // floor((2^63 - 1) / p)
 };
+void lift_basis(const smf_basis& Q, uint32_t p, LiftBasis* q);
 // part: [split][n][m] canonical partials of C R_i mod p -> X (n x m, [0, p)) and
 // the centred residues of X modulo q as t-digit planes [t][L][m][ldd].
-cudaError_t launch_lift_x(const int32_t* part, int split, int64_t n, int64_t m, uint32_t p, int32_t* X,
-                          const LiftBasis& q, void* xdig, int64_t ldd, int t, cudaStream_t s);
+cudaError_t launch_lift_x(const int32_t* part, int split, int64_t n, int64_t m, int32_t* X, const LiftBasis& q,
+                          void* xdig, int64_t ldd, int t, cudaStream_t s);
 // part: [split][L][n][m] canonical partials of A X_i mod q_j -> R = (R - A X_i) / p
 // (flags kStatusInexact on a remainder); rdig, when not null, gets the t-digit
 // planes [t][m][ldd] of R mod p (centred).
 cudaError_t launch_lift_step(const int32_t* part, int split, int64_t n, int64_t m, const LiftBasis& q, int64_t* R,
-                             int64_t ldR, uint32_t p, void* rdig, int64_t ldd, int t, int* status, cudaStream_t s);
+                             int64_t ldR, void* rdig, int64_t ldd, int t, int* status, cudaStream_t s);
 cudaError_t launch_lift_update(int64_t* R, int64_t ldR, const int64_t* AX, int64_t rows, int64_t cols, uint32_t p,
                                int* status, cudaStream_t s);
 
