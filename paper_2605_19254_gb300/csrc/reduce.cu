@@ -11,8 +11,6 @@
 // launch's group are built once per block in shared memory.
 #include <cuda_bf16.h>
 
-#include <vector>
-
 #include "rns_mma.h"
 
 namespace smf {
@@ -264,27 +262,23 @@ __host__ __device__ constexpr size_t rm_frag(int L, int KS) { return sizeof(uint
 template <int W>
 void reduce_image(const uint32_t* p, int L, uint8_t* image) {
     constexpr int KS = RmShape<W>::KS;
-    std::vector<uint64_t> c((size_t)L * 2 * W);  // 2^(32 j) mod p_i
-    for (int i = 0; i < L; i++)
-        for (int j = 0; j < 2 * W; j++) c[i * 2 * W + j] = j ? (c[i * 2 * W + j - 1] << 32) % p[i] : 1 % p[i];
     uint16_t* wf = (uint16_t*)image;
-    for (int nt = 0; nt < (L + 7) / 8 * 3; nt++)
-        for (int ks = 0; ks < KS; ks++)
-            for (int ln = 0; ln < 32; ln++) {
-                const int n = ln >> 2, t = ln & 3, col = nt % 3 * 2 + (n & 1);
-                const int i = 4 * (nt / 3 * 2 + col / 3) + (n >> 1), dig = col % 3, limb = t * KS + ks;
-                const uint64_t w = i < L && limb < 2 * W ? c[i * 2 * W + limb] : 0;
-                for (int k = 0; k < 4; k++) {
-                    int32_t r = 0;
-                    if (i < L && limb < 2 * W) {
-                        r = (int32_t)((w << 8 * k) % p[i]);
-                        if (r > (int32_t)(p[i] >> 1)) r -= (int32_t)p[i];
-                        for (int z = 0; z < dig; z++) r = (r + 128) >> 8;
-                        if (dig < 2) r = ((r + 128) & 255) - 128;
-                    }
-                    *wf++ = half_bits(r);
-                }
+    memset(wf, 0, rm_frag(L, KS));
+    for (int i = 0; i < L; i++) {
+        uint64_t w = 1;  // 2^(8b) mod p_i
+        for (int b = 0; b < 8 * W; b++) {
+            int32_t r = (int32_t)w;
+            if (r > (int32_t)(p[i] >> 1)) r -= (int32_t)p[i];
+            const int limb = b >> 2, t = limb / KS, ks = limb % KS;
+            for (int dig = 0; dig < 3; dig++) {
+                const int c6 = (i >> 2 & 1) * 3 + dig, nt = (i >> 3) * 3 + c6 / 2;
+                const int ln = (2 * (i & 3) + (c6 & 1)) * 4 + t;
+                wf[((nt * KS + ks) * 32 + ln) * 4 + (b & 3)] = half_bits(dig < 2 ? ((r + 128) & 255) - 128 : r);
+                r = (r + 128) >> 8;
             }
+            w = w * 256 % p[i];
+        }
+    }
     uint4* ti = (uint4*)(image + rm_frag(L, KS));
     for (int ints = 0; ints < 2; ints++)
         for (int i = 0; i < L; i++) {
