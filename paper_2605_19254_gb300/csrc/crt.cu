@@ -232,22 +232,14 @@ __device__ __forceinline__ void crt_chunk(const XiExact& q, const CrtSmem<LMAX>&
     int32_t carry[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int l = 0; l < Q::LPT; l++) {
-        float acc[2][2][4] = {};
-#pragma unroll
-        for (int ks = 0; ks < Q::KS; ks++) {
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                const uint2 b = sm.wf[((2 * l + h) * Q::KS + ks) * 32 + lane];
-                mma_f16(acc[0][h], a[0][ks], b);
-                mma_f16(acc[1][h], a[1][ks], b);
-            }
-        }
+        float acc[2][2][4];
+        mma_tiles<2, Q::KS>(acc, a, sm.wf + 2 * l * Q::KS * 32 + lane);
         const uint2 k = sm.cn[t * Q::LPT + l];
 #pragma unroll
         for (int e = 0; e < 4; e++) {
             uint32_t s[4];  // the four column sums, each 0x4B400000 too large
 #pragma unroll
-            for (int b = 0; b < 4; b++) s[b] = __float_as_uint(acc[e >> 1][b >> 1][2 * (e & 1) + (b & 1)] + kMagic);
+            for (int b = 0; b < 4; b++) s[b] = __float_as_uint(acc[e >> 1][b >> 1][2 * (e & 1) + (b & 1)]);
             const int32_t lo = (int32_t)(s[0] + (s[1] << 8) - kMagicBits * 257u);  // below 2^30 in absolute value
             const int32_t hi = (int32_t)(s[2] + (s[3] << 8) - kMagicBits * 257u);
             const int64_t v = (int64_t)((uint64_t)alpha[e] * k.y + k.x) + (int64_t)hi * 65536 + ((int64_t)lo + carry[e]);
@@ -282,13 +274,20 @@ __device__ __forceinline__ void crt_chunk(const XiExact& q, const CrtSmem<LMAX>&
     const int left = (int)min((int64_t)32, count - e0);
     const int de = 32 / W, dw = 32 % W;
     int e = lane / W, w = lane % W;
+    uint64_t* to = X + e0 * W + lane;  // ld = cols: the words follow one another
     while (e < left) {
         const uint32_t* s = sm.st + e * Q::SE;
-        const uint32_t ext = (uint32_t)((int32_t)s[Q::NL - 1] >> 31);
-        const uint32_t lo = 2 * w < Q::NL ? s[2 * w] : ext, hi = 2 * w + 1 < Q::NL ? s[2 * w + 1] : ext;
-        int64_t at = e0 + e;
-        if (ld != cols) at = at / cols * ld + at % cols;
-        X[at * W + w] = (uint64_t)hi << 32 | lo;
+        uint32_t lo, hi;
+        if (2 * w + 1 < Q::NL) {
+            lo = s[2 * w];
+            hi = s[2 * w + 1];
+        } else {  // the sign
+            hi = (uint32_t)((int32_t)s[Q::NL - 1] >> 31);
+            lo = 2 * w < Q::NL ? s[2 * w] : hi;
+        }
+        if (ld == cols) *to = (uint64_t)hi << 32 | lo;
+        else X[((e0 + e) / cols * ld + (e0 + e) % cols) * W + w] = (uint64_t)hi << 32 | lo;
+        to += 32;
         e += de;
         w += dw;
         if (w >= W) {
@@ -300,7 +299,7 @@ __device__ __forceinline__ void crt_chunk(const XiExact& q, const CrtSmem<LMAX>&
 }
 
 template <int LMAX>
-__global__ void __launch_bounds__(kMmaThreads, LMAX <= 24 ? 4 : 1)
+__global__ void __launch_bounds__(kMmaThreads, LMAX <= 16 ? 5 : LMAX <= 32 ? 4 : 3)
 crt_mma_kernel(const uint8_t* __restrict__ image, XiExact q, const int32_t* __restrict__ R, int64_t rows,
                int64_t cols, uint64_t* __restrict__ X, int64_t ld, int W) {
     extern __shared__ __align__(16) uint8_t dyn[];
@@ -314,7 +313,7 @@ crt_mma_kernel(const uint8_t* __restrict__ image, XiExact q, const int32_t* __re
 // Several outputs of one basis in one launch: unit u is the 128 consecutive
 // entries u - base_i of item i (found by bisection).
 template <int LMAX>
-__global__ void __launch_bounds__(kMmaThreads, LMAX <= 24 ? 4 : 1)
+__global__ void __launch_bounds__(kMmaThreads, LMAX <= 16 ? 5 : LMAX <= 32 ? 4 : 3)
 crt_mma_grouped_kernel(const uint8_t* __restrict__ image, XiExact q, const CrtItem* __restrict__ items, int n,
                        int64_t units) {
     extern __shared__ __align__(16) uint8_t dyn[];
@@ -422,22 +421,21 @@ cudaError_t launch_crt_mma_grouped(const CrtHost& h, const CrtItem* items, int n
 // Lane 4g + t owns target primes j = 4b + t, three columns each; three n8 tiles
 // hold two targets of a lane.  A residue is then
 //   v = S_0 + 2^8 S_1 + 2^16 S_2 + C_j - alpha (M mod q_j)  mod q_j:
-// the quotient in fp32 (|v / q_j| < 2^14, its error below 2^-7, so a floor taken
-// 2^-6 low leaves [0, 1.04 q_j)), the remainder in wrapping 32 bits.
+// sums_quot and sums_rem have the arithmetic.
 // 23 -> 23 primes, 1M entries: 159 -> 79 us (28 us of HBM traffic); bound by issue.
 template <int LMAX>
 struct ConvMma {
     const uint4* pc;          // the source's constants (device)
     XiExact xi;
     uint32_t w[LMAX * LMAX];  // w_ij at j LMAX + i
-    uint4 ti[LMAX];           // q_j, M mod q_j, C_j with the biases of the sums and the quotient taken out
-    float4 tf[LMAX];          // 1 / q_j, (M mod q_j) / q_j, C_j / q_j - 1/2 - 2^-6
+    uint4 ti[LMAX];           // q_j, M mod q_j, rem_const of C_j
+    float4 tf[LMAX];          // 1 / q_j, (M mod q_j) / q_j, quot_const of C_j
     int LQ;
 };
 static_assert(sizeof(ConvMma<48>) <= 32000, "kernel parameter space");
 
 template <int LMAX>
-__global__ void __launch_bounds__(kMmaThreads)
+__global__ void __launch_bounds__(kMmaThreads, LMAX <= 24 ? 5 : LMAX <= 32 ? 4 : 3)
 convert_mma_kernel(const __grid_constant__ ConvMma<LMAX> v, const int32_t* __restrict__ R, int32_t* __restrict__ out,
                    int64_t count) {
     constexpr int KS = XiShape<LMAX>::KS, NB = LMAX / 8;  // groups of eight targets
@@ -485,16 +483,8 @@ convert_mma_kernel(const __grid_constant__ ConvMma<LMAX> v, const int32_t* __res
         const int64_t e = e0 + (lane >> 2) * 4;
 #pragma unroll 1
         for (int nb = 0; 8 * nb < LQ; nb++) {
-            float acc[2][3][4] = {};
-#pragma unroll
-            for (int ks = 0; ks < KS; ks++) {
-#pragma unroll
-                for (int h = 0; h < 3; h++) {
-                    const uint2 b = wf[((3 * nb + h) * KS + ks) * 32 + lane];
-                    mma_f16(acc[0][h], a[0][ks], b);
-                    mma_f16(acc[1][h], a[1][ks], b);
-                }
-            }
+            float acc[2][3][4];
+            mma_tiles<3, KS>(acc, a, wf + 3 * nb * KS * 32 + lane);
 #pragma unroll
             for (int b = 0; b < 2; b++) {
                 const int j = 8 * nb + 4 * b + t;
@@ -507,13 +497,8 @@ convert_mma_kernel(const __grid_constant__ ConvMma<LMAX> v, const int32_t* __res
                     float s[3];
 #pragma unroll
                     for (int k = 0; k < 3; k++) s[k] = acc[x >> 1][(3 * b + k) >> 1][2 * (x & 1) + ((3 * b + k) & 1)];
-                    float f = fmaf(fmaf(s[2], 65536.f, fmaf(s[1], 256.f, s[0])), cf.x, cf.z);
-                    f = fmaf(-al[x], cf.y, f);
-                    const uint32_t quo = __float_as_uint(f + kMagic);
-                    uint32_t y = __float_as_uint(s[0] + kMagic) + (__float_as_uint(s[1] + kMagic) << 8) +
-                                 (__float_as_uint(s[2] + kMagic) << 16) + ci.z;
-                    y -= alpha[x] * ci.y;
-                    y -= quo * ci.x;
+                    const float f = fmaf(-al[x], cf.y, sums_quot(s[0], s[1], s[2], cf.x, cf.z));
+                    const uint32_t y = sums_rem(s[0], s[1], s[2], ci.x, ci.z, f) - alpha[x] * ci.y;
                     r[x] = min(y, y - ci.x);
                 }
                 int32_t* o = out + (size_t)j * count + e;
@@ -559,8 +544,9 @@ cudaError_t launch_convert_mma(const CrtHost& h, const uint32_t* q, int LQ, cons
         }
         const uint32_t m = (uint32_t)before, hm = limbs_mod(h.h, h.m_limbs, qj);
         const uint32_t c = (uint32_t)((sum * (128u * 65793u) + qj - hm) % qj);  // (every digit of xi is less 128)
-        v.ti[j] = make_uint4(qj, m, c - kMagicBits * 65793u + qj * kMagicBits, 0);
-        v.tf[j] = make_float4(1.0f / (float)qj, (float)m / (float)qj, (float)c / (float)qj - 0.5f - 0x1p-6f, 0.f);
+        const float iq = 1.0f / (float)qj;
+        v.ti[j] = make_uint4(qj, m, rem_const(c, qj), 0);
+        v.tf[j] = make_float4(iq, (float)m / (float)qj, quot_const(c, iq, qj), 0.f);
     }
     v.LQ = LQ;
     unsigned grid;
@@ -631,7 +617,8 @@ cudaError_t launch_convert_t(const CrtHost& h, const uint32_t* q, int LQ, const 
 }
 
 // The tensor-core kernels take primes below 2^24 (the limb form's bases), whose
-// three digits keep the fp32 sums exact; wider primes keep the multiply-adds.
+// three digits keep the fp32 sums exact; wider primes, and targets below 2^22
+// (kMinPrime), keep the multiply-adds.
 bool narrow_basis(const CrtHost& h) { return h.L > 0 && h.L <= 48 && h.p[0] < (1u << 24); }
 
 }  // namespace
@@ -697,7 +684,7 @@ cudaError_t launch_convert(const CrtHost& from, const uint32_t* q, int LQ, const
     if (count == 0 || LQ == 0) return cudaSuccess;
     const int n = from.L > LQ ? from.L : LQ;
     bool narrow = narrow_basis(from);
-    for (int j = 0; j < LQ; j++) narrow &= q[j] < (1u << 24);
+    for (int j = 0; j < LQ; j++) narrow &= q[j] < (1u << 24) && q[j] >= kMinPrime;
     if (narrow) {
         if (n <= 8) return launch_convert_mma<8>(from, q, LQ, R, out, count, num_sms, s);
         if (n <= 16) return launch_convert_mma<16>(from, q, LQ, R, out, count, num_sms, s);

@@ -227,7 +227,7 @@ reduce_kernel(BasisDev b, ReduceArgs a, int group) {
 }
 
 // ---------------------------------------------------------------------------
-// The reductions modulo at most 64 primes below 2^24 of entries of 1, 2, 4 or 8
+// The reductions modulo at most 64 primes in [2^22, 2^24) of entries of 1, 2, 4 or 8
 // words, on the tensor cores (rns_mma.h has the layout).  x mod p_i is a product
 // of the entry's 8 W bytes with the constants 2^(8b) mod p_i: bytes less 128 (the
 // top one signed as it is) and balanced digits of the constants, fp32 sums below
@@ -256,9 +256,9 @@ __host__ __device__ constexpr size_t rm_frag(int L, int KS) { return sizeof(uint
 
 // The tables of a basis, made with it and copied to shared memory by each block:
 // the constants' fragments (three n8 tiles for the eight primes 8B .. 8B + 7, as in
-// the conversion), and per prime {p, constant, 1 / p, constant / p - 1/2 - 2^-6},
-// for centred and then for canonical results: the constant is what the bytes' 128s
-// take off, (p - 1) / 2 for centred results, and the biases of the sums and the quotient.
+// the conversion), and per prime {p, rem_const, 1 / p, quot_const} of the constant,
+// for centred and then for canonical results: what the bytes' 128s take off, and
+// (p - 1) / 2 for centred results.
 template <int W>
 void reduce_image(const uint32_t* p, int L, uint8_t* image) {
     constexpr int KS = RmShape<W>::KS;
@@ -288,11 +288,11 @@ void reduce_image(const uint32_t* p, int L, uint8_t* image) {
                 w = w * 256 % p[i];
             }
             const uint32_t c = (uint32_t)((sum + (ints ? 0u : p[i] >> 1)) % p[i]);
-            const float ip = 1.0f / (float)p[i], fc = (float)c * ip - 0.5f - 0x1p-6f;
+            const float ip = 1.0f / (float)p[i], fc = quot_const(c, ip, p[i]);
             uint32_t bits[2];
             memcpy(&bits[0], &ip, 4);
             memcpy(&bits[1], &fc, 4);
-            *ti++ = make_uint4(p[i], c - kMagicBits * 65793u + p[i] * kMagicBits, bits[0], bits[1]);
+            *ti++ = make_uint4(p[i], rem_const(c, p[i]), bits[0], bits[1]);
         }
 }
 
@@ -390,16 +390,8 @@ __device__ __forceinline__ void rm_chunk(const RmArgs& a, int L, const uint2* wf
     const uint32_t bias = a.t == 3 ? 0x808080u : a.t == 2 ? 0x8080u : 0x80u;
 #pragma unroll 1
     for (int nb = 0; 8 * nb < L; nb++) {
-        float acc[2][3][4] = {};
-#pragma unroll
-        for (int k = 0; k < KS; k++) {
-#pragma unroll
-            for (int h = 0; h < 3; h++) {
-                const uint2 b = wf[((3 * nb + h) * KS + k) * 32 + lane];
-                mma_f16(acc[0][h], f[0][k], b);
-                mma_f16(acc[1][h], f[1][k], b);
-            }
-        }
+        float acc[2][3][4];
+        mma_tiles<3, KS>(acc, f, wf + 3 * nb * KS * 32 + lane);
 #pragma unroll
         for (int q = 0; q < 2; q++) {
             const int i = 8 * nb + 4 * q + t;
@@ -411,10 +403,8 @@ __device__ __forceinline__ void rm_chunk(const RmArgs& a, int L, const uint2* wf
                 float s[3];
 #pragma unroll
                 for (int k = 0; k < 3; k++) s[k] = acc[x >> 1][(3 * q + k) >> 1][2 * (x & 1) + ((3 * q + k) & 1)];
-                const float g = fmaf(fmaf(s[2], 65536.f, fmaf(s[1], 256.f, s[0])), __uint_as_float(c.z), __uint_as_float(c.w));
-                uint32_t y = __float_as_uint(s[0] + kMagic) + (__float_as_uint(s[1] + kMagic) << 8) +
-                             (__float_as_uint(s[2] + kMagic) << 16) + c.y;
-                y -= __float_as_uint(g + kMagic) * c.x;
+                const uint32_t y =
+                    sums_rem(s[0], s[1], s[2], c.x, c.y, sums_quot(s[0], s[1], s[2], __uint_as_float(c.z), __uint_as_float(c.w)));
                 r[x] = min(y, y - c.x);  // [0, p)
             }
             const int64_t at = at0 + i * a.si;
@@ -461,7 +451,7 @@ __device__ __forceinline__ void rm_chunk(const RmArgs& a, int L, const uint2* wf
 
 // Unit: 32 entries along the minor dimension by kMmaThreads / 32 majors, one per warp.
 template <int W, bool INT>
-__global__ void __launch_bounds__(kMmaThreads)
+__global__ void __launch_bounds__(kMmaThreads, 6)
 reduce_mma_kernel(BasisDev b, const __grid_constant__ RmArgs a) {
     extern __shared__ __align__(16) uint8_t dyn[];
     uint2* wf = (uint2*)dyn;
@@ -674,7 +664,7 @@ cudaError_t launch_reduce_kind(const BasisDev& b, const ReduceArgs& a, dim3 grid
 // The tensor-core reduction takes whole limbs per lane and three digits; other
 // word counts, wider primes and larger bases keep reduce_kernel.
 static bool mma_reducible(const BasisDev& b, const ReduceArgs& a) {
-    return !a.identity && b.L <= 64 && b.p_top < (1u << 24) && (a.W == 1 || a.W == 2 || a.W == 4 || a.W == 8) &&
+    return !a.identity && b.L <= 64 && b.p_top < (1u << 24) && b.p_low >= kMinPrime && (a.W == 1 || a.W == 2 || a.W == 4 || a.W == 8) &&
            ((uintptr_t)a.X & (a.W == 8 ? 15 : 7)) == 0;
 }
 
@@ -704,8 +694,9 @@ static cudaError_t launch_reduce_mma(const BasisDev& b, const ReduceArgs& a, Red
     return cudaGetLastError();
 }
 
-size_t reduce_image_bytes(int L, uint32_t p_top, int W) {
-    if (L > 64 || p_top >= (1u << 24)) return 0;
+size_t reduce_image_bytes(const std::vector<uint32_t>& p, int W) {
+    const int L = (int)p.size();
+    if (L > 64 || p[0] >= (1u << 24) || p[L - 1] < kMinPrime) return 0;
     return rm_frag(L, W == 1 ? 1 : W / 2) + 2 * (size_t)L * sizeof(uint4);
 }
 

@@ -59,11 +59,58 @@ __host__ __device__ inline bool xi_slot(int ks, int kap, int t, int* i, int* u) 
     return a < NQ;
 }
 
+// d = kMagic + a b: the sums start at kMagic, so that they are integers in their
+// low bits as they stand (integers in [2^23, 2^24) all along, exact)
+__device__ __forceinline__ void mma_f16_first(float (&d)[4], const uint32_t (&a)[4], const uint2& b) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%10, %10, %10, %10};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y), "f"(kMagic));
+}
 __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], const uint2& b) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
                  "{%0, %1, %2, %3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
+// The sums of N n8 tiles over KS steps for both m16 tiles; wf: the tiles' fragments of this lane
+template <int N, int KS>
+__device__ __forceinline__ void mma_tiles(float (&acc)[2][N][4], const uint32_t (&a)[2][KS][4], const uint2* wf) {
+#pragma unroll
+    for (int ks = 0; ks < KS; ks++) {
+#pragma unroll
+        for (int h = 0; h < N; h++) {
+            const uint2 b = wf[(h * KS + ks) * 32];
+            if (ks == 0) {
+                mma_f16_first(acc[0][h], a[0][ks], b);
+                mma_f16_first(acc[1][h], a[1][ks], b);
+            } else {
+                mma_f16(acc[0][h], a[0][ks], b);
+                mma_f16(acc[1][h], a[1][ks], b);
+            }
+        }
+    }
+}
+
+// v mod q, or that plus q, for v = S_0 + 2^8 S_1 + 2^16 S_2 + constants, from the sums as
+// they stand (kMagic too large each): the quotient in fp32, f_c (quot_const) holding
+// the constants' part of it and the biases', less 1/2 + 2^-5, and the remainder in
+// wrapping 32 bits, i_c (rem_const) holding the constants, the sums' biases and the
+// quotient's.  For q >= 2^22 the fp32 error is below 2^-5 (2^15 / q of the sum, whose
+// biases are 2^39.6, half a unit of f_c, at most 2^-7, and little of a quotient below
+// 2^14), so the result lies in [0, 1.07 q): min(y, y - q) ends it.
+constexpr uint32_t kMinPrime = 1u << 22;
+inline float quot_const(double c, float iq, uint32_t q) {
+    return (float)(c / q - 0.5 - 0x1p-5 - 12582912.0 * 65793.0 * (double)iq);
+}
+inline uint32_t rem_const(uint32_t c, uint32_t q) { return c - kMagicBits * 65793u + q * kMagicBits; }
+__device__ __forceinline__ float sums_quot(float s0, float s1, float s2, float iq, float f_c) {
+    return fmaf(fmaf(s2, 65536.f, fmaf(s1, 256.f, s0)), iq, f_c);
+}
+__device__ __forceinline__ uint32_t sums_rem(float s0, float s1, float s2, uint32_t q, uint32_t i_c, float f) {
+    const uint32_t y = __float_as_uint(s0) + (__float_as_uint(s1) << 8) + (__float_as_uint(s2) << 16) + i_c;
+    return y - __float_as_uint(f + kMagic) * q;
 }
 
 // two bytes, each in the low bits of 0x6400 (the fp16 value 1024 + byte), as byte - 128
