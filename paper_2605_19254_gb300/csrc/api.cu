@@ -270,7 +270,7 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
     size_t pc = 0;
     const size_t image = crt_image_bytes(b->crt, &pc), o_image = slot(image);
     size_t o_red[4];
-    for (int k = 0; k < 4; k++) o_red[k] = slot(reduce_image_bytes(L, p[0], 1 << k));
+    for (int k = 0; k < 4; k++) o_red[k] = slot(reduce_image_bytes(p, 1 << k));
     std::vector<uint8_t> host(off, 0);
     memcpy(&host[o_p], p.data(), 4 * L);
     memcpy(&host[o_mu], mu.data(), 8 * L);
@@ -284,7 +284,7 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
     memcpy(&host[o_mi], b->mi.data(), 4 * (size_t)L * ml);
     if (image) crt_image_make(b->crt, &host[o_image]);
     for (int k = 0; k < 4; k++)
-        if (reduce_image_bytes(L, p[0], 1 << k)) reduce_image_make(p.data(), L, 1 << k, &host[o_red[k]]);
+        if (reduce_image_bytes(p, 1 << k)) reduce_image_make(p.data(), L, 1 << k, &host[o_red[k]]);
     DeviceGuard g(ctx->device);
     cudaError_t e = cudaMalloc(&b->dev_blob, off);
     // A copy from pageable memory may return before its DMA lands, and kernels on
@@ -304,6 +304,7 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
     b->dev.pow32 = (const uint32_t*)(d + o_pow);
     for (int k = 0; k < 4; k++) b->dev.red[k] = d + o_red[k];
     b->dev.p_top = p[0];
+    b->dev.p_low = p[L - 1];
     b->crt.d_mi = (const uint32_t*)(d + o_mi);
     b->crt.d_m = (const uint32_t*)(d + o_m);
     b->crt.d_image = d + o_image;

@@ -29,7 +29,7 @@ struct BasisDev {
     const uint64_t* mu;       // [L] floor((2^64 - 1) / p_i), Barrett reduction
     const uint32_t* pow32;    // [L] 2^32 mod p_i
     const uint8_t* red[4];    // tables of the tensor-core reductions of entries of 1, 2, 4, 8 words (reduce_image)
-    uint32_t p_top;           // the largest prime
+    uint32_t p_top, p_low;    // the largest and the smallest prime
     int sms;                  // SMs of the device the tables are on
     const double* inv_p;      // [L] 1/p_i rounded to fp64 (Section 3.1 fast reduction)
     // Garner: for j < i, w[i*L + j] = p_j mod p_i with its Shoup companion
@@ -437,7 +437,7 @@ cudaError_t launch_gemm_limb_crt(smf_ctx* ctx, const BasisDev& b, const CrtHost&
 // where the per-prime constants lie in them; the reductions' tables for W words.
 size_t crt_image_bytes(const CrtHost& h, size_t* pc);
 void crt_image_make(const CrtHost& h, uint8_t* image);
-size_t reduce_image_bytes(int L, uint32_t p_top, int W);
+size_t reduce_image_bytes(const std::vector<uint32_t>& p, int W);
 void reduce_image_make(const uint32_t* p, int L, int W, uint8_t* image);
 
 // CRT reconstruction: Lagrange form with an fp32 correction, exact mixed-radix (Garner) fallback.
