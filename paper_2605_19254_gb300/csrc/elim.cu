@@ -524,10 +524,11 @@ cudaError_t elim_columns(smf_ctx* ctx, ElimBufs<T, L>& b, T* M, int64_t n, const
 //    columns are listed in increasing order (dcols[0 .. *ndef)), and the trailing
 //    columns are all of them, the panel's own too, followed by [c1, n).
 //
-// GB300, four 31-bit primes: n = 2003 8.1 ms (44 ms with a launch per column),
-// n = 5003 69 ms (210 ms by panels of 16 columns with two launches per column of
-// the panel).
+// GB300, four 31-bit primes: n = 2003 6.6 ms (44 ms with a launch per column; 8.1 ms
+// without the look-ahead of elim_blocked: 59 panels of 41 to 104 us and as many
+// passes of up to 169 us, one after the other).
 constexpr int kPanel = 32;
+constexpr int64_t kLookAhead = 2 << 20;  // words of a pass (about 20 us)
 
 // trailing column x of a panel: a deferred column, then [c1, n)
 __device__ __forceinline__ int64_t trail_col(int64_t x, int64_t nd, const int* __restrict__ dcols, int64_t c1) {
@@ -554,7 +555,7 @@ __global__ void bd_init_kernel(int64_t n, int* __restrict__ live, int* __restric
 constexpr int kTrailRows = 64, kTrailWords = 128;
 template <int L, PanelRed RED, int KT, bool LOC>
 __global__ void __launch_bounds__(256)
-bd_trail_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c0, int w, int64_t c1,
+bd_trail_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c0, int w, int64_t c1, int64_t ce,
                 const __grid_constant__ PanelMod<L> md, const int* __restrict__ live, const int* __restrict__ count,
                 const int* __restrict__ piv, const uint32_t* __restrict__ G, const int* __restrict__ flag,
                 const int* __restrict__ dcols, const int* __restrict__ ndef) {
@@ -564,8 +565,8 @@ bd_trail_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c0, int w, int64_t 
     pdl_wait();
     pdl_trigger();
     if (*flag) return;
-    const int64_t nd = LOC ? (int64_t)*ndef : 0;
-    const int64_t ncols = nd + (n - c1);
+    const int64_t nd = LOC && ndef ? (int64_t)*ndef : 0;
+    const int64_t ncols = nd + (ce - c1);
     const int nl = *count;
     const int64_t x0 = (int64_t)blockIdx.x * (kTrailWords / L);
     const int r0 = (int)blockIdx.y * kTrailRows;
@@ -607,16 +608,27 @@ bd_trail_kernel(uint32_t* __restrict__ M, int64_t n, int64_t c0, int w, int64_t 
     }
 }
 
-template <int L, PanelRed RED, bool LOC>
-cudaError_t launch_trail(int gw, uint32_t* M, int64_t n, int64_t c0, int w, int64_t c1, int64_t cols, int64_t rows,
-                         const PanelMod<L>& md, const int* live, const int* count, const int* piv, const uint32_t* G,
-                         const int* flag, const int* dcols, const int* ndef, cudaStream_t s) {
+// The trailing columns [c1, ce) of a panel, and the deferred ones when ndef is given.
+// dependent: launched while the kernel before it on the stream still runs (not
+// where an event comes between).
+template <int L, bool LOC>
+cudaError_t launch_trail(const PanelArgs<L>& a, int64_t c1, int64_t ce, const int* ndef, int64_t rows, bool dependent,
+                         cudaStream_t s) {
+    const int64_t cols = ce - c1 + (ndef ? c1 : 0);  // (deferred columns lie before c1)
     const dim3 grid((unsigned)((cols + kTrailWords / L - 1) / (kTrailWords / L)),
                     (unsigned)((rows + kTrailRows - 1) / kTrailRows));
-    return gw > 16 ? launch_pdl(bd_trail_kernel<L, RED, 32, LOC>, grid, dim3(256), 0, s, M, n, c0, w, c1, md, live, count,
-                                piv, G, flag, dcols, ndef)
-                   : launch_pdl(bd_trail_kernel<L, RED, 16, LOC>, grid, dim3(256), 0, s, M, n, c0, w, c1, md, live, count,
-                                piv, G, flag, dcols, ndef);
+    auto go = [&](auto kernel) {
+        if (dependent)
+            return launch_pdl(kernel, grid, dim3(256), 0, s, a.M, a.n, a.c0, a.w, c1, ce, a.md, (const int*)a.live_out,
+                              (const int*)a.count_out, (const int*)a.piv, (const uint32_t*)a.G, (const int*)a.flag,
+                              (const int*)a.dcols, ndef);
+        kernel<<<grid, 256, 0, s>>>(a.M, a.n, a.c0, a.w, c1, ce, a.md, a.live_out, a.count_out, a.piv, a.G, a.flag,
+                                    a.dcols, ndef);
+        return cudaGetLastError();
+    };
+    if (panel_red(a.md) == PanelRed::kNarrow)
+        return a.gw > 16 ? go(bd_trail_kernel<L, PanelRed::kNarrow, 32, LOC>) : go(bd_trail_kernel<L, PanelRed::kNarrow, 16, LOC>);
+    return a.gw > 16 ? go(bd_trail_kernel<L, PanelRed::kWide, 32, LOC>) : go(bd_trail_kernel<L, PanelRed::kWide, 16, LOC>);
 }
 
 // An elimination by panels on the stream: what it leaves on the device.
@@ -637,20 +649,23 @@ cudaError_t elim_blocked(smf_ctx* ctx, uint32_t* M, int64_t n, const Lanes<uint3
     cudaError_t e;
     PanelArgs<L> a{};
     for (int l = 0; l < L; l++) panel_mod(a.md, l, md.m[l < md.n ? l : 0], md.q[l < md.n ? l : 0]);
-    const PanelRed red = panel_red(a.md);
     const int pw = panel_width(n, L, kPanel), gw = pw > 16 ? 32 : 16;
-    // scratch: G, ybuf, then [piv n | flag | det 2L] read back in one copy, live lists, counts, deferred columns
-    const size_t words = (size_t)n * L * gw + panel_scratch(pw * L) + (size_t)n + 1 + 2 * L + 2 * (size_t)n + 2 + (size_t)n + 1;
+    const int64_t panels = (n + pw - 1) / pw;
+    // scratch: G (two, see below), ybuf, then [piv n | flag | det 2L] read back in one copy, live lists, counts,
+    // deferred columns and their number before each panel
+    const size_t gwords = (size_t)n * L * gw;
+    const size_t words = 2 * gwords + panel_scratch(pw * L) + (size_t)n + 1 + 2 * L + 2 * (size_t)n + 2 + (size_t)n +
+                         (size_t)panels + 1;
     if ((e = out->buf.alloc(ctx, sizeof(uint32_t) * words, s))) return e;
     uint32_t* G = (uint32_t*)out->buf.p;
-    uint32_t* ybuf = G + (size_t)n * L * gw;
+    uint32_t* ybuf = G + 2 * gwords;
     int* piv = (int*)(ybuf + panel_scratch(pw * L));
     int* flag = piv + n;
     uint32_t* det = (uint32_t*)flag + 1;
     int* live[2] = {(int*)det + 2 * L, (int*)det + 2 * L + n};
     int* count = live[1] + n;
-    int* ndef = count + 2;
-    int* dcols = ndef + 1;
+    int* dcols = count + 2;
+    int* ndef = dcols + n;
     bd_init_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, live[0], count, flag, ndef, det, 2 * L);
     if ((e = cudaGetLastError())) return e;
     a.M = M;
@@ -658,31 +673,59 @@ cudaError_t elim_blocked(smf_ctx* ctx, uint32_t* M, int64_t n, const Lanes<uint3
     a.ybuf = ybuf;
     a.piv = piv;
     a.flag = flag;
-    a.G = G;
     a.gw = gw;
     a.det = det;
     a.dcols = dcols;
-    a.ndef = ndef;
     int k = 0;
-    for (int64_t c0 = 0; c0 < n; c0 += pw, k ^= 1) {
-        const int64_t c1 = std::min<int64_t>(n, c0 + pw);
-        a.c0 = c0;
-        a.w = (int)(c1 - c0);
-        a.live = live[k];
-        a.count = count + k;
-        a.live_out = live[k ^ 1];
-        a.count_out = count + (k ^ 1);
-        if ((e = launch_panel<L, LOC ? PanelKind::kLocal : PanelKind::kDet>(a, n, s))) return e;
-        if (!LOC && c1 >= n) continue;
-        // a determinant leaves n - c1 rows; a local form's rows and deferred columns are known on the device
-        const int64_t cols = LOC ? n : n - c1, rows = LOC ? n : n - c1;
-        e = red == PanelRed::kNarrow
-                ? launch_trail<L, PanelRed::kNarrow, LOC>(gw, M, n, c0, a.w, c1, cols, rows, a.md, a.live_out, a.count_out,
-                                                          piv, G, flag, dcols, ndef, s)
-                : launch_trail<L, PanelRed::kWide, LOC>(gw, M, n, c0, a.w, c1, cols, rows, a.md, a.live_out, a.count_out,
-                                                        piv, G, flag, dcols, ndef, s);
-        if (e) return e;
-    }
+    // Look-ahead: the columns of the next panel first, then the next panel (16
+    // SMs, a serial chain) beside the pass over the rest, on the context's side
+    // stream.  What the two share is apart: M's columns; G and the live lists, two
+    // of each; the deferred columns, whose number is kept for each panel.  The rest
+    // is done before anything touches its columns or the buffers it reads: the next
+    // panel's own columns wait for it.  Where the rest is short the events cost more
+    // than they hide: below kLookAhead words everything stays on one stream.
+    bool side = false;  // a pass on the side stream that s has not waited for
+    auto join = [&] {
+        if (!side) return cudaSuccess;
+        side = false;
+        return cudaStreamWaitEvent(s, ctx->ev_join, 0);
+    };
+    auto enqueue = [&]() -> cudaError_t {
+        for (int64_t c0 = 0, i = 0; c0 < n; c0 += pw, k ^= 1, i++) {
+            const int64_t c1 = std::min<int64_t>(n, c0 + pw), c2 = std::min<int64_t>(n, c1 + pw);
+            a.c0 = c0;
+            a.w = (int)(c1 - c0);
+            a.live = live[k];
+            a.count = count + k;
+            a.live_out = live[k ^ 1];
+            a.count_out = count + (k ^ 1);
+            a.G = G + (i & 1) * gwords;
+            a.ndef = ndef + i;
+            a.ndef_out = ndef + i + 1;
+            if ((e = launch_panel<L, LOC ? PanelKind::kLocal : PanelKind::kDet>(a, n, s))) return e;
+            const bool dependent = !side;
+            if ((e = join())) return e;
+            if (!LOC && c1 >= n) continue;
+            // a determinant leaves n - c1 rows; a local form's rows and deferred columns are known on the device
+            const int64_t rows = LOC ? n : n - c1;
+            const int* nd = LOC ? a.ndef_out : nullptr;
+            if ((n - c1) * (n - c2) * L < kLookAhead) {
+                if ((e = launch_trail<L, LOC>(a, c1, n, nd, rows, dependent, s))) return e;
+                continue;
+            }
+            if ((e = launch_trail<L, LOC>(a, c1, c2, nullptr, rows, dependent, s)) || (e = cudaEventRecord(ctx->ev_fork, s)) ||
+                (e = cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0)))
+                return e;
+            side = true;
+            e = launch_trail<L, LOC>(a, c2, n, nd, rows, false, ctx->aux);
+            const cudaError_t e2 = cudaEventRecord(ctx->ev_join, ctx->aux);
+            if (e || e2) return e ? e : e2;
+        }
+        return cudaSuccess;
+    };
+    e = enqueue();
+    const cudaError_t ej = join();  // (the scratch goes back on s)
+    if (e || ej) return e ? e : ej;
     out->piv = piv;
     out->flag = flag;
     out->det = det;

@@ -124,7 +124,8 @@ struct PanelArgs {
     int gw;
     uint32_t* det;        // [2 L] the pivots' product as a fraction, numerators and denominators (kDet)
     int* dcols;           // columns without a pivot, ascending, and their count (LOC)
-    int* ndef;
+    const int* ndef;      // the latter before the panel and after it
+    int* ndef_out;
 };
 
 #ifdef __CUDACC__
@@ -627,7 +628,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) panel_kernel(const __grid_co
             int d = *a.ndef;
             for (int j = 0; j < w; j++)
                 if (!got[j]) a.dcols[d++] = (int)(a.c0 + j);
-            *a.ndef = d;
+            *a.ndef_out = d;
         }
         __syncthreads();
         const int base = s_base[rank];
