@@ -180,10 +180,10 @@ convert_kernel(const __grid_constant__ ConvConst<LMAX> v, const int32_t* __restr
 // 2^(8u) M_i, lane 4g + t owns 2 NT consecutive ones (NT / 2 limbs), and the carry
 // into the next lane's limbs is passed by a shuffle.  The limbs go through shared
 // memory, so that the words are stored in order.
-// What bounds it is instruction issue; one limb-sum thread per entry took 1815
-// instructions with 23 primes.  The product of 1009 x 1009 by 1009 x 100 with 34
-// primes (reduction and CRT both so) went from 303 to 218 us, a batch of 512 products
-// from 8.02 to 7.15 ms, one of 64 x 64 by 64 x 16 from 39 to 26 us.
+// 1300 thread instructions an entry with 23 primes (1815 as limb sums, one thread per
+// entry) at half the issue slots: 18.6M entries 1.51 -> 1.47 ms.  The product of 1009 x 1009 by
+// 1009 x 100 with 34 primes (reduction and CRT both so) went from 303 to 216 us, one
+// of 64 x 64 by 64 x 16 from 38 to 25 us.
 template <int LMAX>
 struct CrtMma {
     static constexpr int NT = (3 * LMAX / 4 + 3) / 4 * 2;  // n8 tiles
@@ -422,12 +422,13 @@ cudaError_t launch_crt_mma_grouped(const CrtHost& h, const CrtItem* items, int n
 // hold two targets of a lane.  A residue is then
 //   v = S_0 + 2^8 S_1 + 2^16 S_2 + C_j - alpha (M mod q_j)  mod q_j:
 // sums_quot and sums_rem have the arithmetic.
-// 23 -> 23 primes, 1M entries: 159 -> 79 us (28 us of HBM traffic); bound by issue.
+// 23 -> 23 primes, 1M entries: 159 -> 73 us (28 us of HBM traffic); half the issue
+// slots are busy, the chunks' latencies bound it.
 template <int LMAX>
 struct ConvMma {
     const uint4* pc;          // the source's constants (device)
     XiExact xi;
-    uint32_t w[LMAX * LMAX];  // w_ij at j LMAX + i
+    alignas(16) uint32_t w[LMAX * LMAX];  // w_ij at j LMAX + i (0 for i >= L)
     uint4 ti[LMAX];           // q_j, M mod q_j, rem_const of C_j
     float4 tf[LMAX];          // 1 / q_j, (M mod q_j) / q_j, quot_const of C_j
     int LQ;
@@ -456,19 +457,23 @@ convert_mma_kernel(const __grid_constant__ ConvMma<LMAX> v, const int32_t* __res
     for (int x = threadIdx.x; x < (LQ + 7) / 8 * 3 * KS * 32; x += kMmaThreads) wf[x] = make_uint2(0, 0);
     __syncthreads();
     // the three digits of w_ij 2^(8u) mod q_j to where the fragments have them (xi_slot)
-    for (int x = threadIdx.x; x < LQ * LMAX * 3; x += kMmaThreads) {
-        const int i = x % LMAX, u = x / LMAX % 3, j = x / (3 * LMAX);
-        if (i >= L) continue;
-        const int a = i >> 2, pr = u < 2 ? a : LMAX / 4 + a / 2, kap = 2 * (pr & 1) + (u < 2 ? u : a & 1);
-        // to within half of q_j and a little (the quotient is below 2^16)
-        const uint32_t w = v.w[j * LMAX + i], q = ti[j].x;
-        const int quo = __float2int_rn((float)w * ((float)(1 << 8 * u) * tf[j].x));
-        int32_t r = (int32_t)((w << 8 * u) - (uint32_t)quo * q);
+    // (four w at a time: loads of the parameter bank at an address per lane take turns)
+    for (int x = threadIdx.x; x < LQ * (LMAX / 4) * 3; x += kMmaThreads) {
+        const int a = x % (LMAX / 4), u = x / (LMAX / 4) % 3, j = x / (LMAX / 4 * 3);
+        const int pr = u < 2 ? a : LMAX / 4 + a / 2, kap = 2 * (pr & 1) + (u < 2 ? u : a & 1);
+        const uint4 w4 = *(const uint4*)(v.w + j * LMAX + 4 * a);
+        const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w}, q = ti[j].x;
+        const float s = (float)(1 << 8 * u) * tf[j].x;
 #pragma unroll
-        for (int dig = 0; dig < 3; dig++) {
-            const int c6 = (j >> 2 & 1) * 3 + dig, nt = (j >> 3) * 3 + c6 / 2, ln = (2 * (j & 3) + (c6 & 1)) * 4 + (i & 3);
-            ((__half*)wf)[((nt * KS + pr / 2) * 32 + ln) * 4 + kap] = __int2half_rn(dig < 2 ? ((r + 128) & 255) - 128 : r);
-            r = (r + 128) >> 8;
+        for (int z = 0; z < 4; z++) {  // prime 4a + z; w = 0 beyond L
+            // to within half of q_j and a little (the quotient is below 2^16)
+            int32_t r = (int32_t)((w[z] << 8 * u) - (uint32_t)__float2int_rn((float)w[z] * s) * q);
+#pragma unroll
+            for (int dig = 0; dig < 3; dig++) {
+                const int c6 = (j >> 2 & 1) * 3 + dig, nt = (j >> 3) * 3 + c6 / 2, ln = (2 * (j & 3) + (c6 & 1)) * 4 + z;
+                ((__half*)wf)[((nt * KS + pr / 2) * 32 + ln) * 4 + kap] = __int2half_rn(dig < 2 ? ((r + 128) & 255) - 128 : r);
+                r = (r + 128) >> 8;
+            }
         }
     }
     __syncthreads();

@@ -300,7 +300,7 @@ struct ReduceItem {       // one operand of a grouped digit split or transposed 
     int W, t;
     int bits;             // declared bound of the entries (checked; >= 64 W - 1: not checked)
     int64_t base;
-    // digit split: floor(e / cols) = (umulhi(e, div_m) + e) >> div_s for e < 2^32
+    // digit split: floor(e / (groups of 8 in a row)) = (umulhi(e, div_m) + e) >> div_s for e < 2^32
     // (division by an invariant integer, Granlund and Montgomery; set by split_units)
     uint32_t div_m;
     int div_s;
@@ -332,7 +332,7 @@ __device__ __forceinline__ const Item* find_item(const Item* items, int n, int64
 }
 #endif
 // Work units of one item: transposed reduce of B (32 rows by 16 columns),
-// digit split of a shared-digit A (2048 entries), CRT (128 entries).
+// digit split of a shared-digit A (256 groups of 8 entries of a row), CRT (128 entries).
 int64_t reduce_t_units(int64_t rows, int64_t cols);
 bool reduce_t_groupable(const BasisDev& b, const ReduceArgs& a);  // W in {1, 2, 4, 8}, at most 64 primes below 2^24
 int64_t split_units(int64_t rows, int64_t cols, uint32_t* div_m, int* div_s);

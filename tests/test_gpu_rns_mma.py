@@ -147,3 +147,24 @@ def test_declared_bound(ctx, W, bits):
         with pytest.raises(smf.SmfError) as e:
             ctx.status_sync()
         assert e.value.code == smf.SMF_E_BOUND
+
+
+@pytest.mark.parametrize("a_bits", [1, 7, 15, 20])  # one, two and three digits
+@pytest.mark.parametrize("k,pad,shift", [(1, 0, 0), (7, 0, 0), (8, 0, 0), (8, 0, 1), (9, 1, 0), (40, 8, 0), (65, 0, 0)])
+def test_grouped_split(ctx, a_bits, k, pad, shift):
+    m, n = 35, 6
+    _, va = _entries(m, k, 0, 1, a_bits + k, a_bits)
+    buf = torch.zeros(m * (k + pad) + shift, dtype=torch.int64, device="cuda")
+    A = buf[shift:].view(m, k + pad, 1)[:, :k]
+    A.copy_(torch.tensor(va, dtype=torch.int64).view(m, k, 1))
+    B, vb = _entries(k, n, 0, 2, 3)
+    C = torch.zeros((m, n, 3), dtype=torch.int64, device="cuda")
+    ctx.rns_matmul_grouped([A], [B], [C], a_bits=a_bits)
+    ctx.status_sync()
+    assert _ints(C) == [sum(va[i * k + t] * vb[t * n + j] for t in range(k)) for i in range(m) for j in range(n)]
+    from paper_2605_19254_gb300 import smf
+    A[m - 1, k - 1, 0] = (1 << a_bits) + 1
+    ctx.rns_matmul_grouped([A], [B], [C], a_bits=a_bits)
+    with pytest.raises(smf.SmfError) as e:
+        ctx.status_sync()
+    assert e.value.code == smf.SMF_E_BOUND
