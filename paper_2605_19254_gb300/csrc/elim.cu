@@ -684,11 +684,24 @@ cudaError_t elim_blocked(smf_ctx* ctx, uint32_t* M, int64_t n, const Lanes<uint3
     // is done before anything touches its columns or the buffers it reads: the next
     // panel's own columns wait for it.  Where the rest is short the events cost more
     // than they hide: below kLookAhead words everything stays on one stream.
+    struct Events {  // the call's own: calls on other streams may share the context
+        cudaEvent_t fork = nullptr, join = nullptr;
+        cudaError_t make() {
+            cudaError_t e = cudaSuccess;
+            if (!fork) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+            if (!e && !join) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+            return e;
+        }
+        ~Events() {
+            if (fork) cudaEventDestroy(fork);
+            if (join) cudaEventDestroy(join);
+        }
+    } ev;
     bool side = false;  // a pass on the side stream that s has not waited for
     auto join = [&] {
         if (!side) return cudaSuccess;
         side = false;
-        return cudaStreamWaitEvent(s, ctx->ev_join, 0);
+        return cudaStreamWaitEvent(s, ev.join, 0);
     };
     auto enqueue = [&]() -> cudaError_t {
         for (int64_t c0 = 0, i = 0; c0 < n; c0 += pw, k ^= 1, i++) {
@@ -713,12 +726,12 @@ cudaError_t elim_blocked(smf_ctx* ctx, uint32_t* M, int64_t n, const Lanes<uint3
                 if ((e = launch_trail<L, LOC>(a, c1, n, nd, rows, dependent, s))) return e;
                 continue;
             }
-            if ((e = launch_trail<L, LOC>(a, c1, c2, nullptr, rows, dependent, s)) || (e = cudaEventRecord(ctx->ev_fork, s)) ||
-                (e = cudaStreamWaitEvent(ctx->aux, ctx->ev_fork, 0)))
+            if ((e = ev.make()) || (e = launch_trail<L, LOC>(a, c1, c2, nullptr, rows, dependent, s)) ||
+                (e = cudaEventRecord(ev.fork, s)) || (e = cudaStreamWaitEvent(ctx->aux, ev.fork, 0)))
                 return e;
             side = true;
             e = launch_trail<L, LOC>(a, c2, n, nd, rows, false, ctx->aux);
-            const cudaError_t e2 = cudaEventRecord(ctx->ev_join, ctx->aux);
+            const cudaError_t e2 = cudaEventRecord(ev.join, ctx->aux);
             if (e || e2) return e ? e : e2;
         }
         return cudaSuccess;
