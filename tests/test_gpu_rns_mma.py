@@ -88,6 +88,7 @@ def _entries(rows, cols, pad, W, seed, bits=None):
     b = 64 * W - 1 if bits is None else bits
     top = (1 << b) - (bits is None)
     v = [0, -1, 1, top, -(1 << b), 1 << (b // 2), -(1 << (b // 2)), 255, -256]
+    v = [x for x in v if -(1 << b) <= x <= top]
     rng = np.random.default_rng(seed)
     while len(v) < rows * cols:
         v.append(int.from_bytes(rng.bytes(8 * W + 8), "little") % ((1 << (b + 1)) - 1) - (1 << b) + 1)
