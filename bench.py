@@ -512,7 +512,7 @@ def run_base_convert(dev, local, stream, flush, steps, hbm_peak):
     out = {"workload": f"{count} entries (4096 x 256), {len(src.primes)} -> {len(dst.primes)} primes below 2^24",
            "ms": ms, "entries_per_s": count / (ms * 1e-3), "algorithmic_bytes": nbytes,
            "hbm_gbs": nbytes / (ms * 1e-3) / 1e9, "hbm_frac": nbytes / (ms * 1e-3) / 1e9 / hbm_peak if hbm_peak else None,
-           "bound": "integer issue", "kernel": "convert_kernel<24>", "steps": steps}
+           "bound": "integer issue", "kernel": "convert_mma_kernel<24>", "steps": steps}
     src.destroy()
     dst.destroy()
     ctx.destroy()
