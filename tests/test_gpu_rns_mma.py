@@ -151,12 +151,11 @@ def test_declared_bound(ctx, W, bits):
 
 
 @pytest.mark.parametrize("a_bits", [1, 7, 15, 20])  # one, two and three digits
-@pytest.mark.parametrize("k,pad,shift", [(1, 0, 0), (7, 0, 0), (8, 0, 0), (8, 0, 1), (9, 1, 0), (40, 8, 0), (65, 0, 0)])
-def test_grouped_split(ctx, a_bits, k, pad, shift):
+@pytest.mark.parametrize("k,pad", [(1, 0), (7, 0), (8, 0), (8, 1), (9, 1), (40, 8), (65, 0)])  # (odd row lengths: 8-byte aligned rows)
+def test_grouped_split(ctx, a_bits, k, pad):
     m, n = 35, 6
     _, va = _entries(m, k, 0, 1, a_bits + k, a_bits)
-    buf = torch.zeros(m * (k + pad) + shift, dtype=torch.int64, device="cuda")
-    A = buf[shift:].view(m, k + pad, 1)[:, :k]
+    A = torch.zeros((m, k + pad, 1), dtype=torch.int64, device="cuda")[:, :k]
     A.copy_(torch.tensor(va, dtype=torch.int64).view(m, k, 1))
     B, vb = _entries(k, n, 0, 2, 3)
     C = torch.zeros((m, n, 3), dtype=torch.int64, device="cuda")
