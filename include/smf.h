@@ -443,7 +443,9 @@ int smf_smith_form(smf_ctx* ctx, const smf_bigmat* A, uint64_t seed, uint32_t* l
  * prime, every other unused row subtracts its multiple; det = sign of the
  * pivot permutation times the pivots.  A column with no such row sends the
  * call back to one prime at a time.  Primes below 2^31 run by panels of up to
- * 32 columns (smf_set_elim_panels), with pivots from any rows.
+ * 32 columns (smf_set_elim_panels), with pivots from any rows, in groups of at
+ * most four (two or one where the panels of more would be too narrow, from about
+ * n = 10,700 on).
  * A: square, single-word entries, host or device.  det: host, count values
  * in [0, q_i).  Synchronous; allocates its
  * scratch (about n^2 (4 or 8) bytes per prime).  Errors: SMF_E_INVALID (a q_i
@@ -460,7 +462,8 @@ int smf_det_mod(smf_ctx* ctx, const smf_bigmat* A, const uint64_t* q, int32_t co
  * rows and deferred columns left: elimination over Z/(q^e) with unit pivots,
  * whose leftover block is divisible by q, is divided by q and is reduced
  * again over Z/(q^(e-1)).  Prime powers below 2^31 run by panels of up to 32
- * columns (smf_set_elim_panels), with pivots from any rows.
+ * columns (smf_set_elim_panels), with pivots from any rows, in groups as
+ * smf_det_mod's.
  * A: square, single-word entries, host or device.
  * q_i^e_i < 2^62, count <= 16.  Synchronous.  Errors: SMF_E_INVALID,
  * SMF_E_NOMEM, SMF_E_CUDA. */

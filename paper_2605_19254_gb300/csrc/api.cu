@@ -1156,10 +1156,10 @@ struct InverseLayout {
 };
 
 // By panels: any odd p when one panel holds the matrix; larger matrices need
-// the limb product of three-digit residues.
+// the limb product of three-digit residues, and a panel that fits.
 bool inverse_panels(const smf_ctx* ctx, int64_t n, uint32_t p) {
     if ((p & 1) == 0) return false;
-    return n <= kInvSingle || (ctx->form == SMF_FORM_INT8LIMB && digits_for(p / 2) <= 3);
+    return n <= kInvSingle || (ctx->form == SMF_FORM_INT8LIMB && digits_for(p / 2) <= 3 && inv_sub_width(n) > 0);
 }
 
 // The workspace does not know p: it holds the larger of the two forms (their
@@ -1185,10 +1185,17 @@ InverseLayout inverse_layout(const smf_ctx* ctx, int64_t n) {
         Lw.S = slot((size_t)4 * n * w);
         Lw.Mp = slot((size_t)4 * n * w);
         Lw.C = slot((size_t)4 * n * n);
-        // the largest product plan over the panels (three-digit residues): whole ones and the last
+        // the largest product plan over the panels (three-digit residues), whole ones and the last, and
+        // over the narrower panels within them
+        const int64_t sw = inv_sub_width(n);
         for (const int64_t b : {w, n % w ? n % w : w}) {
             const GemmPlan g = plan_limb(1, n, n - b, b, false, 1u << 23, 1u << 23, ctx->num_sms);
             Lw.gemm_bytes = std::max(Lw.gemm_bytes, g.bytes);
+            if (sw == 0 || sw >= b) continue;
+            for (const int64_t v : {sw, b % sw ? b % sw : sw}) {
+                const GemmPlan h = plan_limb(1, n, b - v, v, false, 1u << 23, 1u << 23, ctx->num_sms);
+                Lw.gemm_bytes = std::max(Lw.gemm_bytes, h.bytes);
+            }
         }
         Lw.gemm = slot(Lw.gemm_bytes);
         end = std::max(end, off);
@@ -1894,15 +1901,29 @@ int smf_inverse_mod_p(smf_ctx* ctx, const smf_basis* p_basis, const smf_bigmat* 
     const uint64_t h = p / 2;
     SMF_CU(ctx, cudaMemsetAsync(flag, 0, sizeof(int), s));
     SMF_CU(ctx, cudaMemsetAsync(rowcol, 0xFF, sizeof(int) * 2 * (size_t)n, s));
-    const int64_t pw = inv_panel_width(n);
+    const int64_t pw = inv_panel_width(n), sw = inv_sub_width(n);
+    // M's columns from b0, bw of them: the b from c0 have their transform in S, the others take it
+    auto apply = [&](int64_t b0, int64_t bw, int64_t c0, int64_t b) -> int {
+        SMF_CU(ctx, launch_inv_gather(Mn, n, b0, bw, c0, (int)b, piv, Mp, flag, s));
+        const int r = run_residue_gemm_i32(ctx, p_basis, S, n * b, Mp, Cb, n, bw - b, b, h, h, w + Lw.gemm, Lw.gemm_bytes, s);
+        if (r) return r;
+        SMF_CU(ctx, launch_inv_update(Mn, n, b0, bw, c0, (int)b, rowcol, Cb, p, s));
+        return SMF_OK;
+    };
     for (int64_t c0 = 0; c0 < n; c0 += pw) {
-        const int64_t b = std::min<int64_t>(pw, n - c0), R = n - b;
-        SMF_CU(ctx, launch_inv_panel(Mn, n, c0, (int)b, p, rowcol, piv, R ? S : nullptr, w + Lw.scratch, flag, ctx->d_status, s));
-        if (R == 0) break;
-        SMF_CU(ctx, launch_inv_gather(Mn, n, c0, (int)b, piv, Mp, flag, s));
-        if ((st = run_residue_gemm_i32(ctx, p_basis, S, n * b, Mp, Cb, n, R, b, h, h, w + Lw.gemm, Lw.gemm_bytes, s)))
-            return st;
-        SMF_CU(ctx, launch_inv_update(Mn, n, c0, (int)b, rowcol, Cb, p, s));
+        const int64_t b = std::min<int64_t>(pw, n - c0);
+        if (b <= sw) {
+            SMF_CU(ctx, launch_inv_panel(Mn, n, c0, (int)b, p, rowcol, piv, b < n ? S : nullptr, w + Lw.scratch, flag,
+                                         ctx->d_status, s));
+        } else {
+            for (int64_t c = c0; c < c0 + b; c += sw) {
+                const int64_t v = std::min<int64_t>(sw, c0 + b - c);
+                SMF_CU(ctx, launch_inv_panel(Mn, n, c, (int)v, p, rowcol, piv, S, w + Lw.scratch, flag, ctx->d_status, s));
+                if ((st = apply(c0, b, c, v))) return st;
+            }
+            SMF_CU(ctx, cudaMemcpy2DAsync(S, 4 * b, Mn + c0, 4 * n, 4 * b, n, cudaMemcpyDeviceToDevice, s));
+        }
+        if (b < n && (st = apply(0, n, c0, b))) return st;
     }
     SMF_CU(ctx, launch_inv_place(Mn, n, piv, rowcol, A_inv, flag, s));
     return SMF_OK;

@@ -530,6 +530,12 @@ cudaError_t elim_columns(smf_ctx* ctx, ElimBufs<T, L>& b, T* M, int64_t n, const
 constexpr int kPanel = 32;
 constexpr int64_t kLookAhead = 2 << 20;  // words of a pass (about 20 us)
 
+// 32-bit entries go by panels from the context's threshold up to the largest
+// matrix of which one column fits the cluster.
+bool by_panels(const smf_ctx* ctx, int64_t n, int L) {
+    return n >= ctx->elim_panel_min_n && panel_width(n, L, kPanel) > 0;
+}
+
 // trailing column x of a panel: a deferred column, then [c1, n)
 __device__ __forceinline__ int64_t trail_col(int64_t x, int64_t nd, const int* __restrict__ dcols, int64_t c1) {
     return x < nd ? dcols[x] : c1 + (x - nd);
@@ -833,13 +839,12 @@ local_small_kernel(const uint32_t* __restrict__ M, int64_t n, const int* __restr
 }
 
 // The column loop of a local form (every column but k stays current), by
-// panels when the entries are 32-bit and the matrix has at least
-// ctx->elim_panel_min_n columns.
+// panels when the entries are 32-bit (by_panels).
 template <typename T, int L>
 cudaError_t elim_local(smf_ctx* ctx, ElimBufs<T, L>& b, T* M, int64_t n, const Lanes<T, L>& md,
                        std::vector<int64_t>* pivrow, std::vector<T>* pivval, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
-        if (n >= ctx->elim_panel_min_n) {
+        if (by_panels(ctx, n, L)) {
             Blocked r;
             const cudaError_t e = elim_blocked<L, true>(ctx, M, n, md, &r, s);
             return e ? e : read_blocked<L>(r, n, pivrow, nullptr, nullptr, s);
@@ -884,7 +889,7 @@ int det_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const uint
     if constexpr (sizeof(T) == 4) {
         // 31-bit primes: by panels.  A column without a joint unit pivot sends
         // several primes back to one at a time (below); with one prime det = 0
-        if (n >= ctx->elim_panel_min_n) {
+        if (by_panels(ctx, n, L)) {
             bool no_pivot = false;
             uint32_t dets[2 * L];
             Blocked r;
@@ -1015,7 +1020,7 @@ int local_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const ui
         if ((ce = cudaGetLastError())) return elim_fail(ctx, "smith_local", ce);
         bool done = false;
         if constexpr (sizeof(T) == 4) {
-            if (n >= ctx->elim_panel_min_n) {  // by panels, and the block left at once when it is small
+            if (by_panels(ctx, n, L)) {  // by panels, and the block left at once when it is small
                 Blocked r;
                 StreamBuf ob;
                 constexpr int words = L * kSmallLevels + 1;
@@ -1081,21 +1086,35 @@ int local_lanes(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const ui
     return SMF_OK;
 }
 
+// How many 32-bit moduli one elimination of an n x n matrix takes at most.  By
+// panels the moduli share the cluster's shared memory: with more of them a large
+// matrix's panels get narrower, and a pass over the rest (which multiplies by 16
+// or 32 columns) comes more often.  Four 31-bit determinants, four at a time /
+// one at a time (start of the panels' 16 and 8 columns with four moduli: n = 5345
+// and 10705):
+//   n = 8009 0.243 / 0.248 s, 10007 0.461 / 0.458, 12007 1.54 / 0.76, 20501 14.9 / 3.6
+// (two at a time, panels of 16 columns: 0.80 and 3.8 s at the last two).
+int elim_group(const smf_ctx* ctx, int64_t n) {
+    if (!by_panels(ctx, n, 1)) return 4;  // by columns
+    return panel_width(n, 4, kPanel) >= 16 ? 4 : panel_width(n, 2, kPanel) >= kPanel ? 2 : 1;
+}
+
 template <typename T>
 int det_dispatch(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const uint64_t* q, int nq, uint64_t* det,
                  cudaStream_t s) {
-    if (nq <= 1) return det_lanes<T, 1>(ctx, A, lda, n, q, nq, det, s);
-    if (nq <= 2) return det_lanes<T, 2>(ctx, A, lda, n, q, nq, det, s);
-    if (nq <= 4) return det_lanes<T, 4>(ctx, A, lda, n, q, nq, det, s);
-    for (int i = 0; i < nq; i += 4) {  // groups of four
-        const int st = det_lanes<T, 4>(ctx, A, lda, n, q + i, std::min(4, nq - i), det + i, s);
+    const int most = sizeof(T) == 4 ? elim_group(ctx, n) : 4;
+    for (int i = 0; i < nq; i += most) {
+        const int k = std::min(most, nq - i);
+        const int st = k == 1   ? det_lanes<T, 1>(ctx, A, lda, n, q + i, k, det + i, s)
+                       : k == 2 ? det_lanes<T, 2>(ctx, A, lda, n, q + i, k, det + i, s)
+                                : det_lanes<T, 4>(ctx, A, lda, n, q + i, k, det + i, s);
         if (st) return st;
     }
     return SMF_OK;
 }
 
-// Prime powers below 2^31 in lockstep groups of four 32-bit lanes (16-byte
-// entries, one column loop per group), wider ones one at a time in 64-bit words.
+// Prime powers below 2^31 in lockstep groups of up to four 32-bit lanes
+// (elim_group), wider ones one at a time in 64-bit words.
 // A joint loop of all eleven prime powers of the n = 5003 test in 64-bit lanes
 // was slower than one at a time (4.35 s against 1.94 s): every update moved 88
 // bytes per entry.
@@ -1113,8 +1132,9 @@ int local_dispatch(smf_ctx* ctx, const int64_t* A, int64_t lda, int64_t n, const
         if (st) return st;
         (*counts)[l] = std::move(one[0]);
     }
-    for (size_t g = 0; g < narrow.size(); g += 4) {
-        const int k = (int)std::min<size_t>(4, narrow.size() - g);
+    const size_t most = (size_t)elim_group(ctx, n);
+    for (size_t g = 0; g < narrow.size(); g += most) {
+        const int k = (int)std::min(most, narrow.size() - g);
         std::vector<uint64_t> qg;
         std::vector<int> eg;
         for (int t = 0; t < k; t++) {

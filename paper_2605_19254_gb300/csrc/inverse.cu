@@ -140,7 +140,12 @@ __global__ void __launch_bounds__(kElimThreads) gj_elim_kernel(uint32_t* __restr
 // with K = w and one pass.  When every column has had its pivot,
 // A^-1[k][c] = M[piv[k]][rowcol[c]].  Up to kInvSingle columns the matrix is one
 // panel, in the shared memory of one cluster (n = 512: 0.70 ms, n = 513 in five
-// panels 0.63 ms, n = 384 0.61 ms).
+// panels 0.63 ms, n = 384 0.61 ms).  Above 5900 the rows of 128 columns do not fit
+// the cluster: those panels are reduced by narrower ones (64 columns up to 11,700,
+// 32 up to 22,000, ...) whose products stay within the 128 columns, so that the
+// whole matrix is still read and written once per 128: n = 10007 138 ms (217 ms
+// with a product over the matrix per narrow panel, 325 ms by two launches a
+// column), n = 20501 0.95 s (3.09 s, 1.72 s).
 //
 // GB300, 24-bit p: n = 1500 2.5 ms (15.3 ms with two launches per column of a
 // panel), n = 1024 1.3 ms, n = 128 0.12 ms.  Of a round of 16 columns at n = 1500
@@ -149,23 +154,24 @@ __global__ void __launch_bounds__(kElimThreads) gj_elim_kernel(uint32_t* __restr
 // pivots 10,000, the barriers and the way of Y through L2 7,000; the products
 // between panels add 60 us each.
 
-// The other columns of M: x < c0 stays, x >= c0 is column x + w.
+// The other columns of a block of M's columns from b0, w of them from c0 being
+// the panel: column x of the R others is b0 + x, or b0 + x + w from the panel on.
 __global__ void __launch_bounds__(kElimThreads)
-    inv_gather_kernel(const uint32_t* __restrict__ M, int64_t ld, int64_t c0, int w, int64_t R,
+    inv_gather_kernel(const uint32_t* __restrict__ M, int64_t ld, int64_t b0, int64_t c0, int w, int64_t R,
                       const int* __restrict__ piv, int32_t* __restrict__ Mp, const int* flag) {
     const int64_t x = (int64_t)blockIdx.x * kElimThreads + threadIdx.x;
     if (x >= R || *flag) return;  // (without a pivot there is no row to read)
     const int t = blockIdx.y;
-    Mp[(int64_t)t * R + x] = (int32_t)M[(int64_t)piv[c0 + t] * ld + (x < c0 ? x : x + w)];
+    Mp[(int64_t)t * R + x] = (int32_t)M[(int64_t)piv[c0 + t] * ld + b0 + (b0 + x < c0 ? x : x + w)];
 }
 
 // M[i] = C[i] on the panel's pivot rows, M[i] + C[i] mod p on the others
 __global__ void __launch_bounds__(kElimThreads)
-    inv_update_kernel(uint32_t* __restrict__ M, int64_t ld, int64_t n, int64_t c0, int w, int64_t R,
+    inv_update_kernel(uint32_t* __restrict__ M, int64_t ld, int64_t n, int64_t b0, int64_t c0, int w, int64_t R,
                       const int* __restrict__ rowcol, const int32_t* __restrict__ C, uint32_t p) {
     const int64_t x = (int64_t)blockIdx.x * kElimThreads + threadIdx.x;
     if (x >= R) return;
-    const int64_t c = x < c0 ? x : x + w;
+    const int64_t c = b0 + (b0 + x < c0 ? x : x + w);
     for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
         const int q = rowcol[i];
         const uint32_t v = (uint32_t)C[i * R + x];
@@ -187,7 +193,9 @@ __global__ void __launch_bounds__(kElimThreads)
 
 }  // namespace
 
-int64_t inv_panel_width(int64_t n) { return n <= kInvSingle ? n : panel_width(n, 1, 128); }
+int64_t inv_panel_width(int64_t n) { return n <= kInvSingle ? n : 128; }
+
+int64_t inv_sub_width(int64_t n) { return n <= kInvSingle ? n : panel_width(n, 1, 128); }
 
 size_t inv_scratch_bytes() { return sizeof(uint32_t) * panel_scratch(kInvSingle); }
 
@@ -208,19 +216,19 @@ cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t
     return launch_panel_red<1, PanelRed::kOddNarrow, PanelKind::kInverse>(a, n, s);  // (p odd, at most 26 bits)
 }
 
-cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t c0, int w, const int* piv, int32_t* Mp,
-                              const int* flag, cudaStream_t s) {
-    const int64_t R = n - w;
+cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t b0, int64_t bw, int64_t c0, int w, const int* piv,
+                              int32_t* Mp, const int* flag, cudaStream_t s) {
+    const int64_t R = bw - w;
     inv_gather_kernel<<<dim3((unsigned)((R + kElimThreads - 1) / kElimThreads), (unsigned)w), kElimThreads, 0, s>>>(
-        M, n, c0, w, R, piv, Mp, flag);
+        M, n, b0, c0, w, R, piv, Mp, flag);
     return cudaGetLastError();
 }
 
-cudaError_t launch_inv_update(uint32_t* M, int64_t n, int64_t c0, int w, const int* rowcol, const int32_t* C,
-                              uint32_t p, cudaStream_t s) {
-    const int64_t R = n - w;
+cudaError_t launch_inv_update(uint32_t* M, int64_t n, int64_t b0, int64_t bw, int64_t c0, int w, const int* rowcol,
+                              const int32_t* C, uint32_t p, cudaStream_t s) {
+    const int64_t R = bw - w;
     inv_update_kernel<<<dim3((unsigned)((R + kElimThreads - 1) / kElimThreads), (unsigned)std::min<int64_t>(n, kMaxGridY)),
-                        kElimThreads, 0, s>>>(M, n, n, c0, w, R, rowcol, C, p);
+                        kElimThreads, 0, s>>>(M, n, n, b0, c0, w, R, rowcol, C, p);
     return cudaGetLastError();
 }
 

@@ -52,6 +52,10 @@ constexpr int kFbStride = kSub + 4; // words of one row's multipliers in one lan
 constexpr int kParts = 4;            // warps that share the columns of a tile
 constexpr size_t kPanelSmem = 216 * 1024;  // of a block's 227 KB: the rows of the panel and the kernel's static arrays
 
+// Words of a panel row in shared memory: an odd multiple of four, so that one
+// column of consecutive rows takes eight banks.
+constexpr int panel_stride(int W) { return ((W + 3) & ~3) | 4; }
+
 // Up to L moduli side by side in each entry; lanes beyond those in use repeat
 // lane 0.  A modulus is a prime or a prime power, R = 2^32.
 template <int L>
@@ -127,6 +131,35 @@ struct PanelArgs {
     const int* ndef;      // the latter before the panel and after it
     int* ndef_out;
 };
+
+// Blocks of a panel's cluster: 16 (the largest), fewer for matrices of few rows
+// (a block wants 32 candidate rows).
+inline int panel_cluster(int64_t n) {
+    int C = 16;
+    while (C > 1 && n < 32 * C) C /= 2;
+    return C;
+}
+
+inline size_t panel_smem(int64_t rows_max, int64_t W, int64_t w) {
+    return sizeof(uint32_t) * (size_t)(rows_max * (panel_stride((int)W) + 2) + w + 32 * W);
+}
+
+// words of a panel's scratch in global memory
+constexpr size_t panel_scratch(size_t W) { return (kSub + 32) * W + 32; }
+
+// dynamic shared memory a panel kernel of L lanes may take
+constexpr size_t panel_smem_limit(int L) {
+    return kPanelSmem - sizeof(uint32_t) * (size_t)(kSub + 2 * kPanelBatch) * L * kFbStride;
+}
+
+// The widest panel of at most `most` columns (a power of two) whose rows fit the
+// blocks; 0 where no panel fits (one lane: n above 142,000).
+inline int panel_width(int64_t n, int L, int most) {
+    const int64_t rows = (n + 15) / 16;
+    int w = most;
+    while (w > 0 && panel_smem(rows, (int64_t)w * L, w) > panel_smem_limit(L)) w /= 2;
+    return w;
+}
 
 #ifdef __CUDACC__
 namespace {
@@ -337,7 +370,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) panel_kernel(const __grid_co
     pdl_trigger();
     if (a.flag && *a.flag) return;  // a column had no pivot (the same for every block)
     const int C = (int)gridDim.x, rank = (int)blockIdx.x;  // one cluster
-    const int w = a.w, W = w * L, stride = ((W + 3) & ~3) + 4;
+    const int w = a.w, W = w * L, stride = panel_stride(W);
     const int nrows = INV ? (int)a.n : *a.count;
     const int rows = (nrows - rank + C - 1) / C;  // <= rows_max
     uint32_t* T = sm;                             // [rows_max][stride]
@@ -646,35 +679,6 @@ __global__ void __launch_bounds__(kPanelThreads, 1) panel_kernel(const __grid_co
 }
 
 }  // namespace
-
-// Blocks of a panel's cluster: 16 (the largest), fewer for matrices of few rows
-// (a block wants 32 candidate rows).
-inline int panel_cluster(int64_t n) {
-    int C = 16;
-    while (C > 1 && n < 32 * C) C /= 2;
-    return C;
-}
-
-inline size_t panel_smem(int64_t rows_max, int64_t W, int64_t w) {
-    return sizeof(uint32_t) * (size_t)(rows_max * (((W + 3) & ~(int64_t)3) + 4 + 2) + w + 32 * W);
-}
-
-// words of a panel's scratch in global memory
-constexpr size_t panel_scratch(size_t W) { return (kSub + 32) * W + 32; }
-
-// dynamic shared memory a panel kernel of L lanes may take
-constexpr size_t panel_smem_limit(int L) {
-    return kPanelSmem - sizeof(uint32_t) * (size_t)(kSub + 2 * kPanelBatch) * L * kFbStride;
-}
-
-// The widest panel of at most `most` columns (a power of two) whose rows fit the blocks.
-inline int panel_width(int64_t n, int L, int most) {
-    const int64_t rows = (n + 15) / 16;
-    int w = most;
-    while (w > 1 && panel_smem(rows, (int64_t)w * L, w) > panel_smem_limit(L))
-        w /= 2;
-    return w;
-}
 
 template <int L, PanelRed RED, PanelKind KIND>
 cudaError_t launch_panel_red(PanelArgs<L>& a, int64_t n, cudaStream_t s) {

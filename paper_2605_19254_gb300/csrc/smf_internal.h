@@ -463,19 +463,23 @@ cudaError_t launch_inverse_mod_p(const int32_t* res, int64_t n, uint32_t p, uint
 // The form by panels (inverse.cu), odd p < 2^31: M (n x n, canonical, the
 // matrix on entry) is reduced in place, panel by panel of w columns from c0:
 // the panel itself in one cluster (rowcol: -1 everywhere at the start; S gets
-// the panel's n x w transform), the pivot rows' other n - w columns gathered
-// into Mp (w x (n - w)), their product C = S Mp taken into M, and at the end
-// A^-1 placed from M by the pivots.  A panel as wide as the matrix (n <=
-// kInvSingle) needs no product: S may be null then.
+// the panel's n x w transform), the pivot rows' other columns (of the bw from
+// b0: the whole matrix) gathered into Mp (w x (bw - w)), their product C = S Mp
+// taken into M, and at the end A^-1 placed from M by the pivots.  A panel as wide
+// as the matrix (n <= kInvSingle) needs no product: S may be null then.  Panels of
+// inv_panel_width columns whose rows do not fit the cluster are reduced in the
+// same way themselves, by panels of inv_sub_width columns (0: none fits) within
+// their own columns; they end as their own transform.
 constexpr int64_t kInvSingle = 512;
 int64_t inv_panel_width(int64_t n);
+int64_t inv_sub_width(int64_t n);
 cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t p, int* rowcol, int* piv, int32_t* S,
                              void* scratch, int* flag, int* status, cudaStream_t s);
 size_t inv_scratch_bytes();
-cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t c0, int w, const int* piv, int32_t* Mp,
-                              const int* flag, cudaStream_t s);
-cudaError_t launch_inv_update(uint32_t* M, int64_t n, int64_t c0, int w, const int* rowcol, const int32_t* C,
-                              uint32_t p, cudaStream_t s);
+cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t b0, int64_t bw, int64_t c0, int w, const int* piv,
+                              int32_t* Mp, const int* flag, cudaStream_t s);
+cudaError_t launch_inv_update(uint32_t* M, int64_t n, int64_t b0, int64_t bw, int64_t c0, int w, const int* rowcol,
+                              const int32_t* C, uint32_t p, cudaStream_t s);
 cudaError_t launch_inv_place(const uint32_t* M, int64_t n, const int* piv, const int* rowcol, int32_t* out,
                              const int* flag, cudaStream_t s);
 // Column sums of the p-adic digits weighted by W (invariant.cu):
