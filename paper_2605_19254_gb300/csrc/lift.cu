@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kThreads)
     pdl_wait();
     pdl_trigger();
     const int64_t nm = n * m;
-    const int64_t k0 = (int64_t)blockIdx.x * kTileK, c0 = (int64_t)blockIdx.y * kTileC;
+    const int64_t k0 = (int64_t)blockIdx.y * kTileK, c0 = (int64_t)blockIdx.x * kTileC;
     {  // X_i = the K-split partials summed mod p, along c
         const int tx = threadIdx.x % kTileC, ty = threadIdx.x / kTileC;
         const int64_t k = k0 + ty, c = c0 + tx;
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kThreads)
     pdl_wait();
     pdl_trigger();
     const int64_t nm = n * m;
-    const int64_t k0 = (int64_t)blockIdx.x * kTileK, c0 = (int64_t)blockIdx.y * kTileC;
+    const int64_t k0 = (int64_t)blockIdx.y * kTileK, c0 = (int64_t)blockIdx.x * kTileC;
     {
         const int tx = threadIdx.x % kTileC, ty = threadIdx.x / kTileC;
         const int64_t k = k0 + ty, c = c0 + tx;
@@ -217,10 +217,16 @@ void lift_basis(const smf_basis& Q, uint32_t p, LiftBasis* q) {
     q->qmax = INT64_MAX / (int64_t)p;
 }
 
+// Tiles of columns along x, which takes 2^31 blocks (y: 65535; A is n x n, so n is
+// never that large, but m can be).
+static dim3 tile_grid(int64_t n, int64_t m) {
+    return dim3((unsigned)((m + kTileC - 1) / kTileC), (unsigned)((n + kTileK - 1) / kTileK));
+}
+
 cudaError_t launch_lift_x(const int32_t* part, int split, int64_t n, int64_t m, int32_t* X, const LiftBasis& q,
                           void* xdig, int64_t ldd, int t, cudaStream_t s) {
     if (n * m == 0) return cudaSuccess;
-    const dim3 grid((unsigned)((n + kTileK - 1) / kTileK), (unsigned)((m + kTileC - 1) / kTileC));
+    const dim3 grid = tile_grid(n, m);
     __nv_bfloat16* xd = (__nv_bfloat16*)xdig;
     switch (q.L) {
     case 1: return launch_pdl(lift_x_kernel<1>, grid, dim3(kThreads), 0, s, part, split, n, m, X, q, xd, ldd, t);
@@ -234,7 +240,7 @@ cudaError_t launch_lift_x(const int32_t* part, int split, int64_t n, int64_t m, 
 cudaError_t launch_lift_step(const int32_t* part, int split, int64_t n, int64_t m, const LiftBasis& q, int64_t* R,
                              int64_t ldR, void* rdig, int64_t ldd, int t, int* status, cudaStream_t s) {
     if (n * m == 0) return cudaSuccess;
-    const dim3 grid((unsigned)((n + kTileK - 1) / kTileK), (unsigned)((m + kTileC - 1) / kTileC));
+    const dim3 grid = tile_grid(n, m);
     __nv_bfloat16* rd = (__nv_bfloat16*)rdig;
     switch (q.L) {
     case 1: return launch_pdl(lift_step_kernel<1>, grid, dim3(kThreads), 0, s, part, split, n, m, q, R, ldR, rd, ldd, t, status);
