@@ -174,7 +174,7 @@ convert_kernel(const __grid_constant__ ConvConst<LMAX> v, const int32_t* __restr
 
 
 // ---------------------------------------------------------------------------
-// CRT of bases of at most 48 primes below 2^24, on the tensor cores (rns_mma.h).
+// CRT of bases of 9 to 48 primes below 2^24, on the tensor cores (rns_mma.h).
 // x = sum_i xi_i M_i - alpha M - H modulo 2^(8 N), where N bytes hold the signed
 // result; the columns of the product are the balanced base-256 digits of the
 // 2^(8u) M_i, lane 4g + t owns 2 NT consecutive ones (NT / 2 limbs), and the carry
@@ -652,18 +652,23 @@ cudaError_t launch_convert_t(const CrtHost& h, const uint32_t* q, int LQ, const 
 // (kMinPrime), keep the multiply-adds.
 bool narrow_basis(const CrtHost& h) { return h.L > 0 && h.L <= 48 && h.p[0] < (1u << 24); }
 
+// The CRT of up to eight primes is few multiply-adds an entry, and no tables to
+// copy: 1M entries as limb sums / digit products (of eight primes, zeros or not)
+// take 13.7 / 29.4 us with one prime, 18.2 / 28.9 with five, 22.2 / 28.0 with eight
+// (41.8 with nine, 47.2 as limb sums), 1024 entries 2.3 to 3.2 / 2.9 to 3.5 us.
+bool mma_crt(const CrtHost& h) { return narrow_basis(h) && h.L > 8; }
+
 }  // namespace
 
 size_t crt_image_bytes(const CrtHost& h, size_t* pc) {
     if (!narrow_basis(h)) return 0;
 #define SMF_IMAGE(N) (*pc = CrtMma<N>::kPc, CrtMma<N>::kImage)
-    return h.L <= 8 ? SMF_IMAGE(8) : h.L <= 16 ? SMF_IMAGE(16) : h.L <= 24 ? SMF_IMAGE(24) : h.L <= 32 ? SMF_IMAGE(32) : SMF_IMAGE(48);
+    return h.L <= 16 ? SMF_IMAGE(16) : h.L <= 24 ? SMF_IMAGE(24) : h.L <= 32 ? SMF_IMAGE(32) : SMF_IMAGE(48);
 #undef SMF_IMAGE
 }
 
 void crt_image_make(const CrtHost& h, uint8_t* image) {
-    if (h.L <= 8) crt_image<8>(h, image);
-    else if (h.L <= 16) crt_image<16>(h, image);
+    if (h.L <= 16) crt_image<16>(h, image);
     else if (h.L <= 24) crt_image<24>(h, image);
     else if (h.L <= 32) crt_image<32>(h, image);
     else crt_image<48>(h, image);
@@ -672,14 +677,15 @@ void crt_image_make(const CrtHost& h, uint8_t* image) {
 cudaError_t launch_crt(const CrtHost& h, const int32_t* R, int64_t rows, int64_t cols, uint64_t* X, int64_t ld,
                        int W, int num_sms, cudaStream_t s) {
     if (rows == 0 || cols == 0) return cudaSuccess;
-    if (narrow_basis(h)) {
-        if (h.L <= 8) return launch_crt_mma<8>(h, R, rows, cols, X, ld, W, num_sms, s);
+    if (mma_crt(h)) {
         if (h.L <= 16) return launch_crt_mma<16>(h, R, rows, cols, X, ld, W, num_sms, s);
         if (h.L <= 24) return launch_crt_mma<24>(h, R, rows, cols, X, ld, W, num_sms, s);
         if (h.L <= 32) return launch_crt_mma<32>(h, R, rows, cols, X, ld, W, num_sms, s);
         return launch_crt_mma<48>(h, R, rows, cols, X, ld, W, num_sms, s);
     }
-    if (h.L <= 8) return launch_crt_t<8, true, 26>(h, R, rows, cols, X, ld, W, s);
+    if (h.L <= 8)  // primes below 2^24: fewer limbs of M
+        return narrow_basis(h) ? launch_crt_t<8, true, 24>(h, R, rows, cols, X, ld, W, s)
+                               : launch_crt_t<8, true, 26>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 16) return launch_crt_t<16, true, 26>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 24) return launch_crt_t<24, true, 26>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 32) return launch_crt_t<32, true, 26>(h, R, rows, cols, X, ld, W, s);
@@ -694,14 +700,15 @@ cudaError_t launch_crt_grouped(const CrtHost& h, const CrtItem* items, int n, in
                                cudaStream_t s) {
     if (n == 0 || units == 0) return cudaSuccess;
     if (units > 0x7FFFFFFF) return cudaErrorInvalidValue;
-    if (narrow_basis(h)) {
-        if (h.L <= 8) return launch_crt_mma_grouped<8>(h, items, n, units, num_sms, s);
+    if (mma_crt(h)) {
         if (h.L <= 16) return launch_crt_mma_grouped<16>(h, items, n, units, num_sms, s);
         if (h.L <= 24) return launch_crt_mma_grouped<24>(h, items, n, units, num_sms, s);
         if (h.L <= 32) return launch_crt_mma_grouped<32>(h, items, n, units, num_sms, s);
         return launch_crt_mma_grouped<48>(h, items, n, units, num_sms, s);
     }
-    if (h.L <= 8) return launch_crt_grouped_t<8, true, 26>(h, items, n, units, s);
+    if (h.L <= 8)
+        return narrow_basis(h) ? launch_crt_grouped_t<8, true, 24>(h, items, n, units, s)
+                               : launch_crt_grouped_t<8, true, 26>(h, items, n, units, s);
     if (h.L <= 16) return launch_crt_grouped_t<16, true, 26>(h, items, n, units, s);
     if (h.L <= 24) return launch_crt_grouped_t<24, true, 26>(h, items, n, units, s);
     if (h.L <= 32) return launch_crt_grouped_t<32, true, 26>(h, items, n, units, s);

@@ -13,8 +13,10 @@
 // an fp32 sum of xi_i * (1/p_i), whose error is below 2^-14; its fractional
 // part is y / M, which lies near 1/2 for every |x| well inside (-M/2, M/2]
 // (H shifts small results to the middle), so the floor is exact unless the
-// fraction falls within 2^-12 of an integer.  Those entries take the exact
-// Garner path below.
+// fraction falls within 2^-12 of an integer.  Those entries (one in 2000 of
+// residues spread over the whole range) take the exact Garner path below; up to
+// eight primes, whose kernels end in a few us, first the fraction in fixed point
+// (kFix), which leaves one in 2^34: 16384 entries with 8 primes 9.7 -> 3.4 us.
 //
 // Garner path (mixed radix).  With weights W_k = p_0 ... p_(k-1), x = sum_k v_k W_k,
 //   v_i = (r_i - sum_(k<i) v_k W_k) * W_i^-1   (mod p_i),   0 <= v_i < p_i,
@@ -55,6 +57,7 @@ __device__ __forceinline__ uint32_t shoup_mul(uint32_t v, uint32_t w, uint32_t w
 template <int LMAX, bool FAST, int PB>  // PB: bits of the largest prime (24 or 26)
 struct CrtConst {
     static constexpr int MLMAX = (LMAX * PB + 31) / 32 + 1;
+    static constexpr bool kFix = FAST && LMAX <= 8;
     uint32_t p[LMAX];
     uint32_t ginv[LMAX], ginvs[LMAX];
     uint32_t gw[LMAX * (LMAX - 1) / 2], gws[LMAX * (LMAX - 1) / 2];
@@ -65,6 +68,7 @@ struct CrtConst {
     float invp[FAST ? LMAX : 1];                       // 1/p_i
     uint32_t mi[FAST ? LMAX * MLMAX : 1];              // limbs of M_i
     uint32_t h[FAST ? MLMAX : 1];                      // limbs of H
+    uint64_t rcp[kFix ? LMAX : 1];                     // floor(2^64 / p_i)
     int L, m_limbs;
 };
 
@@ -204,8 +208,10 @@ __device__ __forceinline__ bool lagrange(const CrtConst<LMAX, true, PB>& q, cons
                                          int64_t count, int64_t e, uint32_t (&x)[CrtConst<LMAX, true, PB>::MLMAX],
                                          uint32_t& ext) {
     constexpr int MLMAX = CrtConst<LMAX, true, PB>::MLMAX;
+    constexpr bool kFix = CrtConst<LMAX, true, PB>::kFix;
     const int L = q.L;
     uint64_t col[MLMAX];
+    uint32_t xi[kFix ? LMAX : 1];
 #pragma unroll
     for (int j = 0; j < MLMAX; j++) col[j] = 0;
     float f = 0.f;
@@ -224,14 +230,25 @@ __device__ __forceinline__ bool lagrange(const CrtConst<LMAX, true, PB>& q, cons
             uint32_t z = shoup_mul(a, q.c[i], q.cs[i], pi);
             if (z >= pi) z -= pi;
             f = fmaf((float)z, q.invp[i], f);
+            if constexpr (kFix) xi[i] = z;
 #pragma unroll
             for (int j = 0; j < MLMAX; j++) col[j] += (uint64_t)z * q.mi[i * MLMAX + j];
+        } else if constexpr (kFix) {
+            xi[i] = 0;
         }
     }
     const float fl = floorf(f);
     const float frac = f - fl;
-    if (frac < 0x1p-12f || frac > 1.f - 0x1p-12f) return false;
-    const uint32_t alpha = (uint32_t)fl;
+    uint32_t alpha = (uint32_t)fl;
+    if (frac < 0x1p-12f || frac > 1.f - 0x1p-12f) {
+        if constexpr (!kFix) return false;
+        // 2^64 times the fraction, too small by less than the sum of the xi_i (below 2^30)
+        uint64_t s = 0;
+#pragma unroll
+        for (int i = 0; i < (kFix ? LMAX : 1); i++) s += xi[i] * q.rcp[i];
+        if (s >= 0ull - (1ull << 30)) return false;
+        alpha = (uint32_t)rintf(f) - (uint32_t)(s >> 63);  // just below an integer, or just above it
+    }
     // y = sum_i xi_i M_i - alpha M limb by limb, then x = y - H
     uint64_t carry = 0;
     uint32_t borrow = 0, borrow2 = 0;
@@ -309,6 +326,7 @@ void crt_const(const CrtHost& h, CrtConst<LMAX, FAST, PB>& q) {
             q.c[i] = h.c[i];
             q.cs[i] = h.cs[i];
             q.invp[i] = 1.0f / (float)h.p[i];
+            if constexpr (Q::kFix) q.rcp[i] = UINT64_MAX / h.p[i];
             for (int j = 0; j < h.m_limbs && j < Q::MLMAX; j++)
                 q.mi[i * Q::MLMAX + j] = h.mi[(size_t)i * h.m_limbs + j];
         }
