@@ -301,36 +301,43 @@ __device__ __forceinline__ void rm_tables(const uint8_t* __restrict__ image, int
 
 constexpr int word_class(int W) { return W == 1 ? 0 : W == 2 ? 1 : W == 4 ? 2 : 3; }
 
-// Does an entry, its limbs spread over the quad's lanes, lie outside [-2^bits, 2^bits] (as over_bits)?
+// Does one of the warp's 32 entries (four in a quad, their limbs spread over its
+// lanes) lie outside [-2^bits, 2^bits] (as over_bits)?  Some lane knows from its own
+// limbs, but for a value with bit `bits` set and none above it: whether a lower bit
+// is set too.  (Three votes an entry instead took a quarter of the reduction's time.)
 template <int W>
-__device__ __forceinline__ bool rm_over(const uint32_t (&v)[RmShape<W>::KS], int bits) {
+__device__ __forceinline__ bool rm_over(const uint32_t (&v)[4][RmShape<W>::KS], int bits) {
     constexpr int KS = RmShape<W>::KS;
     const int lane = threadIdx.x & 31, t = lane & 3, Lb = bits >> 5, sh = bits & 31;
-    const bool neg = __shfl_sync(0xffffffffu, v[KS - 1], (lane & ~3) | (W == 1 ? 1 : 3)) >> 31;
-    bool over = false, one = false, nz = false;
+    bool over = false;
+    unsigned one = 0, nz = 0;  // a bit for each entry
 #pragma unroll
-    for (int k = 0; k < KS; k++) {
-        const int j = t * KS + k;
-        if (j >= 2 * W) continue;
-        if (j < Lb) {
-            nz |= v[k] != 0;
-        } else if (j == Lb) {
-            const uint32_t hi = v[k] >> sh;
-            if (neg) {
-                over |= hi != (0xFFFFFFFFu >> sh);
+    for (int x = 0; x < 4; x++) {
+        const uint32_t sign = (uint32_t)((int32_t)__shfl_sync(0xffffffffu, v[x][KS - 1], lane | 3) >> 31);
+#pragma unroll
+        for (int k = 0; k < KS; k++) {
+            const int j = t * KS + k;
+            if (j < Lb) {
+                nz |= (unsigned)(v[x][k] != 0) << x;
+            } else if (j == Lb) {
+                const uint32_t hi = (v[x][k] ^ sign) >> sh;
+                over |= hi > (sign ? 0u : 1u);
+                one |= (unsigned)(hi == 1 && !sign) << x;
+                nz |= (unsigned)(sh && (v[x][k] << (32 - sh)) != 0) << x;
             } else {
-                over |= hi > 1;
-                one |= hi == 1;
-                nz |= sh && (v[k] << (32 - sh)) != 0;
+                over |= v[x][k] != sign;
             }
-        } else {
-            over |= v[k] != (neg ? 0xFFFFFFFFu : 0u);
         }
     }
-    const unsigned quad = 0xFu << (lane & ~3);
-    const unsigned bo = __ballot_sync(0xffffffffu, over), b1 = __ballot_sync(0xffffffffu, one),
-                   bn = __ballot_sync(0xffffffffu, nz);
-    return (bo & quad) || ((b1 & quad) && (bn & quad));
+    if (__any_sync(0xffffffffu, one)) {
+#pragma unroll
+        for (int d = 1; d < 4; d *= 2) {
+            one |= __shfl_xor_sync(0xffffffffu, one, d);
+            nz |= __shfl_xor_sync(0xffffffffu, nz, d);
+        }
+        over |= (one & nz) != 0;
+    }
+    return over;
 }
 
 // 32 entries from minor m0 of one major, by one warp.
@@ -363,9 +370,13 @@ __device__ __forceinline__ void rm_chunk(const RmArgs& a, int L, const uint2* wf
         }
     }
     if (a.status && a.bits < 64 * W - 1) {
-#pragma unroll
-        for (int x = 0; x < 4; x++)
-            if (rm_over<W>(v[x], a.bits)) flag_bound(a.status);
+        if constexpr (W == 1) {  // an entry per lane, from L1: 60 instructions fewer a warp than from the limbs at hand
+            const int64_t e = m0 + lane;
+            if (e < a.minor_n && over_bits_low((int64_t)__ldg(a.X + (size_t)(e * a.smin + major * a.smaj)), a.bits))
+                flag_bound(a.status);
+        } else if (rm_over<W>(v, a.bits)) {
+            flag_bound(a.status);
+        }
     }
     uint32_t f[2][KS][4];
     const uint32_t top = t == (W == 1 ? 1 : 3) ? 0x80000000u : 0u;  // the sign: the top byte as it is
