@@ -306,6 +306,7 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
     b->dev.p_top = p[0];
     b->dev.p_low = p[L - 1];
     b->crt.d_mi = (const uint32_t*)(d + o_mi);
+    b->crt.d_rcp = (const uint64_t*)(d + o_mu);
     b->crt.d_m = (const uint32_t*)(d + o_m);
     b->crt.d_image = d + o_image;
     b->crt.d_pc = d + o_image + pc;

@@ -399,7 +399,7 @@ void crt_image(const CrtHost& h, uint8_t* image) {
     }
 }
 
-XiExact xi_exact(const CrtHost& h) { return {h.d_mi, h.d_m, h.L, h.m_limbs}; }
+XiExact xi_exact(const CrtHost& h) { return {h.d_mi, h.d_m, h.d_rcp, h.L, h.m_limbs}; }
 
 // As many blocks as are resident at once (each makes the tables once).
 template <auto kernel>

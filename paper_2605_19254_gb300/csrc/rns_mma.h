@@ -43,6 +43,7 @@ struct XiShape {
 struct XiExact {
     const uint32_t* mi;  // [L][m_limbs] limbs of M_i
     const uint32_t* m;   // [m_limbs] limbs of M
+    const uint64_t* rcp; // [L] floor(2^64 / p_i)
     int L, m_limbs;
 };
 
@@ -261,26 +262,29 @@ __device__ __forceinline__ void xi_frags(const XiExact& v, const uint4* pc, cons
         alpha[x] = (uint32_t)fl;
         unsure |= frac < 0x1p-12f || frac > 1.f - 0x1p-12f;
     }
-    // one entry in 2000 (every 16th warp has one): the sum in double precision, whose
-    // error is below 2^-45, and what that leaves open limb by limb (the ends of the
-    // range; settling all of them so left a tail of warps that had several: half of the
-// conversion's 148 us at 1M entries)
+    // One entry in 2000 (of a range taken in full: a warp in 64 has one; results well
+    // inside the range have none).  2^64 times the fraction in wrapping integers, too
+    // small by less than the sum of the xi_i (below 2^30), tells on which side of the
+    // integer the sum lies; what that leaves open (the ends of the range) goes limb
+    // by limb.  (All of them so left a tail of warps that had several, half of the
+    // conversion's 148 us at 1M entries; the sum in double precision, with a division
+    // per prime, 3 us in a call of a few.)
     if (__any_sync(0xffffffffu, unsure)) {
-        double d[4] = {0., 0., 0., 0.};
+        uint64_t d[4] = {0, 0, 0, 0};
 #pragma unroll
         for (int k = 0; k < NQ; k++) {
-            const double iv = 1.0 / (double)pc[4 * k + t].x;
+            const uint64_t rc = 4 * k + t < L ? __ldg(v.rcp + 4 * k + t) : 0;
 #pragma unroll
-            for (int x = 0; x < 4; x++) d[x] = fma((double)r[k][x], iv, d[x]);
+            for (int x = 0; x < 4; x++) d[x] += r[k][x] * rc;
         }
 #pragma unroll
         for (int x = 0; x < 4; x++) {
             d[x] += __shfl_xor_sync(0xffffffffu, d[x], 1);
             d[x] += __shfl_xor_sync(0xffffffffu, d[x], 2);
-            const double fl = floor(d[x]), frac = d[x] - fl;
-            alpha[x] = (uint32_t)fl;
-            if ((frac < 0x1p-40 || frac > 1. - 0x1p-40) && e + x < count)
-                alpha[x] = settle_alpha<LMAX>(v, pc, R, count, e + x, alpha[x]);
+            const float frac = f[x] - floorf(f[x]);
+            if (frac >= 0x1p-12f && frac <= 1.f - 0x1p-12f) continue;
+            if (d[x] < 0ull - (1ull << 30)) alpha[x] = (uint32_t)rintf(f[x]) - (uint32_t)(d[x] >> 63);
+            else if (e + x < count) alpha[x] = settle_alpha<LMAX>(v, pc, R, count, e + x, alpha[x]);
         }
     }
     __syncwarp();

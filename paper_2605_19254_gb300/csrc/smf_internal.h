@@ -56,9 +56,10 @@ struct CrtHost {
     const uint32_t* cs = nullptr;     // [L] Shoup companions of c
     const uint32_t* mi = nullptr;     // [L][m_limbs] limbs of M_i
     const uint32_t* h = nullptr;      // [m_limbs] limbs of H
-    // on the device: limbs of M_i and M; for primes below 2^24 the tensor-core
-    // kernels' tables (crt_image_make), and in them {p_i, H mod p_i, c_i, companion}
+    // on the device: limbs of M_i and M, floor(2^64 / p_i); for primes below 2^24 the
+    // tensor-core kernels' tables (crt_image_make), and in them {p_i, H mod p_i, c_i, companion}
     const uint32_t* d_mi = nullptr;
+    const uint64_t* d_rcp = nullptr;
     const uint32_t* d_m = nullptr;
     const uint8_t* d_image = nullptr;
     const uint8_t* d_pc = nullptr;
