@@ -511,6 +511,84 @@ int64_t rm_resident() {
     return per;
 }
 
+// The transposed reduction of entries of one or two words modulo few primes
+// (limb_sums_t): planes [t][L][cols][ld_out] as above, but limb sums, two or four
+// multiply-adds a prime, where the digit products always work on eight primes.  A
+// block takes 256 rows by four columns (32 bytes of a row of one-word entries); per
+// prime the table has {p, 2^32 mod p, its Shoup companion, floor(2^32 / p)}, then
+// c_j = 2^(32 j) mod p for j <= 2W.  Bound by instruction issue and two-byte stores.
+constexpr int kTCols = 4, kTSumRow = 12;
+template <int W>
+__global__ void __launch_bounds__(kThreads)
+reduce_sums_t_kernel(BasisDev b, const __grid_constant__ ReduceArgs a) {
+    static_assert(4 + 2 * W + 1 <= kTSumRow, "a row of the table");
+    extern __shared__ __align__(16) uint32_t ctab[];  // [L][kTSumRow]
+    for (int e = threadIdx.x; e < b.L; e += kThreads) {
+        const uint32_t p = b.p[e], r32 = b.pow32[e];
+        uint32_t* row = ctab + e * kTSumRow;
+        row[0] = p;
+        row[1] = r32;
+        row[2] = (uint32_t)(((uint64_t)r32 << 32) / p);
+        row[3] = (uint32_t)((1ull << 32) / p);
+        uint32_t c = 1 % p;
+        for (int j = 0; j <= 2 * W; j++) {
+            row[4 + j] = c;
+            c = barrett64((uint64_t)c * r32, p, b.mu[e]);
+        }
+    }
+    __syncthreads();
+    const int64_t r = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (r >= a.rows) return;
+    const int64_t plane = a.cols * a.ld_out, dstride = plane * b.L, cb = (int64_t)blockIdx.y * kTCols;
+    for (int cc = 0; cc < kTCols; cc++) {
+        const int64_t c = cb + cc;
+        if (c >= a.cols) break;
+        const uint64_t* x = a.X + (size_t)(r * a.ld + c) * W;
+        uint32_t v[2 * W];
+        if constexpr (W == 2) {
+            const ulonglong2 q = __ldg((const ulonglong2*)x);
+            v[0] = (uint32_t)q.x;
+            v[1] = (uint32_t)(q.x >> 32);
+            v[2] = (uint32_t)q.y;
+            v[3] = (uint32_t)(q.y >> 32);
+        } else {
+            const uint64_t q = __ldg(x);
+            v[0] = (uint32_t)q;
+            v[1] = (uint32_t)(q >> 32);
+        }
+        const bool neg = v[2 * W - 1] >> 31;
+        if (a.status && over_bits<W>(v, W, a.bits)) flag_bound(a.status);
+        uint16_t* o = (uint16_t*)a.out + c * a.ld_out + r;
+        for (int e = 0; e < b.L; e++, o += plane) {
+            const uint32_t* ct = ctab + e * kTSumRow;
+            const uint4 hd = *(const uint4*)ct, c4 = *(const uint4*)(ct + 4);
+            const uint32_t p = hd.x, cj[4] = {c4.x, c4.y, c4.z, c4.w};
+            uint32_t lo = 0, hi = 0;  // sum_j v_j c_j < 4 * 2^56
+#pragma unroll
+            for (int j = 0; j < 2 * W; j++) mac64(lo, hi, v[j], cj[j]);
+            // hi (2^32 mod p) by Shoup, lo by its reciprocal quotient
+            const uint32_t t1 = hi * hd.y - __umulhi(hi, hd.z) * p;  // [0, 2p)
+            const uint32_t t2 = lo - __umulhi(lo, hd.w) * p;         // [0, 2p)
+            uint32_t rr = t1 + t2;                                   // [0, 4p)
+            if (rr >= 2 * p) rr -= 2 * p;
+            if (rr >= p) rr -= p;
+            if (neg) {  // subtract 2^(64W) mod p
+                const uint32_t cw = W == 1 ? c4.z : ct[8];
+                rr = rr >= cw ? rr - cw : rr + p - cw;
+            }
+            const int32_t val = rr > (p >> 1) ? (int32_t)rr - (int32_t)p : (int32_t)rr;
+            if (a.t == 3) {
+                const int32_t d = val + 128, f = (d >> 8) + 128;
+                o[0] = bf16_bits_small((d & 255) - 128);
+                o[dstride] = bf16_bits_small((f & 255) - 128);
+                o[2 * dstride] = bf16_bits_small(f >> 8);
+            } else {
+                store_digits(val, a.t, (__nv_bfloat16*)o, dstride);
+            }
+        }
+    }
+}
+
 // Digit split of a matrix whose int64 entries (low word of W) are their own
 // centred residues (|x| <= (p_L - 1)/2): planes [t][rows][ld_out].  Eight
 // consecutive entries per thread: 64 bytes in, 16 bytes out per plane.
@@ -718,6 +796,20 @@ static bool mma_reducible(const BasisDev& b, const ReduceArgs& a) {
            ((uintptr_t)a.X & (a.W == 8 ? 15 : 7)) == 0;
 }
 
+// Large matrices of short entries modulo few primes, which limb sums reduce faster
+// (us, limb sums / digit products; small ones the digit products, by a us or so).
+// Canonical residues, 1M entries: one word, one prime 9.7 / 13.5, two primes 11.8 /
+// 13.3, three 14.6 / 13.5; two words, one prime 11.7 / 13.3, two 14.1 / 13.5; four
+// words, one prime 14.7 / 15.7.  Transposed digits, where the digit products take
+// 20 with up to eight primes and 27 with nine to sixteen: one word, four primes 13.2,
+// six 17.2, eleven 28.9; two words, seven 20.6, nine 24.7, twelve 31.7.
+static bool limb_sums(const BasisDev& b, const ReduceArgs& a, ReduceOut kind) {
+    if (a.rows * a.cols < (1 << 18) || (a.W % 2 == 0 && ((uintptr_t)a.X & 15))) return false;
+    if (kind == ReduceOut::kCanonical) return b.L * a.W <= 2 || (b.L == 1 && a.W == 4);
+    return kind == ReduceOut::kDigitsT && a.W <= 2 && 2 * b.L < (b.L + 7) / 8 * 7 + 9 - a.W && a.rows >= 128 &&
+           a.cols <= 65535 * kTCols;
+}
+
 template <int W>
 static cudaError_t launch_reduce_mma(const BasisDev& b, const ReduceArgs& a, ReduceOut kind, cudaStream_t s) {
     const bool trans = kind == ReduceOut::kDigitsT, ints = kind == ReduceOut::kCanonical;
@@ -775,11 +867,20 @@ cudaError_t launch_reduce(const BasisDev& b, const ReduceArgs& a_in, ReduceOut k
     const int nw = (2 * a.W + 1 + 3) & ~3;
     int group = a.identity ? 1 : max(1, min(b.L, kTableWords / (nw + 4)));
     // (canonical residues are asked for without a bound)
-    if (mma_reducible(b, a) && (kind == ReduceOut::kCanonical ? !a.status : kind != ReduceOut::kCentered && a.t <= 3))
-        return a.W == 1   ? launch_reduce_mma<1>(b, a, kind, s)
-               : a.W == 2 ? launch_reduce_mma<2>(b, a, kind, s)
-               : a.W == 4 ? launch_reduce_mma<4>(b, a, kind, s)
-                          : launch_reduce_mma<8>(b, a, kind, s);
+    if (mma_reducible(b, a) && (kind == ReduceOut::kCanonical ? !a.status : kind != ReduceOut::kCentered && a.t <= 3)) {
+        if (!limb_sums(b, a, kind))
+            return a.W == 1   ? launch_reduce_mma<1>(b, a, kind, s)
+                   : a.W == 2 ? launch_reduce_mma<2>(b, a, kind, s)
+                   : a.W == 4 ? launch_reduce_mma<4>(b, a, kind, s)
+                              : launch_reduce_mma<8>(b, a, kind, s);
+        if (kind == ReduceOut::kDigitsT) {
+            const dim3 grid((unsigned)((a.rows + kThreads - 1) / kThreads), (unsigned)((a.cols + kTCols - 1) / kTCols));
+            const size_t sm = sizeof(uint32_t) * (size_t)b.L * kTSumRow;
+            if (a.W == 1) reduce_sums_t_kernel<1><<<grid, kThreads, sm, s>>>(b, a);
+            else reduce_sums_t_kernel<2><<<grid, kThreads, sm, s>>>(b, a);
+            return cudaGetLastError();
+        }
+    }
     const int groups = a.identity ? 1 : (b.L + group - 1) / group;
     const bool trans = kind == ReduceOut::kDigitsT;
     const int64_t minor_n = trans ? a.rows : a.cols;
