@@ -174,7 +174,7 @@ convert_kernel(const __grid_constant__ ConvConst<LMAX> v, const int32_t* __restr
 
 
 // ---------------------------------------------------------------------------
-// CRT of bases of 9 to 48 primes below 2^24, on the tensor cores (rns_mma.h).
+// CRT of bases of 13 to 48 primes below 2^24, on the tensor cores (rns_mma.h).
 // x = sum_i xi_i M_i - alpha M - H modulo 2^(8 N), where N bytes hold the signed
 // result; the columns of the product are the balanced base-256 digits of the
 // 2^(8u) M_i, lane 4g + t owns 2 NT consecutive ones (NT / 2 limbs), and the carry
@@ -652,11 +652,12 @@ cudaError_t launch_convert_t(const CrtHost& h, const uint32_t* q, int LQ, const 
 // (kMinPrime), keep the multiply-adds.
 bool narrow_basis(const CrtHost& h) { return h.L > 0 && h.L <= 48 && h.p[0] < (1u << 24); }
 
-// The CRT of up to eight primes is few multiply-adds an entry, and no tables to
-// copy: 1M entries as limb sums / digit products (of eight primes, zeros or not)
-// take 13.7 / 29.4 us with one prime, 18.2 / 28.9 with five, 22.2 / 28.0 with eight
-// (41.8 with nine, 47.2 as limb sums), 1024 entries 2.3 to 3.2 / 2.9 to 3.5 us.
-bool mma_crt(const CrtHost& h) { return narrow_basis(h) && h.L > 8; }
+// The CRT of up to twelve primes is few multiply-adds an entry, and no tables to
+// copy: 1M entries as limb sums / digit products (of 8 or 16 primes, zeros or not)
+// take 13.7 / 29.4 us with one prime, 18.2 / 28.9 with five, 22.2 / 28.0 with eight,
+// 29.6 / 37.8 with nine, 34.8 / 40.2 with twelve (16 as limb sums 72, as digit products
+// 43); 1024 entries about the same.
+bool mma_crt(const CrtHost& h) { return narrow_basis(h) && h.L > 12; }
 
 }  // namespace
 
@@ -686,6 +687,7 @@ cudaError_t launch_crt(const CrtHost& h, const int32_t* R, int64_t rows, int64_t
     if (h.L <= 8)  // primes below 2^24: fewer limbs of M
         return narrow_basis(h) ? launch_crt_t<8, true, 24>(h, R, rows, cols, X, ld, W, s)
                                : launch_crt_t<8, true, 26>(h, R, rows, cols, X, ld, W, s);
+    if (h.L <= 12 && narrow_basis(h)) return launch_crt_t<12, true, 24>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 16) return launch_crt_t<16, true, 26>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 24) return launch_crt_t<24, true, 26>(h, R, rows, cols, X, ld, W, s);
     if (h.L <= 32) return launch_crt_t<32, true, 26>(h, R, rows, cols, X, ld, W, s);
@@ -709,6 +711,7 @@ cudaError_t launch_crt_grouped(const CrtHost& h, const CrtItem* items, int n, in
     if (h.L <= 8)
         return narrow_basis(h) ? launch_crt_grouped_t<8, true, 24>(h, items, n, units, s)
                                : launch_crt_grouped_t<8, true, 26>(h, items, n, units, s);
+    if (h.L <= 12 && narrow_basis(h)) return launch_crt_grouped_t<12, true, 24>(h, items, n, units, s);
     if (h.L <= 16) return launch_crt_grouped_t<16, true, 26>(h, items, n, units, s);
     if (h.L <= 24) return launch_crt_grouped_t<24, true, 26>(h, items, n, units, s);
     if (h.L <= 32) return launch_crt_grouped_t<32, true, 26>(h, items, n, units, s);

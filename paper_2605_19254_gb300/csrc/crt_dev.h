@@ -15,7 +15,7 @@
 // (H shifts small results to the middle), so the floor is exact unless the
 // fraction falls within 2^-12 of an integer.  Those entries (one in 2000 of
 // residues spread over the whole range) take the exact Garner path below; up to
-// eight primes, whose kernels end in a few us, first the fraction in fixed point
+// twelve primes, whose kernels end in a few us, first the fraction in fixed point
 // (kFix), which leaves one in 2^34: 16384 entries with 8 primes 9.7 -> 3.4 us.
 //
 // Garner path (mixed radix).  With weights W_k = p_0 ... p_(k-1), x = sum_k v_k W_k,
@@ -57,7 +57,7 @@ __device__ __forceinline__ uint32_t shoup_mul(uint32_t v, uint32_t w, uint32_t w
 template <int LMAX, bool FAST, int PB>  // PB: bits of the largest prime (24 or 26)
 struct CrtConst {
     static constexpr int MLMAX = (LMAX * PB + 31) / 32 + 1;
-    static constexpr bool kFix = FAST && LMAX <= 8;
+    static constexpr bool kFix = FAST && LMAX <= 12;
     uint32_t p[LMAX];
     uint32_t ginv[LMAX], ginvs[LMAX];
     uint32_t gw[LMAX * (LMAX - 1) / 2], gws[LMAX * (LMAX - 1) / 2];

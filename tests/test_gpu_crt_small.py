@@ -34,7 +34,7 @@ def _basis(ctx, L, p_max):
 
 
 @pytest.mark.parametrize("L,p_max", [(L, p) for p in (1 << 24, 1 << 26, 1 << 11, 60) for L in (1, 2, 3, 5, 8, 9)] +
-                         [(L, 1 << 24) for L in (16, 17, 24, 31, 48)])
+                         [(L, 1 << 24) for L in (12, 13, 16, 17, 24, 31, 48)])
 def test_quotients(ctx, L, p_max):
     b = _basis(ctx, L, p_max)
     primes = [int(p) for p in b.primes]
