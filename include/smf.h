@@ -369,7 +369,7 @@ int smf_padic_lift(smf_ctx* ctx, const smf_basis* p_basis, const smf_bigmat* A, 
  * p-adic lifting, Section 3): Gauss-Jordan elimination over GF(p) on the
  * device, by panels of up to 128 columns (up to 512 columns in one), each
  * reduced in the shared memory of one thread-block cluster; matrices that the
- * panels do not take (p = 2, and above 512 columns the FP64 form or residues of
+ * panels do not take (n = 1, and above 512 columns the FP64 form or residues of
  * more than three digits) one column at a time.  A: device,
  * n x n, any word count.  A_inv: device int32 [n][n], canonical residues.
  * `workspace` holds smf_inverse_mod_p_workspace(n) bytes (NULL: the context

@@ -11,9 +11,9 @@
 //   gj_elim:  every row i != k subtracts f_i times row k, over the columns
 //             j >= k (row k is zero left of column k).
 // Afterwards the right half is A^-1 mod p.  That is the general form; matrices
-// of up to kInvSingle columns (p odd), and larger ones in the limb form, go by
-// panels instead (below).  A column without a pivot means p | det A: the pivot launch sets kStatusSingular and a device flag, and
-// every later launch returns at once.
+// of 2 to kInvSingle columns, and larger ones in the limb form, go by panels
+// instead (below).  A column without a pivot means p | det A: the pivot launch
+// sets kStatusSingular and a device flag, and every later launch returns at once.
 #include <algorithm>
 
 #include "panel.h"
