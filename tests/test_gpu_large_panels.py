@@ -105,3 +105,28 @@ def test_moduli_in_smaller_groups(ctx, n):
     qe = [(2, 5), (3, 3), (5, 2), (7, 1)]
     got = ctx.smith_local(A, [v for v, _ in qe], [e for _, e in qe], a_bits=bits)
     assert got == [[n] + [sum(s % v ** t == 0 for s in tail) for t in range(1, e + 1)] for v, e in qe]
+
+
+# The column loops of 32-bit moduli, which a threshold above n leaves: determinants and local forms, one
+# lane (a pivot step and an update a column) and four in lockstep, against the planted factors.
+@pytest.mark.parametrize("n", [1, 65, 300])
+def test_column_loops(ctx, n):
+    tail = [2, 6, 6, 60, 360, 2520][-min(n, 6):]
+    diag = torch.ones(n, device="cuda")
+    diag[-len(tail):] = torch.tensor(tail, dtype=torch.float32)
+    A = _planted(n, diag, n)
+    bits = max(1, int(A.abs().max()).bit_length())
+    det = 1
+    for v in tail:
+        det *= v
+    ctx.set_elim_panels(1 << 30)
+    try:
+        for q in ([2147483647], [2147483647, 11, 2147483629, 13], [65537, 11, 13, 17, 19]):
+            assert ctx.det_mod(A, q, a_bits=bits) == [det % v for v in q]
+        for qe in ([(2, 5)], [(3, 3)], [(2, 30)], [(2, 5), (3, 3)], [(2, 5), (3, 3), (5, 2), (7, 1)],
+                   [(2, 1), (3, 1), (5, 1), (7, 1), (11, 1)]):
+            got = ctx.smith_local(A, [v for v, _ in qe], [e for _, e in qe], a_bits=bits)
+            want = [[n] + [sum(s % v ** t == 0 for s in tail) for t in range(1, e + 1)] for v, e in qe]
+            assert got == want
+    finally:
+        ctx.set_elim_panels(0)
