@@ -201,6 +201,7 @@ size_t inv_scratch_bytes() { return sizeof(uint32_t) * panel_scratch(kInvSingle)
 
 cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t p, int* rowcol, int* piv, int32_t* S,
                              void* scratch, int* flag, int* status, cudaStream_t s) {
+    if (p >= kInvMaxP || !(p & 1)) return cudaErrorInvalidValue;
     PanelArgs<1> a{};
     a.M = M;
     a.n = a.ld = n;
@@ -213,7 +214,7 @@ cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t
     a.rowcol = rowcol;
     a.S = S;
     a.status = status;
-    return launch_panel_red<1, PanelRed::kOddNarrow, PanelKind::kInverse>(a, n, s);  // (p odd, at most 26 bits)
+    return launch_panel_red<1, PanelRed::kOddNarrow, PanelKind::kInverse>(a, n, s);
 }
 
 cudaError_t launch_inv_gather(const uint32_t* M, int64_t n, int64_t b0, int64_t bw, int64_t c0, int w, const int* piv,

@@ -461,7 +461,8 @@ cudaError_t launch_widen(const int32_t* x, int64_t count, int64_t* out, cudaStre
 // scratch; C gets A^-1 mod p ([n][n]) unless kStatusSingular is raised.
 cudaError_t launch_inverse_mod_p(const int32_t* res, int64_t n, uint32_t p, uint32_t* M, uint32_t* col, int* flag,
                                  int32_t* C, int* status, int num_sms, cudaStream_t s);
-// The form by panels (inverse.cu), odd p < 2^31: M (n x n, canonical, the
+// The form by panels (inverse.cu), odd p < kInvMaxP (16 products of two residues
+// are summed unreduced; a basis has primes below 2^26): M (n x n, canonical, the
 // matrix on entry) is reduced in place, panel by panel of w columns from c0:
 // the panel itself in one cluster (rowcol: -1 everywhere at the start; S gets
 // the panel's n x w transform), the pivot rows' other columns (of the bw from
@@ -472,6 +473,7 @@ cudaError_t launch_inverse_mod_p(const int32_t* res, int64_t n, uint32_t p, uint
 // same way themselves, by panels of inv_sub_width columns (0: none fits) within
 // their own columns; they end as their own transform.
 constexpr int64_t kInvSingle = 512;
+constexpr uint32_t kInvMaxP = 1u << 28;
 int64_t inv_panel_width(int64_t n);
 int64_t inv_sub_width(int64_t n);
 cudaError_t launch_inv_panel(uint32_t* M, int64_t n, int64_t c0, int w, uint32_t p, int* rowcol, int* piv, int32_t* S,
