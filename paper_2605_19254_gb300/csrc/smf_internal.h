@@ -135,7 +135,7 @@ struct smf_ctx {
     // it again: 0.2 ms of a 16 x 16 determinant's 0.28 ms); they go back when the
     // context is destroyed
     cudaMemPool_t pool = nullptr;  // made on first use
-    std::once_flag pool_once;
+    std::mutex pool_mu;
     uint64_t pool_keep = kPoolKeep;
     // pinned host staging of the Smith-form driver's digit sums, kept across calls
     // (allocating and freeing pinned memory per call would synchronise the device)
@@ -204,6 +204,27 @@ struct ProfScope {
     }
 };
 
+// The context's memory pool, made by the first caller that needs it; where that
+// fails the next one tries again.  (Safe from several threads.)
+inline cudaError_t make_pool(smf_ctx* ctx) {
+    std::lock_guard<std::mutex> lk(ctx->pool_mu);
+    if (ctx->pool) return cudaSuccess;
+    cudaMemPoolProps pp{};
+    pp.allocType = cudaMemAllocationTypePinned;
+    pp.location.type = cudaMemLocationTypeDevice;
+    pp.location.id = ctx->device;
+    cudaMemPool_t pool = nullptr;
+    const cudaError_t e = cudaMemPoolCreate(&pool, &pp);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+    }
+    uint64_t keep = ctx->pool_keep;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    ctx->pool = pool;
+    return cudaSuccess;
+}
+
 // Stream-ordered device scratch from the context's own memory pool (freed on the
 // stream the work runs on): no device-wide synchronisation when it is freed, so
 // calls on different streams keep overlapping.
@@ -216,20 +237,8 @@ struct StreamBuf {
     cudaError_t alloc(smf_ctx* ctx, size_t bytes, cudaStream_t st) {
         release();
         s = st;
-        std::call_once(ctx->pool_once, [ctx] {
-            cudaMemPoolProps pp{};
-            pp.allocType = cudaMemAllocationTypePinned;
-            pp.location.type = cudaMemLocationTypeDevice;
-            pp.location.id = ctx->device;
-            if (cudaMemPoolCreate(&ctx->pool, &pp) != cudaSuccess) {
-                cudaGetLastError();
-                ctx->pool = nullptr;
-            } else {
-                uint64_t keep = ctx->pool_keep;
-                cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
-            }
-        });
-        if (!ctx->pool) return cudaErrorMemoryAllocation;
+        const cudaError_t e = make_pool(ctx);
+        if (e != cudaSuccess) return e;
         return cudaMallocFromPoolAsync(&p, bytes ? bytes : 1, ctx->pool, st);
     }
     void release() {
