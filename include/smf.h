@@ -79,7 +79,9 @@ typedef struct {
 
 /* Create a context on CUDA device `device` using residue-product engine
  * `form`.  hbm_budget_bytes caps workspace the library may allocate itself
- * (0 = no cap).  Errors: SMF_E_INVALID, SMF_E_CUDA, SMF_E_UNSUPPORTED (the
+ * (0 = no cap).  Beside it the context keeps up to 256 MiB (no more than the
+ * cap) of the scratch that the eliminations and the Smith-form driver have freed,
+ * for their next call; smf_destroy gives it back.  Errors: SMF_E_INVALID, SMF_E_CUDA, SMF_E_UNSUPPORTED (the
  * device is not sm_103). */
 int smf_create(smf_ctx** ctx, int device, smf_form form, size_t hbm_budget_bytes);
 
@@ -542,7 +544,9 @@ int smf_server_admit(size_t budget_left, int n, const size_t* bytes, int max_bat
  * concurrently on the workers' streams and overlap on the GPU; each job's
  * state stays on the device for its whole run, and the driver's scratch is
  * allocated in stream order so that one job's frees do not stall another's
- * kernels.  Results are those of smf_smith_form on each job alone (bit for
+ * kernels.  An idle worker keeps some of its scratch for its next job (up to 64
+ * MiB, without a budget 256); with a budget that is given back as soon as a job
+ * that starts would not fit beside it.  Results are those of smf_smith_form on each job alone (bit for
  * bit: the seed fixes every random choice).  Errors: SMF_E_INVALID,
  * SMF_E_NOMEM (a job larger than the budget), SMF_E_CUDA. */
 typedef struct smf_smith_server smf_smith_server;

@@ -21,6 +21,7 @@
 #include <thread>
 #include <vector>
 
+#include "pool_book.h"
 #include "smf_internal.h"
 
 namespace {
@@ -53,6 +54,7 @@ struct smf_smith_server {
     std::deque<int64_t> queue;         // job ids in arrival order
     std::deque<SmithJob> jobs;         // stable addresses: workers hold references while jobs are added
     size_t in_use = 0;
+    smf::PoolBook pools;               // with a budget
     int running = 0;
     bool stop = false;
     std::vector<std::thread> threads;
@@ -103,6 +105,8 @@ void worker(smf_smith_server* S, int w) {
             jp->t[1] = now_s(S);
             S->in_use += jp->bytes;
             S->running++;
+            if (S->budget)
+                S->pools.start(w, S->in_use, S->budget, [&](int i) { cudaMemPoolTrimTo(S->ctxs[i]->pool, 0); });
         }
         SmithJob& j = *jp;  // the job's fields are this worker's until it is marked done
         smf_bigmat A{j.n, j.n, j.n, 1, j.bits, j.A.data(), 0, 0};
@@ -116,8 +120,14 @@ void worker(smf_smith_server* S, int w) {
             rc = smf_smith_form(ctx, &A, j.seed, limbs.data(), cap, offsets.data(), nullptr, nullptr, st);
         }
         if (rc == SMF_OK) limbs.resize(offsets[j.n]);
+        uint64_t kept = 0;
+        if (S->budget && ctx->pool) {  // (the last frees of the job are on its stream)
+            cudaStreamSynchronize(st);
+            cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &kept);
+        }
         {
             std::lock_guard<std::mutex> lk(S->mu);
+            if (S->budget) S->pools.finish(w, (size_t)kept);
             j.status = rc;
             if (rc != SMF_OK) j.msg = smf_last_error(ctx);
             j.limbs = std::move(limbs);
@@ -150,7 +160,7 @@ int smf_smith_server_create(int device, smf_form form, size_t budget_bytes, int 
     for (int w = 0; w < workers; w++) {
         smf_ctx* c = nullptr;
         int rc = smf_create(&c, device, form, 0);
-        if (rc == SMF_OK && budget_bytes) c->pool_keep = 64ull << 20;  // no more than the constant part of a footprint
+        if (rc == SMF_OK && budget_bytes) c->pool_keep = 64ull << 20;  // as much as the constant part of a footprint
         cudaStream_t st = nullptr;
         if (rc == SMF_OK && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
             cudaGetLastError();
@@ -170,6 +180,7 @@ int smf_smith_server_create(int device, smf_form form, size_t budget_bytes, int 
         S->streams.push_back(st);
     }
     cudaSetDevice(dev0);
+    S->pools.kept.assign(workers, 0);
     for (int w = 0; w < workers; w++) S->threads.emplace_back(worker, S, w);
     *out = S;
     return SMF_OK;
