@@ -45,8 +45,9 @@ int fail(smf_ctx* c, int code, const std::string& msg) {
 bool is_prime_u32(uint32_t n) {
     if (n < 2) return false;
     if (n % 2 == 0) return n == 2;
-    for (uint32_t d = 3; (uint64_t)d * d <= n; d += 2)
-        if (n % d == 0) return false;
+    if (n % 3 == 0) return n == 3;
+    for (uint32_t d = 5; (uint64_t)d * d <= n; d += 6)  // 6k - 1 and 6k + 1
+        if (n % d == 0 || n % (d + 2) == 0) return false;
     return true;
 }
 
@@ -264,39 +265,44 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
         off = align256(off + bytes);
         return o;
     };
+    // first what the device makes itself, then what is copied from the host
+    size_t o_red[4], pc = 0;
+    for (int k = 0; k < 4; k++) o_red[k] = slot(reduce_image_bytes(p, 1 << k));
+    const size_t image = crt_image_bytes(b->crt, &pc), o_image = slot(image), copied = image ? o_image + pc : off;
     const size_t o_p = slot(4 * L), o_mu = slot(8 * L), o_pow = slot(4 * L), o_inv = slot(8 * L);
     const size_t o_gw = slot(4 * (size_t)L * L), o_gws = slot(4 * (size_t)L * L), o_ginv = slot(4 * L),
                  o_ginvs = slot(4 * L), o_m = slot(4 * ml), o_mi = slot(4 * (size_t)L * ml);
-    size_t pc = 0;
-    const size_t image = crt_image_bytes(b->crt, &pc), o_image = slot(image);
-    size_t o_red[4];
-    for (int k = 0; k < 4; k++) o_red[k] = slot(reduce_image_bytes(p, 1 << k));
-    std::vector<uint8_t> host(off, 0);
-    memcpy(&host[o_p], p.data(), 4 * L);
-    memcpy(&host[o_mu], mu.data(), 8 * L);
-    memcpy(&host[o_pow], pow32.data(), 4 * L);
-    memcpy(&host[o_inv], inv_p.data(), 8 * L);
-    memcpy(&host[o_gw], gw.data(), 4 * (size_t)L * L);
-    memcpy(&host[o_gws], gws.data(), 4 * (size_t)L * L);
-    memcpy(&host[o_ginv], ginv.data(), 4 * L);
-    memcpy(&host[o_ginvs], ginvs.data(), 4 * L);
-    memcpy(&host[o_m], M.data(), 4 * ml);
-    memcpy(&host[o_mi], b->mi.data(), 4 * (size_t)L * ml);
-    if (image) crt_image_make(b->crt, &host[o_image]);
-    for (int k = 0; k < 4; k++)
-        if (reduce_image_bytes(p, 1 << k)) reduce_image_make(p.data(), L, 1 << k, &host[o_red[k]]);
+    std::vector<uint8_t> bytes(off - copied, 0);
+    uint8_t* const host = bytes.data() - copied;  // (at the blob's offsets)
+    memcpy(host + o_p, p.data(), 4 * L);
+    memcpy(host + o_mu, mu.data(), 8 * L);
+    memcpy(host + o_pow, pow32.data(), 4 * L);
+    memcpy(host + o_inv, inv_p.data(), 8 * L);
+    memcpy(host + o_gw, gw.data(), 4 * (size_t)L * L);
+    memcpy(host + o_gws, gws.data(), 4 * (size_t)L * L);
+    memcpy(host + o_ginv, ginv.data(), 4 * L);
+    memcpy(host + o_ginvs, ginvs.data(), 4 * L);
+    memcpy(host + o_m, M.data(), 4 * ml);
+    memcpy(host + o_mi, b->mi.data(), 4 * (size_t)L * ml);
+    if (image) crt_image_make(b->crt, host + o_image);
     DeviceGuard g(ctx->device);
     cudaError_t e = cudaMalloc(&b->dev_blob, off);
     // A copy from pageable memory may return before its DMA lands, and kernels on
     // non-blocking streams are not ordered after the legacy stream: wait for it.
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->dev_blob, host.data(), off, cudaMemcpyHostToDevice, cudaStreamLegacy);
+    uint8_t* d = (uint8_t*)b->dev_blob;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(d + copied, bytes.data(), off - copied, cudaMemcpyHostToDevice, cudaStreamLegacy);
+    if (e == cudaSuccess && reduce_image_bytes(p, 1))
+        e = launch_reduce_images((const uint32_t*)(d + o_p), L, {d + o_red[0], d + o_red[1], d + o_red[2], d + o_red[3]},
+                                 cudaStreamLegacy);
+    b->crt.d_mi = (const uint32_t*)(d + o_mi);
+    if (e == cudaSuccess) e = launch_crt_image(b->crt, d + o_image, cudaStreamLegacy);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) {
         if (b->dev_blob) cudaFree(b->dev_blob);
         delete b;
         return fail(ctx, SMF_E_CUDA, std::string("basis tables: ") + cudaGetErrorString(e));
     }
-    uint8_t* d = (uint8_t*)b->dev_blob;
     b->dev.L = L;
     b->dev.m_limbs = ml;
     b->dev.p = (const uint32_t*)(d + o_p);
@@ -305,7 +311,6 @@ int basis_build(smf_ctx* ctx, int32_t bound_bits, uint32_t p_max, smf_basis** ou
     for (int k = 0; k < 4; k++) b->dev.red[k] = d + o_red[k];
     b->dev.p_top = p[0];
     b->dev.p_low = p[L - 1];
-    b->crt.d_mi = (const uint32_t*)(d + o_mi);
     b->crt.d_rcp = (const uint64_t*)(d + o_mu);
     b->crt.d_m = (const uint32_t*)(d + o_m);
     b->crt.d_image = d + o_image;

@@ -351,35 +351,42 @@ crt_mma_grouped_kernel(const uint8_t* __restrict__ image, XiExact q, const CrtIt
     }
 }
 
-// The image of the tables for a basis.  Lane 4n + t of tile nt owns result bytes
-// (n / 2) 2 NT + 2 nt and + 1, whose digit of 2^(8u) M_i is digit (byte - u) of M_i.
+// The fragments of a basis, a block for each tile, on the device from the limbs of
+// the M_i.  Lane 4n + t of tile nt owns result bytes (n / 2) 2 NT + 2 nt and + 1, whose
+// digit of 2^(8u) M_i is digit (byte - u) of M_i.
+template <int LMAX>
+__global__ void __launch_bounds__(kMmaThreads)
+crt_image_kernel(const uint32_t* __restrict__ mi, int L, int m_limbs, __half* __restrict__ wf) {
+    using Q = CrtMma<LMAX>;
+    constexpr int NL = Q::NL;
+    __shared__ uint32_t bal[LMAX * NL];  // M_i + 0x80..80: its bytes less 128 are the balanced digits of M_i
+    const int nt = blockIdx.x;
+    if (threadIdx.x < L) {
+        uint64_t c = 0;
+        for (int k = 0; k < NL; k++) {
+            c += (uint64_t)(k < m_limbs ? mi[threadIdx.x * m_limbs + k] : 0u) + 0x80808080u;
+            bal[threadIdx.x * NL + k] = (uint32_t)c;
+            c >>= 32;
+        }
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < Q::KS * 128; x += kMmaThreads) {
+        const int ks = x / 128, lane = x / 4 % 32, n = lane >> 2, byte = (n >> 1) * 2 * Q::NT + 2 * nt + (n & 1);
+        int i, u, d = 0;
+        if (xi_slot<LMAX>(ks, x & 3, lane & 3, &i, &u) && i < L && byte >= u)
+            d = (int)(bal[i * NL + ((byte - u) >> 2)] >> (8 * ((byte - u) & 3)) & 255u) - 128;
+        wf[nt * Q::KS * 128 + x] = __int2half_rn(d);
+    }
+}
+
+// The image's other tables.
 template <int LMAX>
 void crt_image(const CrtHost& h, uint8_t* image) {
     using Q = CrtMma<LMAX>;
     constexpr int NL = Q::NL;
-    std::vector<uint32_t> bal((size_t)h.L * NL);  // M_i + 0x80..80: its bytes less 128 are the balanced digits of M_i
     uint64_t sum[NL] = {};
-    for (int i = 0; i < h.L; i++) {
-        uint64_t c = 0;
-        for (int k = 0; k < NL; k++) {
-            const uint32_t mi = k < h.m_limbs ? h.mi[(size_t)i * h.m_limbs + k] : 0u;
-            sum[k] += mi;
-            c += (uint64_t)mi + 0x80808080u;
-            bal[(size_t)i * NL + k] = (uint32_t)c;
-            c >>= 32;
-        }
-    }
-    uint16_t* wf = (uint16_t*)image;
-    for (int nt = 0; nt < Q::NT; nt++)
-        for (int ks = 0; ks < Q::KS; ks++)
-            for (int lane = 0; lane < 32; lane++)
-                for (int kap = 0; kap < 4; kap++) {
-                    const int n = lane >> 2, byte = (n >> 1) * 2 * Q::NT + 2 * nt + (n & 1);
-                    int i, u, d = 0;
-                    if (xi_slot<LMAX>(ks, kap, lane & 3, &i, &u) && i < h.L && byte >= u)
-                        d = (int)(bal[(size_t)i * NL + ((byte - u) >> 2)] >> (8 * ((byte - u) & 3)) & 255u) - 128;
-                    *wf++ = half_bits(d);
-                }
+    for (int i = 0; i < h.L; i++)
+        for (int k = 0; k < NL && k < h.m_limbs; k++) sum[k] += h.mi[(size_t)i * h.m_limbs + k];
     uint4* pc = (uint4*)(image + Q::kPc);
     float* ip = (float*)(image + Q::kIp);
     for (int i = 0; i < LMAX; i++) {  // beyond L: xi = 0
@@ -673,6 +680,16 @@ void crt_image_make(const CrtHost& h, uint8_t* image) {
     else if (h.L <= 24) crt_image<24>(h, image);
     else if (h.L <= 32) crt_image<32>(h, image);
     else crt_image<48>(h, image);
+}
+
+cudaError_t launch_crt_image(const CrtHost& h, uint8_t* image, cudaStream_t s) {
+    if (!mma_crt(h)) return cudaSuccess;
+    __half* wf = (__half*)image;
+    if (h.L <= 16) crt_image_kernel<16><<<CrtMma<16>::NT, kMmaThreads, 0, s>>>(h.d_mi, h.L, h.m_limbs, wf);
+    else if (h.L <= 24) crt_image_kernel<24><<<CrtMma<24>::NT, kMmaThreads, 0, s>>>(h.d_mi, h.L, h.m_limbs, wf);
+    else if (h.L <= 32) crt_image_kernel<32><<<CrtMma<32>::NT, kMmaThreads, 0, s>>>(h.d_mi, h.L, h.m_limbs, wf);
+    else crt_image_kernel<48><<<CrtMma<48>::NT, kMmaThreads, 0, s>>>(h.d_mi, h.L, h.m_limbs, wf);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_crt(const CrtHost& h, const int32_t* R, int64_t rows, int64_t cols, uint64_t* X, int64_t ld,

@@ -254,41 +254,49 @@ struct RmShape {
 
 __host__ __device__ constexpr size_t rm_frag(int L, int KS) { return sizeof(uint2) * ((L + 7) / 8 * 3) * KS * 32; }
 
-// The tables of a basis, made with it and copied to shared memory by each block:
-// the constants' fragments (three n8 tiles for the eight primes 8B .. 8B + 7, as in
-// the conversion), and per prime {p, rem_const, 1 / p, quot_const} of the constant,
-// for centred and then for canonical results: what the bytes' 128s take off, and
-// (p - 1) / 2 for centred results.
-template <int W>
-void reduce_image(const uint32_t* p, int L, uint8_t* image) {
-    constexpr int KS = RmShape<W>::KS;
-    uint16_t* wf = (uint16_t*)image;
-    memset(wf, 0, rm_frag(L, KS));
-    uint4* ti = (uint4*)(image + rm_frag(L, KS));
-    for (int i = 0; i < L; i++) {
-        uint64_t w = 1, sum = 0;  // 2^(8b) mod p_i, and 128 times their sum over the bytes below the top one
-        for (int b = 0; b < 8 * W; b++) {
-            int32_t r = (int32_t)w;
-            if (r > (int32_t)(p[i] >> 1)) r -= (int32_t)p[i];
-            const int limb = b >> 2, t = limb / KS, ks = limb % KS;
-            for (int dig = 0; dig < 3; dig++) {
-                const int c6 = (i >> 2 & 1) * 3 + dig, nt = (i >> 3) * 3 + c6 / 2;
-                const int ln = (2 * (i & 3) + (c6 & 1)) * 4 + t;
-                wf[((nt * KS + ks) * 32 + ln) * 4 + (b & 3)] = half_bits(dig < 2 ? ((r + 128) & 255) - 128 : r);
-                r = (r + 128) >> 8;
-            }
-            if (b < 8 * W - 1) sum += 128 * w;
-            w = w * 256 % p[i];
-        }
-        for (int ints = 0; ints < 2; ints++) {
-            const uint32_t c = (uint32_t)((sum + (ints ? 0u : p[i] >> 1)) % p[i]);
-            const float ip = 1.0f / (float)p[i], fc = quot_const(c, ip, p[i]);
-            uint32_t bits[2];
-            memcpy(&bits[0], &ip, 4);
-            memcpy(&bits[1], &fc, 4);
-            ti[ints * L + i] = make_uint4(p[i], rem_const(c, p[i]), bits[0], bits[1]);
+// The tables of a basis, made with it (on the device: on the host they took as long
+// as a small product) and copied to shared memory by each block: the constants'
+// fragments (three n8 tiles for the eight primes 8B .. 8B + 7, as in the
+// conversion), and per prime {p, rem_const, 1 / p, quot_const} of the constant, for
+// centred and then for canonical results: what the bytes' 128s take off, and
+// (p - 1) / 2 for centred results.  A block makes prime i's part of the four (zeros
+// beyond L), a thread that of 2^(8b) mod p.
+struct ReduceImages {
+    uint8_t* to[4];  // for entries of 1, 2, 4, 8 words
+};
+constexpr int kImageBytes = 64;  // bytes of the longest entry
+__global__ void __launch_bounds__(kImageBytes)
+reduce_images_kernel(const uint32_t* __restrict__ primes, int L, ReduceImages im) {
+    __shared__ uint32_t ws[kImageBytes];
+    const int i = blockIdx.x, b = threadIdx.x;
+    const uint32_t p = i < L ? primes[i] : 1u;
+    uint32_t w = 1 % p;
+    for (int k = 0; k < b; k++) w = (w << 8) % p;  // (p below 2^24)
+    ws[b] = w;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        const int W = 1 << c, KS = W == 1 ? 1 : W / 2;
+        if (b >= 16 * KS) continue;
+        __half* wf = (__half*)im.to[c];
+        int32_t r = i < L && b < 8 * W ? (int32_t)w : 0;
+        if (r > (int32_t)(p >> 1)) r -= (int32_t)p;
+        const int limb = b >> 2, t = limb / KS, ks = limb % KS;
+        for (int dig = 0; dig < 3; dig++) {
+            const int c6 = (i >> 2 & 1) * 3 + dig, nt = (i >> 3) * 3 + c6 / 2;
+            const int ln = (2 * (i & 3) + (c6 & 1)) * 4 + t;
+            wf[((nt * KS + ks) * 32 + ln) * 4 + (b & 3)] = __int2half_rn(dig < 2 ? ((r + 128) & 255) - 128 : r);
+            r = (r + 128) >> 8;
         }
     }
+    if (i >= L || b >= 8) return;
+    const int c = b >> 1, ints = b & 1, n = (8 << c) - 1;
+    uint64_t sum = 0;  // 128 times the 2^(8b) of the bytes below the top one
+    for (int k = 0; k < n; k++) sum += 128ull * ws[k];
+    const uint32_t k = (uint32_t)((sum + (ints ? 0u : p >> 1)) % p);
+    const float ip = 1.0f / (float)p;
+    uint4* ti = (uint4*)(im.to[c] + rm_frag(L, c == 0 ? 1 : 1 << (c - 1)));
+    ti[ints * L + i] = make_uint4(p, rem_const(k, p), __float_as_uint(ip), __float_as_uint(quot_const(k, ip, p)));
 }
 
 template <int W, bool INT>
@@ -842,11 +850,11 @@ size_t reduce_image_bytes(const std::vector<uint32_t>& p, int W) {
     return rm_frag(L, W == 1 ? 1 : W / 2) + 2 * (size_t)L * sizeof(uint4);
 }
 
-void reduce_image_make(const uint32_t* p, int L, int W, uint8_t* image) {
-    if (W == 1) reduce_image<1>(p, L, image);
-    else if (W == 2) reduce_image<2>(p, L, image);
-    else if (W == 4) reduce_image<4>(p, L, image);
-    else reduce_image<8>(p, L, image);
+cudaError_t launch_reduce_images(const uint32_t* d_p, int L, uint8_t* const (&to)[4], cudaStream_t s) {
+    ReduceImages im;
+    for (int k = 0; k < 4; k++) im.to[k] = to[k];
+    reduce_images_kernel<<<(unsigned)((L + 7) / 8 * 8), kImageBytes, 0, s>>>(d_p, L, im);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_reduce(const BasisDev& b, const ReduceArgs& a_in, ReduceOut kind, int* d_status,

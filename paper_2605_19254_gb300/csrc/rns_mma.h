@@ -22,7 +22,6 @@
 
 #ifdef __CUDACC__
 #include <cuda_fp16.h>
-#include <string.h>
 
 namespace smf {
 namespace {
@@ -102,10 +101,10 @@ __device__ __forceinline__ void mma_tiles(float (&acc)[2][N][4], const uint32_t 
 // biases are 2^39.6, half a unit of f_c, at most 2^-7, and little of a quotient below
 // 2^14), so the result lies in [0, 1.07 q): min(y, y - q) ends it.
 constexpr uint32_t kMinPrime = 1u << 22;
-inline float quot_const(double c, float iq, uint32_t q) {
+__host__ __device__ inline float quot_const(double c, float iq, uint32_t q) {
     return (float)(c / q - 0.5 - 0x1p-5 - 12582912.0 * 65793.0 * (double)iq);
 }
-inline uint32_t rem_const(uint32_t c, uint32_t q) { return c - kMagicBits * 65793u + q * kMagicBits; }
+__host__ __device__ inline uint32_t rem_const(uint32_t c, uint32_t q) { return c - kMagicBits * 65793u + q * kMagicBits; }
 __device__ __forceinline__ float sums_quot(float s0, float s1, float s2, float iq, float f_c) {
     return fmaf(fmaf(s2, 65536.f, fmaf(s1, 256.f, s0)), iq, f_c);
 }
@@ -135,14 +134,6 @@ __device__ __forceinline__ void stage(void* to, const void* from, size_t n) {
         for (int k = 0; k < 8; k++)
             if (x0 + k * kMmaThreads < m) ((uint4*)to)[x0 + k * kMmaThreads] = v[k];
     }
-}
-
-// fp16 bits of an integer of at most 11 bits (host tables; __float2half takes 20 ns on the host)
-inline uint16_t half_bits(int v) {
-    if (v == 0) return 0;
-    const unsigned u = v < 0 ? 0u - (unsigned)v : (unsigned)v;
-    const int e = 31 - __builtin_clz(u);
-    return (uint16_t)((v < 0 ? 0x8000 : 0) | (15 + e) << 10 | ((u << (10 - e)) & 0x3FF));
 }
 
 // alpha where the estimate's fraction is too near an integer: within one of its

@@ -445,10 +445,13 @@ cudaError_t launch_gemm_limb_crt(smf_ctx* ctx, const BasisDev& b, const CrtHost&
 
 // The CRT's tables for the tensor cores (0 bytes: the basis is not for them), and
 // where the per-prime constants lie in them; the reductions' tables for W words.
+// Made in two parts: what the host fills in (from `pc` on), and the fragments before
+// it on the device, from the limbs of the M_i and the primes there.
 size_t crt_image_bytes(const CrtHost& h, size_t* pc);
 void crt_image_make(const CrtHost& h, uint8_t* image);
+cudaError_t launch_crt_image(const CrtHost& h, uint8_t* image, cudaStream_t s);
 size_t reduce_image_bytes(const std::vector<uint32_t>& p, int W);
-void reduce_image_make(const uint32_t* p, int L, int W, uint8_t* image);
+cudaError_t launch_reduce_images(const uint32_t* d_p, int L, uint8_t* const (&to)[4], cudaStream_t s);
 
 // CRT reconstruction: Lagrange form with an fp32 correction, exact mixed-radix (Garner) fallback.
 cudaError_t launch_crt(const CrtHost& h, const int32_t* R, int64_t rows, int64_t cols,
