@@ -434,7 +434,7 @@ def run(args):
     crt_bytes = L * Mr * N_ * 4 + Mr * N_ * C_WORDS * 8
     secondary = {
         name: {"ms": ms, "algorithmic_bytes": nbytes, "hbm_gbs": nbytes / (ms * 1e-3) / 1e9,
-               "hbm_frac": nbytes / (ms * 1e-3) / 1e9 / hbm if hbm else None, "bound": "integer issue"}
+               "hbm_frac": nbytes / (ms * 1e-3) / 1e9 / hbm if hbm else None, "bound": "latency at 16 to 24 warps per SM"}
         for name, ms, nbytes in (("reduce_phase", red_ms, red_bytes), ("crt", crt_ms, crt_bytes)) if ms > 0}
     out = {
         "metric": METRIC, "value": value, "unit": "TOPS", "n_gpus": ws, "steps": args.steps,
@@ -512,7 +512,7 @@ def run_base_convert(dev, local, stream, flush, steps, hbm_peak):
     out = {"workload": f"{count} entries (4096 x 256), {len(src.primes)} -> {len(dst.primes)} primes below 2^24",
            "ms": ms, "entries_per_s": count / (ms * 1e-3), "algorithmic_bytes": nbytes,
            "hbm_gbs": nbytes / (ms * 1e-3) / 1e9, "hbm_frac": nbytes / (ms * 1e-3) / 1e9 / hbm_peak if hbm_peak else None,
-           "bound": "integer issue", "kernel": "convert_mma_kernel<24>", "steps": steps}
+           "bound": "latency at 20 warps per SM", "kernel": "convert_mma_kernel<24>", "steps": steps}
     src.destroy()
     dst.destroy()
     ctx.destroy()

@@ -182,7 +182,7 @@ convert_kernel(const __grid_constant__ ConvConst<LMAX> v, const int32_t* __restr
 // memory, so that the words are stored in order.
 // 1300 thread instructions an entry with 23 primes (1815 as limb sums, one thread per
 // entry) at half the issue slots: 18.6M entries 1.51 -> 1.47 ms.  The product of 1009 x 1009 by
-// 1009 x 100 with 34 primes (reduction and CRT both so) went from 303 to 216 us, one
+// 1009 x 100 with 34 primes (reduction and CRT both so) went from 303 to 208 us, one
 // of 64 x 64 by 64 x 16 from 38 to 25 us.
 template <int LMAX>
 struct CrtMma {
@@ -455,7 +455,7 @@ cudaError_t launch_crt_mma_grouped(const CrtHost& h, const CrtItem* items, int n
 // hold two targets of a lane.  A residue is then
 //   v = S_0 + 2^8 S_1 + 2^16 S_2 + C_j - alpha (M mod q_j)  mod q_j:
 // sums_quot and sums_rem have the arithmetic.
-// 23 -> 23 primes, 1M entries: 159 -> 73 us (28 us of HBM traffic); half the issue
+// 23 -> 23 primes, 1M entries: 159 -> 68 us (28 us of HBM traffic); half the issue
 // slots are busy, the chunks' latencies bound it.
 template <int LMAX>
 struct ConvMma {

@@ -7,35 +7,36 @@
 //  - Phase 3 checks prod s_i = +-det A modulo primes q: det A mod q by
 //    Gaussian elimination over GF(q).
 //
-// Column k takes as pivot the first row not yet used whose entry in column k
-// is a unit (not divisible by q).  Every other unused row i subtracts
-// f_i = M[i][k] / M[p][k] times the pivot row (no row is moved, so the
-// determinant is the sign of the permutation k -> pivot row times the product
-// of the pivots).  A column without a unit is left for later ("deferred"):
-// in the local form, once every column has been seen, the unused rows and the
-// deferred columns hold a square block whose entries are all divisible by q;
-// it is divided by q and reduced again modulo q^(e-1).  Its size at each
-// level counts the invariant factors divisible by the next power of q.
+// Every column takes as pivot a row not yet used whose entry in it is a unit (not
+// divisible by q), and every other unused row i subtracts f_i = M[i][k] / M[p][k]
+// times the pivot row (no row is moved, so the determinant is the sign of the
+// permutation k -> pivot row times the product of the pivots).  A column without
+// a unit is left for later ("deferred"): in the local form, once every column has
+// been seen, the unused rows and the deferred columns hold a square block whose
+// entries are all divisible by q; it is divided by q and reduced again modulo
+// q^(e-1).  Its size at each level counts the invariant factors divisible by the
+// next power of q.
 //
-// Products modulo m use Shoup's method: for a multiplier f fixed across a row,
-// f' = floor(f 2^w / m) makes f y mod m = f y - floor(y f' / 2^w) m, at most
-// one m too large (w = 32 for m < 2^31, 64 for m < 2^62).
+// Moduli below 2^31 go by panels of columns at every size (from the threshold of
+// smf_set_elim_panels on), each panel reduced by one thread-block cluster: see
+// "Elimination by panels" below, and panel.h.
 //
-// Moduli below 2^31 go by panels of columns, each reduced by one thread-block
-// cluster (see "Elimination by panels" below).  Wider ones, and matrices below
-// the threshold of smf_set_elim_panels, go column by column: determinants and
-// lockstep local forms (two or more lanes) take one launch per
-// column: the launch for column k eliminates it and, in the threads that update column k+1, copies that column's new values
-// into a compact buffer and finds its first unused unit row (atomicMin).  The
-// last of those blocks to finish (a counter, no waiting) takes that row as
-// column k+1's pivot, marks it used and stores its inverse, so the next launch
-// finds everything it needs; each block then forms the multipliers of its own
-// rows from the compact column.  A local form in one lane keeps two launches
-// per column (a one-block pivot step that writes every row's multiplier, then
-// the update): there every column stays live and the per-block multipliers cost
-// more than the pivot step saves (measured at n = 5003: 0.185 s against 0.227 s
-// for one local form; four lockstep determinants 0.527 s against 0.418 s fused;
-// four lockstep local forms 0.645 s against 0.604 s fused).
+// Wider moduli, and matrices below the threshold, go column by column, with the
+// first unused unit row as the pivot.  Products modulo m use Shoup's method there:
+// for a multiplier f fixed across a row, f' = floor(f 2^w / m) makes f y mod m =
+// f y - floor(y f' / 2^w) m, at most one m too large (w = 32 for m < 2^31, 64 for
+// m < 2^62).  Determinants and lockstep local forms (two or more lanes) take one
+// launch per column: the launch for column k eliminates it and, in the threads that
+// update column k+1, copies that column's new values into a compact buffer and finds
+// its first unused unit row (atomicMin).  The last of those blocks to finish (a
+// counter, no waiting) takes that row as column k+1's pivot, marks it used and stores
+// its inverse, so the next launch finds everything it needs; each block then forms
+// the multipliers of its own rows from the compact column.  A local form in one lane
+// keeps two launches per column (a one-block pivot step that writes every row's
+// multiplier, then the update): there every column stays live and the per-block
+// multipliers cost more than the pivot step saves (measured at n = 5003: 0.185 s
+// against 0.227 s for one local form; four lockstep determinants 0.527 s against
+// 0.418 s fused; four lockstep local forms 0.645 s against 0.604 s fused).
 #include <algorithm>
 #include <vector>
 
@@ -525,8 +526,8 @@ cudaError_t elim_columns(smf_ctx* ctx, ElimBufs<T, L>& b, T* M, int64_t n, const
 //    columns are all of them, the panel's own too, followed by [c1, n).
 //
 // GB300, four 31-bit primes: n = 2003 6.6 ms (44 ms with a launch per column; 8.1 ms
-// without the look-ahead of elim_blocked: 59 panels of 41 to 104 us and as many
-// passes of up to 169 us, one after the other).
+// without the look-ahead of elim_blocked).  With it 63 panels of 36 to 97 us, 4.1 ms
+// in all, run beside passes of 11 to 157 us, 4.6 ms in all.  n = 5003 59 ms, 10007 0.46 s.
 constexpr int kPanel = 32;
 constexpr int64_t kLookAhead = 2 << 20;  // words of a pass (about 20 us)
 

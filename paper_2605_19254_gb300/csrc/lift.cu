@@ -63,7 +63,8 @@ __device__ __forceinline__ void put_digits(__nv_bfloat16* d, int64_t plane, int3
 // lift_step and 5.6 us for lift_x at n = 1024, m = 64.  Every division is by a number
 // fixed for the call, so all of them are products with constants (LiftBasis).  The
 // whole Smith form of a planted n = 1009 matrix went from 37.9 to 35.5 ms; the loop at
-// n = 1024, m = 64 from 34.6 to 33.9 us a step: the two products bound it.
+// n = 1024, m = 64 from 34.6 to 33.9 us a step (32.7 with the tiles of columns along
+// the grid's first dimension): the two products bound it.
 constexpr int kTileK = 32, kTileC = 8;
 
 // x mod q, rcp = floor(2^32 / q): the quotient is at most one low

@@ -233,9 +233,11 @@ reduce_kernel(BasisDev b, ReduceArgs a, int group) {
 // top one signed as it is) and balanced digits of the constants, fp32 sums below
 // 2^20, exact.  Lane 4g + t takes a quarter of the bytes of entries 4g .. 4g+3,
 // which follow one another along the output's contiguous dimension, so that its
-// results are stored 8 or 16 bytes at a time: the limb sums stored two bytes at a
-// time, 69 stores an entry with 23 primes.  The bound is instruction issue: about
-// 650 thread instructions per entry with 23 primes (2670 as limb sums).
+// results are stored 8 or 16 bytes at a time (the limb sums stored two bytes at a
+// time, 69 stores an entry with 23 primes).  512-bit entries and 23 primes take 700
+// thread instructions an entry as canonical residues, 1200 as transposed digits
+// (2016 as limb sums), at 49 and 61 % of the issue slots: the latency of the 32-entry
+// chunks at 24 warps per SM bounds it.
 struct RmArgs {
     const uint64_t* X;
     int64_t minor_n, major_n;  // entries along the output's contiguous dimension, and across it

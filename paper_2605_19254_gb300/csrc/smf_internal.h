@@ -28,7 +28,7 @@ struct BasisDev {
     const uint32_t* p;        // [L] primes, descending
     const uint64_t* mu;       // [L] floor((2^64 - 1) / p_i), Barrett reduction
     const uint32_t* pow32;    // [L] 2^32 mod p_i
-    const uint8_t* red[4];    // tables of the tensor-core reductions of entries of 1, 2, 4, 8 words (reduce_image)
+    const uint8_t* red[4];    // tables of the tensor-core reductions of entries of 1, 2, 4, 8 words (launch_reduce_images)
     uint32_t p_top, p_low;    // the largest and the smallest prime
     int sms;                  // SMs of the device the tables are on
     const double* inv_p;      // [L] 1/p_i rounded to fp64 (Section 3.1 fast reduction)
@@ -87,7 +87,7 @@ struct smf_prof_rec {
 
 // default threshold of the eliminations by panels (smf_set_elim_panels): every
 // size.  Four 31-bit determinants, by panels / one launch per column: n = 16
-// 0.10 / 0.30 ms, 128 0.32 / 1.7, 1009 2.7 / 14.4, 2003 8.1 / 44; three local
+// 0.10 / 0.30 ms, 128 0.32 / 1.7, 1009 2.6 / 14.4, 2003 6.6 / 44; three local
 // forms of a planted matrix: n = 32 0.13 / 1.2 ms, 1009 2.5 / 12.9.
 constexpr int64_t kElimPanelMinN = 1;
 
